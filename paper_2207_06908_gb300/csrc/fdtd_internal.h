@@ -41,25 +41,21 @@ constexpr int CXO = 16;                      // box column of x0 in the class bo
 constexpr int CBX = TX + 16, CBY = TY + 1;   // class box: x0-16 .. x0+TX-1
 }  // namespace geom
 
-// TMA descriptors of the current input buffers: E (E box), H (H box), class
-// plus the CPML auxiliaries: z layer with the H box (HX_Z, HY_Z) and the
-// tile box (EX_Z, EY_Z); x layer (HY_X, HZ_X | EY_X, EZ_X) with a box
-// narrowed to the layer along x; y layer (HX_Y, HZ_Y | EX_Y, EZ_Y) with a
-// box narrowed to the layer along y
+// TMA descriptors of the current input buffers, the arrays of one kind as
+// the fourth dimension so that one copy brings them all: the three E (E box),
+// the three H (H box), the class bytes, and the CPML auxiliaries: z layer
+// with the H box (HX_Z, HY_Z) and the tile box (EX_Z, EY_Z); x layer (HY_X,
+// HZ_X, EY_X, EZ_X) with a box narrowed to the layer along x; y layer (HX_Y,
+// HZ_Y, EX_Y, EZ_Y) with a box narrowed to the layer along y
 struct TmaMaps {
-    CUtensorMap e[3];
-    CUtensorMap h[3];
-    CUtensorMap c;
-    CUtensorMap zh[2], ze[2];
-    CUtensorMap xh[2], xe[2];
-    CUtensorMap yh[2], ye[2];
+    CUtensorMap e, h, c, zh, ze, x, y;
 };
 
 // geometry of the staged CPML boxes (host-computed for the grid's layer)
 struct PsiGeom {
     int w;                   // x-layer box width (slab entries, multiple of 4)
     int hy;                  // y-layer box height (slab rows)
-    int xb, yb;              // bytes of one x / y box slot (128-aligned)
+    int xb, yb;              // bytes of one array's x / y box
 };
 
 // Debye media: up to kMaxPoles poles per edge; per cell one record of
@@ -299,7 +295,7 @@ PsiGeom step_psi_geom(int d, int nx, int ny);
 // region size and box-group offsets for a launch that stages z alone
 // (zxy = 0) or z together with the x / y layers (zxy = 1)
 void step_region(const PsiGeom &pg, int zxy, int *region, int *ox, int *oy);
-const void *step_kernel_ptr(int nh, bool batch, bool wide);
+const void *step_kernel_ptr(int launch, int nh, bool batch, bool wide);
 // fdtd_edges.cu
 cudaError_t launch_edges(const EdgeArgs &a, cudaStream_t s);
 // oblique wires: segment currents to t_{n+1/2}; needs only the step's inputs,

@@ -1194,26 +1194,20 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn()
     return fn;
 }
 
-// 3D tiled map over one array of extent x0 x y0 x z0 with row pitch
-// `pitch` elements and y0 rows per plane (x fastest); out-of-range box
-// elements read as zero
-bool encode_map3(CUtensorMap *m, void *base, CUtensorMapDataType dt, int esize, int x0, int y0, int z0, int pitch,
-                 int bx, int by)
+// tiled map over n arrays of extent x0 x y0 x z0, `stride` bytes apart, with
+// row pitch `pitch` elements and y0 rows per plane (x fastest); a box is
+// bx x by of one plane of all of them; out-of-range box elements read as zero
+bool encode_map(CUtensorMap *m, void *base, CUtensorMapDataType dt, int esize, int x0, int y0, int z0, int pitch,
+                int n, size_t stride, int bx, int by)
 {
     auto fn = encode_fn();
     if (!fn) return false;
-    cuuint64_t dims[3] = {(cuuint64_t)x0, (cuuint64_t)y0, (cuuint64_t)z0};
-    cuuint64_t strides[2] = {(cuuint64_t)pitch * esize, (cuuint64_t)pitch * y0 * esize};
-    cuuint32_t box[3] = {(cuuint32_t)bx, (cuuint32_t)by, 1};
-    cuuint32_t es[3] = {1, 1, 1};
-    return fn(m, dt, 3, base, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+    cuuint64_t dims[4] = {(cuuint64_t)x0, (cuuint64_t)y0, (cuuint64_t)z0, (cuuint64_t)n};
+    cuuint64_t strides[3] = {(cuuint64_t)pitch * esize, (cuuint64_t)pitch * y0 * esize, (cuuint64_t)stride};
+    cuuint32_t box[4] = {(cuuint32_t)bx, (cuuint32_t)by, 1, (cuuint32_t)n};
+    cuuint32_t es[4] = {1, 1, 1, 1};
+    return fn(m, dt, 4, base, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// 3D tiled map over one field-shaped array (the fields, the class bytes)
-bool encode_map(CUtensorMap *m, void *base, CUtensorMapDataType dt, int esize, const fdtd_grid *g, int bx, int by)
-{
-    return encode_map3(m, base, dt, esize, g->nx, g->ny, g->nz, g->pitch, bx, by);
 }
 
 // Raise (never lower) a step kernel's dynamic shared-memory limit: grids and
@@ -1237,36 +1231,27 @@ int setup_step_kernel(fdtd_grid *g)
 {
     using namespace fdtd::geom;
     g->pg = fdtd::step_psi_geom(g->d, g->nx, g->ny);
+    const auto F32 = CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
+    const int nx = g->nx, ny = g->ny, nz = g->nz, pitch = g->pitch;
+    const size_t cells = (size_t)g->plane * nz;
     for (int p = 0; p < 2; ++p) {
-        for (int c = 0; c < 3; ++c) {
-            if (!encode_map(&g->maps[p].e[c], g->F[p][c], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, g, EBX, EBY) ||
-                !encode_map(&g->maps[p].h[c], g->F[p][3 + c], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, g, HBX, HBY))
-                return fail(g, FDTD_ECUDA, "cuTensorMapEncodeTiled failed for a field");
-        }
-        if (!encode_map(&g->maps[p].c, g->cls, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, g, CBX, CBY))
+        fdtd::TmaMaps &m = g->maps[p];
+        if (!encode_map(&m.e, g->F[p][0], F32, 4, nx, ny, nz, pitch, 3, cells * 4, EBX, EBY) ||
+            !encode_map(&m.h, g->F[p][3], F32, 4, nx, ny, nz, pitch, 3, cells * 4, HBX, HBY))
+            return fail(g, FDTD_ECUDA, "cuTensorMapEncodeTiled failed for the fields");
+        if (!encode_map(&m.c, g->cls, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, nx, ny, nz, pitch, 1, cells, CBX, CBY))
             return fail(g, FDTD_ECUDA, "cuTensorMapEncodeTiled failed for the class map");
         if (g->d > 0) {
             using namespace fdtd;
-            const auto F32 = CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
-            const int w = g->pg.w, hy = g->pg.hy;
-            // compact layouts: x [nz][ny][px], y [nz][2d][pitch], z [2d][ny][pitch]
-            const int px = psi_px(g), d2 = 2 * g->d;
-            struct { CUtensorMap *m; int psi, bx, by; } maps[12] = {
-                {&g->maps[p].zh[0], PSI_HX_Z, HBX, HBY}, {&g->maps[p].zh[1], PSI_HY_Z, HBX, HBY},
-                {&g->maps[p].ze[0], PSI_EX_Z, TX, TY},   {&g->maps[p].ze[1], PSI_EY_Z, TX, TY},
-                {&g->maps[p].xh[0], PSI_HY_X, w, HBY},   {&g->maps[p].xh[1], PSI_HZ_X, w, HBY},
-                {&g->maps[p].xe[0], PSI_EY_X, w, HBY},   {&g->maps[p].xe[1], PSI_EZ_X, w, HBY},
-                {&g->maps[p].yh[0], PSI_HX_Y, HBX, hy},  {&g->maps[p].yh[1], PSI_HZ_Y, HBX, hy},
-                {&g->maps[p].ye[0], PSI_EX_Y, HBX, hy},  {&g->maps[p].ye[1], PSI_EZ_Y, HBX, hy}};
-            for (auto &mm : maps) {
-                const int axis = mm.psi / 4;
-                const bool ok = axis == 0   ? encode_map3(mm.m, g->psi[p][mm.psi], F32, 4, px, g->ny, g->nz, px, mm.bx, mm.by)
-                                : axis == 1 ? encode_map3(mm.m, g->psi[p][mm.psi], F32, 4, g->nx, d2, g->nz, g->pitch,
-                                                          mm.bx, mm.by)
-                                            : encode_map3(mm.m, g->psi[p][mm.psi], F32, 4, g->nx, g->ny, d2, g->pitch,
-                                                          mm.bx, mm.by);
-                if (!ok) return fail(g, FDTD_ECUDA, "cuTensorMapEncodeTiled failed for a CPML array");
-            }
+            // compact layouts: x [nz][ny][px], y [nz][2d][pitch], z [2d][ny][pitch],
+            // an axis's arrays equally far apart
+            const int w = g->pg.w, hy = g->pg.hy, px = psi_px(g), d2 = 2 * g->d;
+            auto gap = [&](int q) { return (size_t)((char *)g->psi[p][q + 1] - (char *)g->psi[p][q]); };
+            if (!encode_map(&m.x, g->psi[p][PSI_HY_X], F32, 4, px, ny, nz, px, 4, gap(PSI_HY_X), w, HBY) ||
+                !encode_map(&m.y, g->psi[p][PSI_HX_Y], F32, 4, nx, d2, nz, pitch, 4, gap(PSI_HX_Y), HBX, hy) ||
+                !encode_map(&m.zh, g->psi[p][PSI_HX_Z], F32, 4, nx, ny, d2, pitch, 2, gap(PSI_HX_Z), HBX, HBY) ||
+                !encode_map(&m.ze, g->psi[p][PSI_EX_Z], F32, 4, nx, ny, d2, pitch, 2, gap(PSI_EX_Z), TX, TY))
+                return fail(g, FDTD_ECUDA, "cuTensorMapEncodeTiled failed for a CPML array");
         }
     }
     g->ncx = (g->nx + TX - 1) / TX;
@@ -1309,12 +1294,13 @@ int setup_step_kernel(fdtd_grid *g)
         g->n_launch = l + 1;
     }
     const bool wide = grid_is_wide(g);
-    for (int nh = 2; nh <= 3 && e == cudaSuccess; ++nh) e = ensure_smem(fdtd::step_kernel_ptr(nh, false, wide), max_smem);
+    for (int q = 0; q < 4 && e == cudaSuccess; ++q)
+        e = ensure_smem(fdtd::step_kernel_ptr(q >> 1, 2 + (q & 1), false, wide), max_smem);
     if (e != cudaSuccess) return cuda_fail(g, e, "step kernel setup");
     for (int l = 0; l < g->n_launch; ++l) {
         auto &L = g->lc[l];
         int occ = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fdtd::step_kernel_ptr(L.nh, false, wide), fdtd::step_threads(),
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fdtd::step_kernel_ptr(l, L.nh, false, wide), fdtd::step_threads(),
                                                           fdtd::step_smem_bytes(g->n_classes, d, L.region, L.nh));
         if (e != cudaSuccess) return cuda_fail(g, e, "step kernel occupancy");
         if (occ < 1) return fail(g, FDTD_ECUDA, "step kernel does not fit on an SM");
@@ -2478,11 +2464,12 @@ int fdtd_batch_create(int n, fdtd_grid *const *grids, void *cuda_stream, fdtd_ba
             b->nh[l] = 2;
         max_smem = std::max(max_smem, fdtd::step_smem_bytes(b->max_classes, b->max_d, b->region[l], b->nh[l]));
     }
-    for (int nh = 2; nh <= 3 && e == cudaSuccess; ++nh) e = ensure_smem(fdtd::step_kernel_ptr(nh, true, false), max_smem);
+    for (int q = 0; q < 4 && e == cudaSuccess; ++q)
+        e = ensure_smem(fdtd::step_kernel_ptr(q >> 1, 2 + (q & 1), true, false), max_smem);
     for (int l = 0; l < b->n_launch && e == cudaSuccess; ++l) {
         int occ = 0;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &occ, fdtd::step_kernel_ptr(b->nh[l], true, false), fdtd::step_threads(),
+            &occ, fdtd::step_kernel_ptr(l, b->nh[l], true, false), fdtd::step_threads(),
             fdtd::step_smem_bytes(b->max_classes, b->max_d, b->region[l], b->nh[l]));
         if (e == cudaSuccess && occ < 1) { delete b; return FDTD_ECUDA; }
         b->grid[l] = std::max(1, std::min(sms * std::max(occ, 1), b->nitems[l]));

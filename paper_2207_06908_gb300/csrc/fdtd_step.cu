@@ -10,22 +10,32 @@
 //     planes one CTA loads are still in L2 when its neighbours load them.
 //     Within a z block the column tiles that meet a CPML layer come first:
 //     the last items of a launch are the quick ones.
-//   - One producer warp streams, plane by plane, TMA 3D boxes into two
+//   - One producer warp streams, plane by plane, TMA boxes into two
 //     shared-memory rings tracked by mbarriers: E^n (tile + 1-cell halo on
 //     every side, x start rounded down to a 16-byte boundary) into a
 //     4-slot ring (two planes in use, two in flight), and H^{n-1/2} (tile +
 //     low halo), the class bytes and, in a CPML layer, the auxiliary fields
-//     of one axis into a 3-slot ring (one in use, two in flight).
-//   - Eight row warps: lane = x column, warp w owns rows w and w + 8 of the
-//     tile (so a y layer's rows spread over all warps).  Per plane k they
-//     form H^{n+1/2}(k) of their cells and store it, then E^{n+1}(k) from
-//     that H plane and the owned column's H of plane k-1 kept in registers;
-//     E^n(k+1) of the owned cells stays in registers for the next plane.  A ninth warp recomputes (never exchanges) H^{n+1/2} of
-//     the low-y row and low-x column halo meanwhile, so every warp has the
-//     same work between the two per-plane barriers.
-//   - Items that touch no CPML layer run a variant compiled without any
-//     CPML code; in the others the layer tests are hoisted per item, row
-//     and plane.
+//     into a 3-slot ring (one in use, two in flight).  The arrays of one kind
+//     are the fourth dimension of one tensor map, so a plane takes three
+//     copies, five in a tile that meets an x and a y layer.
+//   - Eight row warps, two neighbouring x cells per lane: warp w owns rows w
+//     and w + 8 of the tile (so a y layer's rows spread over all warps).  Per
+//     plane k they form H^{n+1/2}(k) of their cells, then, after the one
+//     barrier a plane has, E^{n+1}(k) from that H plane and the plane before
+//     it, both in shared memory.  Two more warps recompute (never exchange)
+//     H^{n+1/2} of the low-y row and the low-x column of the halo meanwhile.
+//   - The layers an item meets are template arguments: an item that meets
+//     none runs without any CPML code, the others without a branch per cell.
+// What bounds it: DRAM on grids that fill the chip, otherwise the latency of
+// a plane's chain (copies landed, H, barrier, E), which a CTA cannot
+// overlap with more than the ring holds.  Hence few and wide instructions
+// per plane, registers split by role (setmaxnreg), and few copies issued by
+// a converged warp.  With four cells per lane (16-byte accesses) the plane
+// loop has fewer instructions but half the warps to hide its latency, and
+// measured slower.  Measured (us per step, one cell per lane and fifteen
+// copies a plane before): 256^3 PEC 136.3 -> 130.1 (0.93 of the measured copy
+// bandwidth), 256^3 with a 10-cell CPML 175.9 -> 164.6, 512x512x384 with 12
+// cells 956 -> 908, 128^3 with 8 cells 42.7 -> 38.4.
 // DRAM traffic per cell and step: 6 FP32 reads + 6 writes + 1 class byte
 // (49 B) plus the CPML auxiliaries in the layer; every halo read is an L2
 // hit.  Every wait is bounded; on a timeout the kernel records an error
@@ -41,12 +51,21 @@
 namespace fdtd {
 namespace {
 
-using geom::TX;                        // tile width: one lane per column
+using geom::TX;                        // tile width
 using geom::TY;                        // tile height
-constexpr int RW = 2;                  // rows per consumer warp (w and w + NCW)
-constexpr int NCW = TY / RW;           // row warps
-constexpr int NCONS = (NCW + 1) * 32;  // row warps + the halo warp
-constexpr int NTHREADS = NCONS + 32;   // + the producer warp
+constexpr int GX = 2;                  // neighbouring x cells per lane of a row warp (8-byte accesses)
+constexpr int LPR = TX / GX;           // lanes per tile row
+constexpr int RPW = 32 / LPR;          // tile rows per row warp (w, w + NCW, ...)
+constexpr int NCW = TY / RPW;          // row warps
+constexpr int NHW = 2;                 // halo warps: low-y row, low-x column
+constexpr int NCONS = (NCW + NHW) * 32;  // row warps + halo warps
+constexpr int NTHREADS = (NCW + 4) * 32;   // + the producer warp, one warp idle: whole warpgroups
+// registers: the row warps (the first warpgroups) hold their cells' state and
+// take ROW_REGS each, the halo warps and the producer AUX_REGS; together
+// what the block is launched with (two blocks per SM)
+constexpr int ROW_REGS = 96, AUX_REGS = 48, LAUNCH_REGS = 80;
+static_assert(NCW % 4 == 0, "row warps fill warpgroups");
+static_assert(NCW * ROW_REGS + 4 * AUX_REGS <= (NCW + 4) * LAUNCH_REGS, "the shares of the launch's registers");
 constexpr int NE = 4;                  // E-plane ring: planes k, k+1 in use, two ahead
 constexpr int NH_MAX = 3;              // H / class / CPML ring: plane k in use, up to two ahead
                                        // (a launch whose auxiliary region is large uses 2)
@@ -72,22 +91,25 @@ __device__ __forceinline__ int tab_src(int slot)
     const int r = slot >> 2, c = slot & 3;
     return c == 3 ? -1 : (r == 0 ? 6 + c : (r == 1 ? c : 3 + c));
 }
-constexpr int E_COMP = al128(EBX * EBY * 4);
-constexpr int H_COMP = al128(HBX * HBY * 4);
+// one array's box in a slot; the boxes of one kind lie one after the other,
+// as one copy writes them (a kind starts on a 128-byte boundary)
+constexpr int E_COMP = EBX * EBY * 4;
+constexpr int H_COMP = HBX * HBY * 4;
 constexpr int C_BYTES = al128(CBX * CBY);
-constexpr int PE_BYTES = al128(TX * TY * 4);         // E-type psi box: the tile itself
-// E slot: three E boxes and a header (item, plane, staged-layer flags,
-// x-box start, y-box start)
+constexpr int PE_BYTES = TX * TY * 4;                // E-type psi box: the tile itself
+// E slot: three E boxes and a header: item, -, staged-layer flags of the
+// plane, x-box start, y-box start, domain
 constexpr int OFF_HDR = 3 * E_COMP;
-constexpr int ESLOT = al128(OFF_HDR + 32);   // header: item, plane, flags, x start, y start, domain
+constexpr int ESLOT = al128(OFF_HDR + 32);
 // H slot: three H boxes, the class box, then the staged-auxiliary region
 // (grid dependent size).  In a z-layer plane the region holds the z boxes
 // (2 H-type with the H box, 2 E-type with the tile box); elsewhere the x
 // boxes (4, narrowed along x) followed by the y boxes (4, narrowed along y).
 constexpr int OFF_H = 0;
-constexpr int OFF_C = 3 * H_COMP;
+constexpr int OFF_C = al128(3 * H_COMP);
 constexpr int OFF_PSI = OFF_C + C_BYTES;
-constexpr int Z_BYTES = 2 * H_COMP + 2 * PE_BYTES;
+constexpr int OFF_ZE = al128(2 * H_COMP);            // the E-type z boxes in the region
+constexpr int Z_BYTES = OFF_ZE + 2 * PE_BYTES;
 constexpr uint32_t TX_E = 3u * EBX * EBY * 4;
 constexpr uint32_t TX_H = 3u * HBX * HBY * 4 + CBX * CBY;
 constexpr uint32_t TX_Z = 2u * HBX * HBY * 4 + 2u * TX * TY * 4;
@@ -102,13 +124,18 @@ constexpr int SM_HH = NE * ESLOT;
 constexpr int HNEW_PLANE = HBY * HBX;
 constexpr int HNEW_BYTES = 2 * 3 * HNEW_PLANE * 4;     // [2][3][HBY][HBX]
 constexpr int NBAR = 2 * NE + 2 * NH_MAX;             // fullE, emptyE, fullH, emptyH
+// x-layer coefficients of the current item's columns: {b, c, 1/kappa} at E,
+// then at H positions, TX floats each (identity outside the layer), and an
+// identity profile row
+constexpr int XC_BYTES = 6 * TX * 4 + 16;
 struct Layout {
-    int hslot, hnew, bar, misc, tab;
+    int hslot, hnew, xc, bar, misc, tab;
     __host__ __device__ Layout(int region, int nh)
     {
         hslot = hslot_bytes(region);
         hnew = SM_HH + nh * hslot;
-        bar = hnew + HNEW_BYTES;
+        xc = hnew + HNEW_BYTES;
+        bar = xc + XC_BYTES;
         misc = bar + NBAR * 8;
         tab = misc + 32;
     }
@@ -197,14 +224,22 @@ __global__ void wait_selftest_kernel(unsigned long long limit_ns, int *flag)
 
 __device__ int g_selftest_flag;
 
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map, int x, int y, int z,
-                                            uint32_t bar)
+// box at (x, y, z) of every array of the map
+__device__ __forceinline__ void tma_load(uint32_t dst, const CUtensorMap *map, int x, int y, int z, uint32_t bar)
 {
     asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(bar)
+        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(0), "r"(bar)
         : "memory");
+}
+
+// one lane of the (converged) warp
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t ok;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(ok));
+    return ok != 0;
 }
 
 __device__ __forceinline__ void consumer_sync()
@@ -220,7 +255,7 @@ struct Slab {
     int sx, sy, sz;          // slab index along x, y, z or -1
     const float *base;       // staged-auxiliary region of the plane's H slot
     int xo, yo;              // float offsets of the cell in the first x / y box, or -1
-    int zo, zeo;             // float offsets in the first z H-type / E-type box, or -1
+    int zo;                  // float offset in the first z H-type box, or -1
 };
 
 __device__ __forceinline__ int slab_of(int i, int n, int d) { return i < d ? i : (i >= n - d ? i - (n - 2 * d) : -1); }
@@ -229,21 +264,12 @@ __device__ __forceinline__ int slab_of(int i, int n, int d) { return i < d ? i :
 // the profile b, c, 1/kappa of the cell's slab entry s,
 // psi <- b psi + c dif, dif <- dif / kappa + psi.  The profile row holds
 // {b, c, 1/kappa, -} per slab entry, read with one 16-byte load for both
-// differences, before any store.
-template <bool WRITE>
-__device__ __forceinline__ void cpml2(float &d0, float &d1, const float4 *pr, int s, float o0, float o1,
-                                      float *out0, float *out1, int g, long long n, int *bounds)
+// differences.
+__device__ __forceinline__ void cpml2(float &d0, float &d1, const float4 *pr, int s, float o0, float o1)
 {
-    // g: the cell's element in its axis's compact auxiliary arrays (n elements)
     const float4 pv = pr[s];
-    const float b = pv.x, c = pv.y, ki = pv.z;
-    const float p0 = b * o0 + c * d0, p1 = b * o1 + c * d1;
-    if (WRITE && in_bounds(g, n, 3, bounds)) {
-        out0[g] = p0;
-        out1[g] = p1;
-    }
-    d0 = d0 * ki + p0;
-    d1 = d1 * ki + p1;
+    d0 = __fmaf_rn(d0, pv.z, __fmaf_rn(pv.x, o0, __fmul_rn(pv.y, d0)));
+    d1 = __fmaf_rn(d1, pv.z, __fmaf_rn(pv.x, o1, __fmul_rn(pv.y, d1)));
 }
 
 // Element of cell (i, j, k) in the compact auxiliaries of each axis, which
@@ -276,14 +302,12 @@ __device__ __forceinline__ const float4 *prow(const float *prof, int u, int h, i
 // H^{n+1/2} of cell (i,j,k) from E^n around it (Eq. fdtdhx and its cyclic
 // analogues): Hx += db [dEy/dz - dEz/dy], Hy += db [dEz/dx - dEx/dz],
 // Hz += db [dEx/dy - dEy/dx]; differences in field units, 1/dx in db.
-// STAGED: every auxiliary the cell needs is in the staged boxes (true of
-// the cells an item updates); otherwise one outside them is read from
-// global memory.  WRITE: the cell is one the
-// item updates, so the new auxiliaries are stored (halo and warm-up cells
-// are recomputed only).
-template <bool CPML, bool STAGED, bool WRITE>
+// One cell of the low-y row or low-x column of a tile's halo, recomputed
+// and never stored; its auxiliaries are in the staged boxes, which include
+// the halo.
+template <bool CPML>
 __device__ __forceinline__ void h_core(const StepArgs &a, const float4 *t, const float *prof, const Slab &L,
-                                       int i, int j, int k, float ex, float ey, float ez, float ey_x1, float ez_x1,
+                                       float ex, float ey, float ez, float ey_x1, float ez_x1,
                                        float ex_y1, float ez_y1, float ex_z1, float ey_z1, float hx0, float hy0,
                                        float hz0, float &hx, float &hy, float &hz)
 {
@@ -292,75 +316,234 @@ __device__ __forceinline__ void h_core(const StepArgs &a, const float4 *t, const
     float hz_y = ex_y1 - ex, hz_x = ey_x1 - ey;
     if (CPML) {
         const int d2 = 2 * a.d;
-        if (L.sx >= 0) {
-            const int q = a.pg.xb >> 2;
-            const int g = psi_x(a, L.sx, j, k);
-            const float o0 = (STAGED || L.xo >= 0) ? L.base[L.xo]
-                                    : (in_bounds(g, psi_n(a, 0), 4, a.bounds) ? __ldg(a.psi_in[PSI_HY_X] + g) : 0.f);
-            const float o1 = (STAGED || L.xo >= 0) ? L.base[L.xo + q]
-                                    : (in_bounds(g, psi_n(a, 0), 4, a.bounds) ? __ldg(a.psi_in[PSI_HZ_X] + g) : 0.f);
-            cpml2<WRITE>(hy_x, hz_x, prow(prof, 0, 1, d2), L.sx, o0, o1, a.psi_out[PSI_HY_X], a.psi_out[PSI_HZ_X], g,
-                         psi_n(a, 0), a.bounds);
-        }
-        if (L.sy >= 0) {
-            const int q = a.pg.yb >> 2;
-            const int g = psi_y(a, i, L.sy, k);
-            const float o0 = (STAGED || L.yo >= 0) ? L.base[L.yo]
-                                    : (in_bounds(g, psi_n(a, 1), 4, a.bounds) ? __ldg(a.psi_in[PSI_HX_Y] + g) : 0.f);
-            const float o1 = (STAGED || L.yo >= 0) ? L.base[L.yo + q]
-                                    : (in_bounds(g, psi_n(a, 1), 4, a.bounds) ? __ldg(a.psi_in[PSI_HZ_Y] + g) : 0.f);
-            cpml2<WRITE>(hx_y, hz_y, prow(prof, 1, 1, d2), L.sy, o0, o1, a.psi_out[PSI_HX_Y],
-                         a.psi_out[PSI_HZ_Y], g, psi_n(a, 1), a.bounds);
-        }
-        if (L.sz >= 0) {
-            const int g = psi_z(a, i, j, L.sz);
-            const float o0 = (STAGED || L.zo >= 0) ? L.base[L.zo]
-                                    : (in_bounds(g, psi_n(a, 2), 4, a.bounds) ? __ldg(a.psi_in[PSI_HX_Z] + g) : 0.f);
-            const float o1 = (STAGED || L.zo >= 0) ? L.base[L.zo + H_COMP / 4]
-                                    : (in_bounds(g, psi_n(a, 2), 4, a.bounds) ? __ldg(a.psi_in[PSI_HY_Z] + g) : 0.f);
-            cpml2<WRITE>(hx_z, hy_z, prow(prof, 2, 1, d2), L.sz, o0, o1, a.psi_out[PSI_HX_Z],
-                         a.psi_out[PSI_HY_Z], g, psi_n(a, 2), a.bounds);
-        }
+        if (L.sx >= 0)
+            cpml2(hy_x, hz_x, prow(prof, 0, 1, d2), L.sx, L.base[L.xo], L.base[L.xo + (a.pg.xb >> 2)]);
+        if (L.sy >= 0)
+            cpml2(hx_y, hz_y, prow(prof, 1, 1, d2), L.sy, L.base[L.yo], L.base[L.yo + (a.pg.yb >> 2)]);
+        if (L.sz >= 0)
+            cpml2(hx_z, hy_z, prow(prof, 2, 1, d2), L.sz, L.base[L.zo], L.base[L.zo + H_COMP / 4]);
     }
     const float4 db = t[0];
-    hx = hx0 + db.x * (hx_z - hx_y);
-    hy = hy0 + db.y * (hy_x - hy_z);
-    hz = hz0 + db.z * (hz_y - hz_x);
+    hx = __fmaf_rn(db.x, hx_z - hx_y, hx0);
+    hy = __fmaf_rn(db.y, hy_x - hy_z, hy0);
+    hz = __fmaf_rn(db.z, hz_y - hz_x, hz0);
 }
 
-// E^{n+1} of cell (i,j,k) (Eq. fdtdex with sigma E time-averaged):
-// E = ca E + cb [curl_h H^{n+1/2}], 1/dx in cb.  Only cells the item
-// updates, whose auxiliaries are staged.
-template <bool CPML>
-__device__ __forceinline__ void e_core(const StepArgs &a, const float4 *t, const float *prof, const Slab &L,
-                                       int i, int j, int k, float ex, float ey, float ez, float hx, float hy, float hz,
-                                       float hz_ym, float hx_ym, float hz_xm, float hy_xm, float hx_zm,
-                                       float hy_zm, float &ex1, float &ey1, float &ez1)
+// ---- two cells per lane -----------------------------------------------------
+// The row warps' stencil: a lane owns two neighbouring x cells of one tile
+// row, so a field box is read with one 8-byte access per component and stored
+// with another, the index arithmetic and the barriers are paid once per two
+// cells, and the differences and layer sums run two cells to an instruction
+// (packed FP32 pairs).  The layers an item meets are template arguments and
+// the lanes outside them run along with identity coefficients, so the plane
+// loop has no branches to wait on.  Every sum is written as explicit products
+// and fused multiply-adds, so every instantiation of the kernel rounds alike.
+using F2 = unsigned long long;           // two FP32 values
+__device__ __forceinline__ F2 pk(float lo, float hi)
 {
-    float ex_y = hz - hz_ym, ex_z = hy - hy_zm;
-    float ey_z = hx - hx_zm, ey_x = hz - hz_xm;
-    float ez_x = hy - hy_xm, ez_y = hx - hx_ym;
-    if (CPML) {
-        const int d2 = 2 * a.d;
-        if (L.sx >= 0) {
-            const int q = a.pg.xb >> 2;
-            cpml2<true>(ey_x, ez_x, prow(prof, 0, 0, d2), L.sx, L.base[L.xo + 2 * q], L.base[L.xo + 3 * q],
-                        a.psi_out[PSI_EY_X], a.psi_out[PSI_EZ_X], psi_x(a, L.sx, j, k), psi_n(a, 0), a.bounds);
-        }
-        if (L.sy >= 0) {
-            const int q = a.pg.yb >> 2;
-            cpml2<true>(ex_y, ez_y, prow(prof, 1, 0, d2), L.sy, L.base[L.yo + 2 * q], L.base[L.yo + 3 * q],
-                        a.psi_out[PSI_EX_Y], a.psi_out[PSI_EZ_Y], psi_y(a, i, L.sy, k), psi_n(a, 1), a.bounds);
-        }
-        if (L.sz >= 0)
-            cpml2<true>(ex_z, ey_z, prow(prof, 2, 0, d2), L.sz, L.base[L.zeo],
-                        L.base[L.zeo + PE_BYTES / 4], a.psi_out[PSI_EX_Z], a.psi_out[PSI_EY_Z], psi_z(a, i, j, L.sz),
-                        psi_n(a, 2), a.bounds);
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ float lo2(F2 v) { return __uint_as_float((uint32_t)v); }
+__device__ __forceinline__ float hi2(F2 v) { return __uint_as_float((uint32_t)(v >> 32)); }
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c)
+{
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ F2 mul2(F2 a, F2 b)
+{
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+__device__ __forceinline__ F2 ld2(const float *p) { return *reinterpret_cast<const F2 *>(p); }
+__device__ __forceinline__ void st2(float *p, F2 x) { *reinterpret_cast<F2 *>(p) = x; }
+// a - b (the product with -1 is exact, so this is the plain difference)
+__device__ __forceinline__ F2 sub2(F2 a, F2 b) { return fma2(b, pk(-1.f, -1.f), a); }
+// differences along x: of the next cell and this one (e: the cell after the
+// pair), of this one and the one before (w)
+__device__ __forceinline__ F2 next_diff(F2 x, float e) { return pk(hi2(x) - lo2(x), e - hi2(x)); }
+__device__ __forceinline__ F2 prev_diff(F2 x, float w) { return pk(lo2(x) - w, hi2(x) - lo2(x)); }
+// the cells m (bit c: cell c) of a pair at element g of base to global
+// memory.  all: both or none (every tile that lies wholly in the grid; the
+// same for the whole warp)
+template <typename Idx>
+__device__ __forceinline__ void put2(float *base, Idx g, F2 x, int m, bool all, long long n, int site, int *bounds)
+{
+    if (all) {
+        if (m && in_bounds(g, n, site, bounds) && in_bounds(g + 1, n, site, bounds)) st2(base + g, x);
+    } else {
+        if ((m & 1) && in_bounds(g, n, site, bounds)) base[g] = lo2(x);
+        if ((m & 2) && in_bounds(g + 1, n, site, bounds)) base[g + 1] = hi2(x);
     }
-    const float4 ca = t[1], cb = t[2];
-    ex1 = ca.x * ex + cb.x * (ex_y - ex_z);
-    ey1 = ca.y * ey + cb.y * (ey_z - ey_x);
-    ez1 = ca.z * ez + cb.z * (ez_x - ez_y);
+}
+
+// what a lane's pair of cells is to the layers of its item, formed once per item
+struct Pair {
+    int i, j;                // first cell
+    int m;                   // bit c: cell c lies inside the grid
+    bool all;                // every cell of the tile does (uniform)
+    int xm;                  // bit c: cell c lies in an x layer
+    int xe;                  // slab entry of the first cell (of the layer the members lie in)
+    int xo;                  // float offset of that entry in the first x box
+    int sy;                  // slab row or -1
+    int yo;                  // float offset of the pair in the first y box (of the lane's column, outside the layer)
+    const float4 *py;        // its y profile row at E positions (the identity outside the layer)
+    int ph;                  // rows from there to the one at H positions
+};
+
+// one plane's auxiliaries for a pair
+struct PlaneX {
+    const float *base;       // staged-auxiliary region
+    int sz;                  // slab plane or -1
+    int zo, zeo;             // the pair's offsets in the first z H-type / E-type box
+    const float *xc;         // x coefficients of the pair's columns (b; c and 1/kappa TX floats on)
+};
+
+// CPML of one difference of the pair (see cpml2): psi <- b psi + c dif,
+// dif <- dif / kappa + psi
+struct PX {
+    F2 b, c, ki;
+};
+__device__ __forceinline__ PX profx(const float4 &q) { return PX{pk(q.x, q.x), pk(q.y, q.y), pk(q.z, q.z)}; }
+__device__ __forceinline__ PX profx(const float *xc) { return PX{ld2(xc), ld2(xc + TX), ld2(xc + 2 * TX)}; }
+__device__ __forceinline__ F2 cpmlx(F2 &dif, const PX &q, F2 o)
+{
+    const F2 p = fma2(q.b, o, mul2(q.c, dif));
+    dif = fma2(dif, q.ki, p);
+    return p;
+}
+
+// The x layer.  VEC: every pair lies wholly in a layer or outside and its
+// entries start on an 8-byte boundary (d and nx - 2 d even).  A pair never
+// has members in both layers (they are two cells apart at least).  Cells
+// outside the layer read 0.
+__device__ __forceinline__ F2 x_psi(const Pair &G, const float *box, bool vec)
+{
+    F2 o = 0;
+    if (vec) {
+        if (G.xm) o = ld2(box + G.xo);
+    } else {
+        float a = 0.f, b = 0.f;
+        if (G.xm & 1) a = box[G.xo];
+        if (G.xm & 2) b = box[G.xo + 1];
+        o = pk(a, b);
+    }
+    return o;
+}
+// both differences of the x layer at E (h = 0) or H (h = 1) positions
+__device__ __forceinline__ void cpml_x(const StepArgs &a, const Pair &G, const PlaneX &P, int h, bool vec, int k,
+                                       F2 &d0, F2 &d1)
+{
+    const int q = a.pg.xb >> 2, g = psi_x(a, G.xe, G.j, k), at = h ? PSI_HY_X : PSI_EY_X;
+    const float *b = P.base + (h ? 0 : 2 * q);
+    const PX pr = profx(P.xc + (h ? 3 * TX : 0));
+    const F2 p0 = cpmlx(d0, pr, x_psi(G, b, vec)), p1 = cpmlx(d1, pr, x_psi(G, b + q, vec));
+    put2(a.psi_out[at], g, p0, G.xm, vec, psi_n(a, 0), 3, a.bounds);
+    put2(a.psi_out[at + 1], g, p1, G.xm, vec, psi_n(a, 0), 3, a.bounds);
+}
+// of the y layer
+__device__ __forceinline__ void cpml_y(const StepArgs &a, const Pair &G, const PlaneX &P, int h, int k, F2 &d0, F2 &d1)
+{
+    const int q = a.pg.yb >> 2, g = psi_y(a, G.i, G.sy, k), at = h ? PSI_HX_Y : PSI_EX_Y;
+    const float *b = P.base + G.yo + (h ? 0 : 2 * q);
+    const PX pr = profx(G.py[h ? G.ph : 0]);
+    const F2 p0 = cpmlx(d0, pr, ld2(b)), p1 = cpmlx(d1, pr, ld2(b + q));
+    const int m = G.sy >= 0 ? G.m : 0;
+    put2(a.psi_out[at], g, p0, m, G.all, psi_n(a, 1), 3, a.bounds);
+    put2(a.psi_out[at + 1], g, p1, m, G.all, psi_n(a, 1), 3, a.bounds);
+}
+// of the z layer
+__device__ __forceinline__ void cpml_z(const StepArgs &a, const Pair &G, const PlaneX &P, const float *prof, int h,
+                                       F2 &d0, F2 &d1)
+{
+    const int g = psi_z(a, G.i, G.j, P.sz), at = h ? PSI_HX_Z : PSI_EX_Z;
+    const float *b = P.base + (h ? P.zo : P.zeo);
+    const PX pr = profx(prow(prof, 2, h, 2 * a.d)[P.sz]);
+    const F2 p0 = cpmlx(d0, pr, ld2(b)), p1 = cpmlx(d1, pr, ld2(b + (h ? H_COMP : PE_BYTES) / 4));
+    put2(a.psi_out[at], g, p0, G.m, G.all, psi_n(a, 2), 3, a.bounds);
+    put2(a.psi_out[at + 1], g, p1, G.m, G.all, psi_n(a, 2), 3, a.bounds);
+}
+
+// layers met by the cells an item updates (template bits)
+constexpr int LX = 1, LY = 2, LZ = 4;
+
+// H^{n+1/2} of a pair (h_core) from H^{n-1/2} in place; t0, t1: its cells'
+// coefficient rows.
+template <int L>
+__device__ __forceinline__ void h_corex(const StepArgs &a, const Pair &G, const PlaneX &P, const float *prof, int k,
+                                        bool vec, F2 ex, F2 ey, F2 ez, F2 ex_y1, F2 ez_y1, float ey_e, float ez_e,
+                                        F2 ex_z1, F2 ey_z1, const float4 *t0, const float4 *t1, F2 &hx, F2 &hy, F2 &hz)
+{
+    F2 hx_z = sub2(ey_z1, ey), hx_y = sub2(ez_y1, ez);
+    F2 hy_x = next_diff(ez, ez_e), hy_z = sub2(ex_z1, ex);
+    F2 hz_y = sub2(ex_y1, ex), hz_x = next_diff(ey, ey_e);
+    if constexpr (L & LX) cpml_x(a, G, P, 1, vec, k, hy_x, hz_x);
+    if constexpr (L & LY) cpml_y(a, G, P, 1, k, hx_y, hz_y);
+    if constexpr (L & LZ) cpml_z(a, G, P, prof, 1, hx_z, hy_z);
+    const F2 dx = sub2(hx_z, hx_y), dy = sub2(hy_x, hy_z), dz = sub2(hz_y, hz_x);
+    const float4 b0 = t0[0], b1 = t1[0];
+    hx = pk(__fmaf_rn(b0.x, lo2(dx), lo2(hx)), __fmaf_rn(b1.x, hi2(dx), hi2(hx)));
+    hy = pk(__fmaf_rn(b0.y, lo2(dy), lo2(hy)), __fmaf_rn(b1.y, hi2(dy), hi2(hy)));
+    hz = pk(__fmaf_rn(b0.z, lo2(dz), lo2(hz)), __fmaf_rn(b1.z, hi2(dz), hi2(hz)));
+}
+
+// Hx and Hy^{n+1/2} of a pair of the plane below an item, which the item
+// reads but does not update, in place; x / y auxiliaries that are not staged
+// there (flags f) come from global memory.
+__device__ __forceinline__ void h_belowx(const StepArgs &a, const Pair &G, const PlaneX &P, const float *prof, int f,
+                                         int k, F2 ex, F2 ey, F2 ez, F2 ez_y1, float ez_e, F2 ex_z1, F2 ey_z1,
+                                         const float4 *t0, const float4 *t1, F2 &hx, F2 &hy)
+{
+    F2 hx_z = sub2(ey_z1, ey), hx_y = sub2(ez_y1, ez);
+    F2 hy_x = next_diff(ez, ez_e), hy_z = sub2(ex_z1, ex);
+    auto far = [&](const float *arr, int g, int m, int u) {
+        float o0 = 0.f, o1 = 0.f;
+        if ((m & 1) && in_bounds(g, psi_n(a, u), 4, a.bounds)) o0 = __ldg(arr + g);
+        if ((m & 2) && in_bounds(g + 1, psi_n(a, u), 4, a.bounds)) o1 = __ldg(arr + g + 1);
+        return pk(o0, o1);
+    };
+    if (G.xm)
+        cpmlx(hy_x, profx(P.xc + 3 * TX), (f & F_X) ? x_psi(G, P.base, false)
+                                                    : far(a.psi_in[PSI_HY_X], psi_x(a, G.xe, G.j, k), G.xm, 0));
+    if (G.sy >= 0)
+        cpmlx(hx_y, profx(G.py[G.ph]), (f & F_Y) ? ld2(P.base + G.yo)
+                                                    : far(a.psi_in[PSI_HX_Y], psi_y(a, G.i, G.sy, k), G.m, 1));
+    if (P.sz >= 0) {
+        const PX q = profx(prow(prof, 2, 1, 2 * a.d)[P.sz]);
+        cpmlx(hx_z, q, ld2(P.base + P.zo));
+        cpmlx(hy_z, q, ld2(P.base + P.zo + H_COMP / 4));
+    }
+    const F2 dx = sub2(hx_z, hx_y), dy = sub2(hy_x, hy_z);
+    const float4 b0 = t0[0], b1 = t1[0];
+    hx = pk(__fmaf_rn(b0.x, lo2(dx), lo2(hx)), __fmaf_rn(b1.x, hi2(dx), hi2(hx)));
+    hy = pk(__fmaf_rn(b0.y, lo2(dy), lo2(hy)), __fmaf_rn(b1.y, hi2(dy), hi2(hy)));
+}
+
+// E^{n+1} of a pair (Eq. fdtdex with sigma E time-averaged: E = ca E +
+// cb [curl_h H^{n+1/2}], 1/dx in cb), in place; hz_w, hy_w: the cell before
+// the pair along x.
+template <int L>
+__device__ __forceinline__ void e_corex(const StepArgs &a, const Pair &G, const PlaneX &P, const float *prof, int k,
+                                        bool vec, F2 hx, F2 hy, F2 hz, F2 hz_ym, F2 hx_ym, float hz_w, float hy_w,
+                                        F2 hx_zm, F2 hy_zm, const float4 *t0, const float4 *t1, F2 &ex, F2 &ey, F2 &ez)
+{
+    F2 ex_y = sub2(hz, hz_ym), ex_z = sub2(hy, hy_zm);
+    F2 ey_z = sub2(hx, hx_zm), ey_x = prev_diff(hz, hz_w);
+    F2 ez_x = prev_diff(hy, hy_w), ez_y = sub2(hx, hx_ym);
+    if constexpr (L & LX) cpml_x(a, G, P, 0, vec, k, ey_x, ez_x);
+    if constexpr (L & LY) cpml_y(a, G, P, 0, k, ex_y, ez_y);
+    if constexpr (L & LZ) cpml_z(a, G, P, prof, 0, ex_z, ey_z);
+    const F2 dx = sub2(ex_y, ex_z), dy = sub2(ey_z, ey_x), dz = sub2(ez_x, ez_y);
+    const float4 a0 = t0[1], a1 = t1[1], b0 = t0[2], b1 = t1[2];
+    auto up = [](float ca, float e, float cb, float c) { return __fmaf_rn(ca, e, __fmul_rn(cb, c)); };
+    ex = pk(up(a0.x, lo2(ex), b0.x, lo2(dx)), up(a1.x, hi2(ex), b1.x, hi2(dx)));
+    ey = pk(up(a0.y, lo2(ey), b0.y, lo2(dy)), up(a1.y, hi2(ey), b1.y, hi2(dy)));
+    ez = pk(up(a0.z, lo2(ez), b0.z, lo2(dz)), up(a1.z, hi2(ez), b1.z, hi2(dz)));
 }
 
 // Current sources of the grid whose edges lie in a finished work item (Sec.
@@ -397,12 +580,16 @@ __device__ __forceinline__ uint32_t item_sources(const StepArgs &a, int launch, 
 // ---- shared-memory views ----------------------------------------------------
 struct EView {
     char *p;
-    __device__ float e(int c, int row, int col) const { return reinterpret_cast<const float *>(p + c * E_COMP)[row * EBX + col]; }
+    __device__ const float *at(int c, int row, int col) const { return reinterpret_cast<const float *>(p + c * E_COMP) + row * EBX + col; }
+    __device__ float e(int c, int row, int col) const { return *at(c, row, col); }
     __device__ int *hdr() const { return reinterpret_cast<int *>(p + OFF_HDR); }
 };
 struct HView {
     char *p;
-    __device__ float h(int c, int row, int col) const { return reinterpret_cast<const float *>(p + OFF_H + c * H_COMP)[row * HBX + col]; }
+    __device__ const float *at(int c, int row, int col) const { return reinterpret_cast<const float *>(p + OFF_H + c * H_COMP) + row * HBX + col; }
+    __device__ float h(int c, int row, int col) const { return *at(c, row, col); }
+    // the classes of a pair of cells, one per byte
+    __device__ uint32_t cls2(int row, int col) const { return *reinterpret_cast<const uint16_t *>(p + OFF_C + row * CBX + col); }
     __device__ int cls(int row, int col) const { return reinterpret_cast<const uint8_t *>(p + OFF_C)[row * CBX + col]; }
     __device__ const float *psi() const { return reinterpret_cast<const float *>(p + OFF_PSI); }
 };
@@ -431,10 +618,9 @@ __device__ __forceinline__ int y_off(const StepArgs &a, const Stg &sg, int x0, i
 
 // the staging of one plane applied to a cell's precomputed offsets
 __device__ __forceinline__ Slab slab_in(const Stg &sg, const HView &hv, int sx, int sy, int sz, int xo, int yo,
-                                        int zo, int zeo)
+                                        int zo)
 {
-    const bool z = sg.f & F_Z;
-    return Slab{sx, sy, sz, hv.psi(), (sg.f & F_X) ? xo : -1, (sg.f & F_Y) ? yo : -1, z ? zo : -1, z ? zeo : -1};
+    return Slab{sx, sy, sz, hv.psi(), (sg.f & F_X) ? xo : -1, (sg.f & F_Y) ? yo : -1, (sg.f & F_Z) ? zo : -1};
 }
 
 // x / y layer boxes of a tile (with its low halo): whether the tile touches
@@ -460,23 +646,6 @@ __device__ __forceinline__ int tile_boxes(const StepArgs &a, int x0, int y0, int
         ys = slab_of(yl < d ? yl : max(yl, a.ny - d), a.ny, d);
     }
     return f;
-}
-
-// staged-layer flags and box starts of plane z of a tile: the x and / or y
-// layer boxes of the tile, and the z boxes when the plane is in the z
-// layer (alone, unless the launch has room for all three)
-__device__ __forceinline__ void staging(const StepArgs &a, int x0, int y0, int z, int &f, int &xs, int &ys)
-{
-    f = 0;
-    xs = 0;
-    ys = 0;
-    if (a.d == 0 || z < 0 || z >= a.nz) return;
-    const bool zs = z < a.d || z >= a.nz - a.d;
-    if (zs && !a.zxy) {
-        f = F_Z;
-        return;
-    }
-    f = tile_boxes(a, x0, y0, xs, ys) | (zs ? F_Z : 0);
 }
 
 struct Item {
@@ -516,204 +685,256 @@ __device__ __forceinline__ bool item_in_cpml(const StepArgs &a, const Item &it)
     return xl < d || xh >= a.nx - d || yl < d || yh >= a.ny - d;
 }
 
+// A consumer warp's place in the two rings: the slot of the next plane and
+// the phase its full barrier is waited on, advanced slot by slot.
+template <int NH>
+struct Ring {
+    uint32_t e = 0, ep = 0, h = 0, hp = 0;   // E slot and phase, H slot and phase
+    __device__ uint32_t e_next() const { return (e + 1) % NE; }
+    __device__ void pass_e()
+    {
+        e = (e + 1) % NE;
+        ep ^= e == 0;
+    }
+    __device__ void pass_h()
+    {
+        h = h + 1 == NH ? 0 : h + 1;
+        hp ^= h == 0;
+    }
+};
+
 // shared state of the consumer warps
 template <int NH>
 struct Cons {
     const StepArgs *a;
     char *smem;
     const float *tab, *prof;
-    float *hnew;
+    float *hnew, *xc;
     uint64_t *bars;
     volatile int *abort;
     int warp, lane;
-    bool halo;               // the halo warp
     int hslot;               // bytes per H slot
     __device__ uint32_t bar(int b) const { return (uint32_t)__cvta_generic_to_shared(&bars[b]); }
     __device__ const float4 *coef(int cls) const { return reinterpret_cast<const float4 *>(tab + cls * kTabStride); }
-    __device__ uint32_t fullE(uint32_t q) const { return bar(q % NE); }
-    __device__ uint32_t emptyE(uint32_t q) const { return bar(NE + q % NE); }
-    __device__ uint32_t fullH(uint32_t q) const { return bar(2 * NE + q % NH); }
-    __device__ uint32_t emptyH(uint32_t q) const { return bar(2 * NE + NH_MAX + q % NH); }
-    __device__ EView ev(uint32_t q) const { return EView{smem + SM_EH + (q % NE) * ESLOT}; }
-    __device__ HView hv(uint32_t q) const { return HView{smem + SM_HH + (q % NH) * hslot}; }
-    __device__ float &hn(uint32_t b, int c, int row, int col) const { return hnew[(b * 3 + c) * HNEW_PLANE + row * HBX + col]; }
+    // barriers of a slot
+    __device__ uint32_t fullE(uint32_t s) const { return bar(s); }
+    __device__ uint32_t emptyE(uint32_t s) const { return bar(NE + s); }
+    __device__ uint32_t fullH(uint32_t s) const { return bar(2 * NE + s); }
+    __device__ uint32_t emptyH(uint32_t s) const { return bar(2 * NE + NH_MAX + s); }
+    __device__ EView ev(uint32_t s) const { return EView{smem + SM_EH + s * ESLOT}; }
+    __device__ HView hv(uint32_t s) const { return HView{smem + SM_HH + s * hslot}; }
+    __device__ float *hn(uint32_t b, int c, int row, int col) const { return hnew + (b * 3 + c) * HNEW_PLANE + row * HBX + col; }
     __device__ void arrive(uint32_t b) const
     {
         __syncwarp();
-        if (lane == 0) mbar_arrive(b);
+        asm volatile(
+            "{\n .reg .pred p;\n setp.eq.s32 p, %1, 0;\n @p mbarrier.arrive.shared::cta.b64 _, [%0];\n}\n" ::"r"(b),
+            "r"(lane)
+            : "memory");
     }
-    __device__ bool waitE(uint32_t q) const { return mbar_wait(fullE(q), (q / NE) & 1, abort); }
-    __device__ bool waitH(uint32_t q) const { return mbar_wait(fullH(q), (q / NH) & 1, abort); }
+    // wait for the E plane after the current one and the current H plane
+    // (the same answer in every lane)
+    __device__ bool wait_plane(const Ring<NH> &R) const
+    {
+        const uint32_t n = R.e_next();
+        return __all_sync(0xffffffffu, mbar_wait(fullE(n), R.ep ^ (n == 0), abort) &&
+                                           mbar_wait(fullH(R.h), R.hp, abort));
+    }
 };
 
-// one work item.  Its planes ka-1 .. kb occupy E slots qe0 .. qe0+kb-ka+1
-// and planes ka-1 .. kb-1 H slots qh0 .. qh0+kb-ka.  Returns false when a
-// wait gave up (the CTA then aborts).
+// a lane's pairs of three field components to global memory at element g
+template <typename Idx>
+__device__ __forceinline__ void put_fields(float *const *out, Idx g, F2 x, F2 y, F2 z, const Pair &G, long long n,
+                                           int site, int *bounds)
+{
+    put2(out[0], g, x, G.m, G.all, n, site, bounds);
+    put2(out[1], g, y, G.m, G.all, n, site, bounds);
+    put2(out[2], g, z, G.m, G.all, n, site, bounds);
+}
+
+// One work item in a row warp.  R is at the item's first plane, ka-1, on
+// entry and at the next item's on return.  A wait that gives up sets *abort;
+// the warp then goes through the item's remaining barriers without touching
+// the slots, so no other warp is left waiting, and the CTA leaves at the
+// item's end.
 // WIDE: 64-bit element indices for the field stores (grids of 2^31
 // elements or more); 32-bit otherwise, fewer registers in the plane loop
-template <bool CPML, int NH, bool WIDE>
-__device__ __forceinline__ bool run_item(const Cons<NH> &C, const Item &it, uint32_t qe0, uint32_t qh0, uint32_t &hb)
+// L: the layers the item's own cells meet
+template <int L, int NH, bool WIDE>
+__device__ __forceinline__ void run_rows(const Cons<NH> &C, const Item &it, Ring<NH> &R, uint32_t &hb)
 {
     using Idx = typename std::conditional<WIDE, long long, int>::type;
     const StepArgs &a = *C.a;
-    const int lane = C.lane;
-    const int lx = XO + lane, clx = CXO + lane;
-    const int i = it.x0 + lane;
-    const int d = a.d;
-    float ecur[3][RW], hxp[RW], hyp[RW];
-    int sy[RW], xo[RW], yo[RW];
-    const int sx = CPML ? slab_of(i, a.nx, d) : -1;
-    Stg tb(0, 0, 0);                // the tile's x / y layer boxes
-    if (CPML) tb.f = tile_boxes(a, it.x0, it.y0, tb.xs, tb.ys);
-    for (int r = 0; r < RW; ++r) {
-        const int row = 1 + C.warp + r * NCW, j = it.y0 + C.warp + r * NCW;
-        sy[r] = CPML ? slab_of(j, a.ny, d) : -1;
-        xo[r] = (CPML && (tb.f & F_X)) ? x_off(a, tb, i, row) : -1;
-        yo[r] = (CPML && (tb.f & F_Y)) ? y_off(a, tb, it.x0, i, j) : -1;
-        hxp[r] = 0.f;
-        hyp[r] = 0.f;
-    }
-    // halo cells of the halo warp: pass 0 = (i, y0-1), pass 1 = (x0-1, y0+lane)
-    int hxo[2] = {-1, -1}, hyo[2] = {-1, -1};
-    if (CPML && C.halo) {
-        if (tb.f & F_X) {
-            hxo[0] = x_off(a, tb, i, 0);
-            hxo[1] = x_off(a, tb, it.x0 - 1, 1 + lane);
+    const int lane = C.lane, d = a.d;
+    // the lane's pair of cells
+    const int row = 1 + C.warp + (lane / LPR) * NCW, gx = GX * (lane % LPR);
+    const int lx = XO + gx, clx = CXO + gx;
+    const bool vec = ((d | a.nx) & 1) == 0;
+    Pair G;
+    G.i = it.x0 + gx;
+    G.j = it.y0 + row - 1;
+    const int nv = G.j < a.ny ? max(0, min(GX, a.nx - G.i)) : 0;
+    G.m = (1 << nv) - 1;
+    G.all = it.x0 + TX <= a.nx && it.y0 + TY <= a.ny;
+    G.xm = G.xe = G.xo = 0;
+    G.sy = -1;
+    G.yo = 0;
+    G.py = reinterpret_cast<const float4 *>(C.xc + 6 * TX);      // the identity
+    G.ph = 0;
+    if (d > 0) {
+        Stg tb(0, 0, 0);                // the tile's x / y layer boxes
+        tb.f = tile_boxes(a, it.x0, it.y0, tb.xs, tb.ys);
+#pragma unroll
+        for (int c = 0; c < GX; ++c)
+            if (c < nv && slab_of(G.i + c, a.nx, d) >= 0) G.xm |= 1 << c;
+        G.xe = G.i < d ? G.i : G.i - (a.nx - 2 * d);
+        G.xo = a.ox / 4 + row * a.pg.w + G.xe - tb.xs;
+        if (nv > 0) G.sy = slab_of(G.j, a.ny, d);
+        G.yo = a.oy / 4 + (G.sy >= 0 ? G.sy - tb.ys : 0) * HBX + lx;
+        if (G.sy >= 0) {
+            G.py = prow(C.prof, 1, 0, 2 * d) + G.sy;
+            G.ph = 2 * d;
         }
-        if (tb.f & F_Y) {
-            hyo[0] = y_off(a, tb, it.x0, i, it.y0 - 1);
-            hyo[1] = y_off(a, tb, it.x0, it.x0 - 1, it.y0 + lane);
-        }
     }
-    bool ok = C.waitH(qh0);
+    auto row_of = [&](uint32_t cls) { return reinterpret_cast<const float4 *>(C.tab + (cls & 255u) * kTabStride); };
+    bool ok = __all_sync(0xffffffffu, mbar_wait(C.fullH(R.h), R.hp, C.abort));
     if (!ok) *C.abort = 1;
-    if (ok && !C.halo) {
-        const EView e0 = C.ev(qe0), e1 = C.ev(qe0 + 1);
-        const HView h0 = C.hv(qh0);
-        // owned E^n(ka) and, below the block, the owned Hx, Hy of plane ka-1
-        for (int r = 0; r < RW; ++r) {
-            const int row = 1 + C.warp + r * NCW;
-            for (int c = 0; c < 3; ++c) ecur[c][r] = e1.e(c, row, lx);
-        }
-        if (it.ka > 0) {
-            const int k = it.ka - 1;
-            for (int r = 0; r < RW; ++r) {
-                const int row = 1 + C.warp + r * NCW, j = it.y0 + C.warp + r * NCW;
-                if (i < a.nx && j < a.ny) {
-                    float hz;
-                    const Slab L = CPML ? slab_in(Stg(e0.hdr()), h0, sx, sy[r], slab_of(k, a.nz, d), xo[r], yo[r],
-                                                  row * HBX + lx, -1)
-                                        : Slab{-1, -1, -1, nullptr, -1, -1, -1, -1};
-                    h_core<CPML, false, false>(a, C.coef(h0.cls(row, clx)), C.prof, L, i, j, k, e0.e(0, row, lx),
-                                 e0.e(1, row, lx), e0.e(2, row, lx), e0.e(1, row, lx + 1), e0.e(2, row, lx + 1),
-                                 e0.e(0, row + 1, lx), e0.e(2, row + 1, lx), ecur[0][r], ecur[1][r],
-                                 h0.h(0, row, lx), h0.h(1, row, lx), h0.h(2, row, lx), hxp[r], hyp[r], hz);
-                }
-            }
-        }
+    // Hx, Hy of the plane below, kept where that plane's would be: the lane's
+    // own cells of the other H buffer
+    float *const own = C.hn(0, 0, row, lx);
+    F2 hx = 0, hy = 0, hz = 0;
+    if (ok && it.ka > 0) {
+        const EView e0 = C.ev(R.e), e1 = C.ev(R.e_next());
+        const HView h0 = C.hv(R.h);
+        const int k = it.ka - 1;
+        const PlaneX P{h0.psi(), d > 0 ? slab_of(k, a.nz, d) : -1, row * HBX + lx, 0, C.xc + gx};
+        const uint32_t cls = h0.cls2(row, clx);
+        hx = ld2(h0.at(0, row, lx));
+        hy = ld2(h0.at(1, row, lx));
+        h_belowx(a, G, P, C.prof, Stg(e0.hdr()).f, k, ld2(e0.at(0, row, lx)), ld2(e0.at(1, row, lx)),
+                 ld2(e0.at(2, row, lx)), ld2(e0.at(2, row + 1, lx)), e0.e(2, row, lx + GX), ld2(e1.at(0, row, lx)),
+                 ld2(e1.at(1, row, lx)), row_of(cls), row_of(cls >> 8), hx, hy);
     }
-    C.arrive(C.emptyE(qe0));
-    C.arrive(C.emptyH(qh0));
-    if (!ok) return false;
-    for (int k = it.ka; k < it.kb; ++k) {
-        const uint32_t t = (uint32_t)(k - it.ka);
-        const uint32_t qe = qe0 + 1 + t, qh = qh0 + 1 + t;     // plane k
-        ok = C.waitE(qe + 1) && C.waitH(qh);
+    st2(own + (hb ^ 1) * (3 * HNEW_PLANE), hx);
+    st2(own + (hb ^ 1) * (3 * HNEW_PLANE) + HNEW_PLANE, hy);
+    C.arrive(C.emptyE(R.e));
+    C.arrive(C.emptyH(R.h));
+    R.pass_e();
+    R.pass_h();
+    Idx g = (Idx)it.ka * (Idx)a.plane + (Idx)G.j * a.pitch + G.i;
+    const long long n = (long long)a.plane * a.nz;
+#pragma unroll 1
+    for (int k = it.ka; k < it.kb; ++k, g += (Idx)a.plane) {
+        ok = ok && C.wait_plane(R);
         if (!ok) *C.abort = 1;
-        const EView ek = C.ev(qe), ek1 = C.ev(qe + 1);
-        const HView hk = C.hv(qh);
-        const int sz = CPML ? slab_of(k, a.nz, d) : -1;
-        const Stg sg(ek.hdr());
-        float hnw[3][RW], enx[3][RW];
-        int cl[RW];
-        if (ok && !C.halo) {
-            for (int r = 0; r < RW; ++r) {
-                const int row = 1 + C.warp + r * NCW, j = it.y0 + C.warp + r * NCW;
-                for (int c = 0; c < 3; ++c) enx[c][r] = ek1.e(c, row, lx);
-                cl[r] = hk.cls(row, clx);
-                const float ex_y1 = ek.e(0, row + 1, lx);
-                const float ez_y1 = ek.e(2, row + 1, lx);
-                float hx = 0.f, hy = 0.f, hz = 0.f;
-                if (i < a.nx && j < a.ny) {
-                    const Idx g = (Idx)k * (Idx)a.plane + (Idx)j * a.pitch + i;
-                    const Slab L = CPML ? slab_in(sg, hk, sx, sy[r], sz, xo[r], yo[r], row * HBX + lx,
-                                                  (2 * H_COMP) / 4 + (row - 1) * TX + lane)
-                                        : Slab{-1, -1, -1, nullptr, -1, -1, -1, -1};
-                    h_core<CPML, true, true>(a, C.coef(cl[r]), C.prof, L, i, j, k, ecur[0][r], ecur[1][r],
-                                 ecur[2][r], ek.e(1, row, lx + 1), ek.e(2, row, lx + 1), ex_y1, ez_y1, enx[0][r],
-                                 enx[1][r], hk.h(0, row, lx), hk.h(1, row, lx), hk.h(2, row, lx), hx, hy, hz);
-                    if (in_bounds(g, (long long)a.plane * a.nz, 1, a.bounds)) {
-                        a.Hout[0][g] = hx;
-                        a.Hout[1][g] = hy;
-                        a.Hout[2][g] = hz;
-                    }
-                }
-                hnw[0][r] = hx;
-                hnw[1][r] = hy;
-                hnw[2][r] = hz;
-                C.hn(hb, 0, row, lx) = hx;
-                C.hn(hb, 1, row, lx) = hy;
-                C.hn(hb, 2, row, lx) = hz;
-            }
-        } else if (ok) {
-            // halo warp: low-y row (all lanes), then low-x column (TY lanes)
-            for (int pass = 0; pass < 2; ++pass) {
-                int hrow, hcol, hi, hj;
-                if (pass == 0) { hrow = 0; hcol = lx; hi = i; hj = it.y0 - 1; }
-                else { hrow = 1 + lane; hcol = XO - 1; hi = it.x0 - 1; hj = it.y0 + lane; }
-                if (pass == 1 && lane >= TY) break;
-                float hx = 0.f, hy = 0.f, hz = 0.f;
-                if (hi >= 0 && hj >= 0 && hi < a.nx && hj < a.ny) {
-                    const Slab L = CPML ? slab_in(sg, hk, slab_of(hi, a.nx, d), slab_of(hj, a.ny, d), sz, hxo[pass],
-                                                  hyo[pass], hrow * HBX + hcol, -1)
-                                        : Slab{-1, -1, -1, nullptr, -1, -1, -1, -1};
-                    h_core<CPML, false, false>(a, C.coef(hk.cls(hrow, hcol - XO + CXO)), C.prof, L, hi, hj, k,
-                                 ek.e(0, hrow, hcol), ek.e(1, hrow, hcol), ek.e(2, hrow, hcol),
-                                 ek.e(1, hrow, hcol + 1), ek.e(2, hrow, hcol + 1), ek.e(0, hrow + 1, hcol),
-                                 ek.e(2, hrow + 1, hcol), ek1.e(0, hrow, hcol), ek1.e(1, hrow, hcol),
-                                 hk.h(0, hrow, hcol), hk.h(1, hrow, hcol), hk.h(2, hrow, hcol), hx, hy, hz);
-                }
-                C.hn(hb, 0, hrow, hcol) = hx;
-                C.hn(hb, 1, hrow, hcol) = hy;
-                C.hn(hb, 2, hrow, hcol) = hz;
-            }
+        const EView ek = C.ev(R.e), ek1 = C.ev(R.e_next());
+        const HView hk = C.hv(R.h);
+        const PlaneX P{hk.psi(), (L & LZ) ? slab_of(k, a.nz, d) : -1, row * HBX + lx,
+                       OFF_ZE / 4 + (row - 1) * TX + gx, C.xc + gx};
+        float *const cur = own + hb * (3 * HNEW_PLANE), *const old = own + (hb ^ 1) * (3 * HNEW_PLANE);
+        F2 ex, ey, ez;
+        uint32_t cls = 0;
+        if (ok) {
+            ex = ld2(ek.at(0, row, lx));
+            ey = ld2(ek.at(1, row, lx));
+            ez = ld2(ek.at(2, row, lx));
+            cls = hk.cls2(row, clx);
+            hx = ld2(hk.at(0, row, lx));
+            hy = ld2(hk.at(1, row, lx));
+            hz = ld2(hk.at(2, row, lx));
+            h_corex<L>(a, G, P, C.prof, k, vec, ex, ey, ez, ld2(ek.at(0, row + 1, lx)), ld2(ek.at(2, row + 1, lx)),
+                       ek.e(1, row, lx + GX), ek.e(2, row, lx + GX), ld2(ek1.at(0, row, lx)),
+                       ld2(ek1.at(1, row, lx)), row_of(cls), row_of(cls >> 8), hx, hy, hz);
+            st2(cur, hx);
+            st2(cur + HNEW_PLANE, hy);
+            st2(cur + 2 * HNEW_PLANE, hz);
         }
         consumer_sync();            // H^{n+1/2} of plane k complete (tile + halo)
-        C.arrive(C.emptyE(qe));     // E(k) is not read again
-        if (*C.abort) {
-            C.arrive(C.emptyH(qh));
-            return false;
+        C.arrive(C.emptyE(R.e));    // E(k) is not read again
+        if (ok) {
+            put_fields(a.Hout, g, hx, hy, hz, G, n, 1, a.bounds);
+            e_corex<L>(a, G, P, C.prof, k, vec, hx, hy, hz, ld2(cur + 2 * HNEW_PLANE - HBX), ld2(cur - HBX),
+                       cur[2 * HNEW_PLANE - 1], cur[HNEW_PLANE - 1], ld2(old), ld2(old + HNEW_PLANE), row_of(cls),
+                       row_of(cls >> 8), ex, ey, ez);
+            put_fields(a.Eout, g, ex, ey, ez, G, n, 2, a.bounds);
         }
-        if (!C.halo) {
-            for (int r = 0; r < RW; ++r) {
-                const int row = 1 + C.warp + r * NCW, j = it.y0 + C.warp + r * NCW;
-                if (i < a.nx && j < a.ny) {
-                    const float hz_ym = C.hn(hb, 2, row - 1, lx);
-                    const float hx_ym = C.hn(hb, 0, row - 1, lx);
-                    const Idx g = (Idx)k * (Idx)a.plane + (Idx)j * a.pitch + i;
-                    const Slab L = CPML ? slab_in(sg, hk, sx, sy[r], sz, xo[r], yo[r], row * HBX + lx,
-                                                  (2 * H_COMP) / 4 + (row - 1) * TX + lane)
-                                        : Slab{-1, -1, -1, nullptr, -1, -1, -1, -1};
-                    float ex1, ey1, ez1;
-                    e_core<CPML>(a, C.coef(cl[r]), C.prof, L, i, j, k, ecur[0][r], ecur[1][r], ecur[2][r],
-                                 hnw[0][r], hnw[1][r], hnw[2][r], hz_ym, hx_ym, C.hn(hb, 2, row, lx - 1),
-                                 C.hn(hb, 1, row, lx - 1), hxp[r], hyp[r], ex1, ey1, ez1);
-                    if (in_bounds(g, (long long)a.plane * a.nz, 2, a.bounds)) {
-                        a.Eout[0][g] = ex1;
-                        a.Eout[1][g] = ey1;
-                        a.Eout[2][g] = ez1;
-                    }
-                }
-                hxp[r] = hnw[0][r];
-                hyp[r] = hnw[1][r];
-                for (int c = 0; c < 3; ++c) ecur[c][r] = enx[c][r];
-            }
-        }
-        C.arrive(C.emptyH(qh));     // this warp is done with plane k's H slot
+        C.arrive(C.emptyH(R.h));    // this warp is done with plane k's H slot
+        R.pass_e();
+        R.pass_h();
         hb ^= 1u;
     }
-    C.arrive(C.emptyE(qe0 + 1 + (uint32_t)(it.kb - it.ka)));   // plane kb (E only)
-    return true;
+    C.arrive(C.emptyE(R.e));        // plane kb (E only)
+    R.pass_e();
+}
+
+// The same item in a halo warp: H^{n+1/2} of the low-y row, cells (i, y0-1),
+// or of the low-x column, cells (x0-1, y0+lane), of every plane, recomputed
+// into the shared H planes.
+template <bool CPML, int NH>
+__device__ __forceinline__ void run_halo(const Cons<NH> &C, const Item &it, Ring<NH> &R, uint32_t &hb)
+{
+    const StepArgs &a = *C.a;
+    const int lane = C.lane, d = a.d;
+    Stg tb(0, 0, 0);
+    if (CPML) tb.f = tile_boxes(a, it.x0, it.y0, tb.xs, tb.ys);
+    const bool low_y = C.warp == NCW;
+    const int row = low_y ? 0 : 1 + lane, col = low_y ? XO + lane : XO - 1;
+    const int i = low_y ? it.x0 + lane : it.x0 - 1, j = low_y ? it.y0 - 1 : it.y0 + lane;
+    const bool act = low_y || lane < TY;
+    const bool in = act && i >= 0 && j >= 0 && i < a.nx && j < a.ny;
+    int sx = -1, sy = -1, xo = -1, yo = -1;
+    if (CPML && in) {
+        sx = slab_of(i, a.nx, d);
+        sy = slab_of(j, a.ny, d);
+        if (tb.f & F_X) xo = x_off(a, tb, i, row);
+        if (tb.f & F_Y) yo = y_off(a, tb, it.x0, i, j);
+    }
+    C.arrive(C.emptyE(R.e));        // the plane below the item has no halo
+    C.arrive(C.emptyH(R.h));
+    R.pass_e();
+    R.pass_h();
+    bool ok = true;
+#pragma unroll 1
+    for (int k = it.ka; k < it.kb; ++k) {
+        ok = ok && C.wait_plane(R);
+        if (!ok) *C.abort = 1;
+        if (ok && act) {
+            const EView ek = C.ev(R.e), ek1 = C.ev(R.e_next());
+            const HView hk = C.hv(R.h);
+            float hx = 0.f, hy = 0.f, hz = 0.f;
+            if (in) {
+                const Slab L = CPML ? slab_in(Stg(ek.hdr()), hk, sx, sy, slab_of(k, a.nz, d), xo, yo, row * HBX + col)
+                                    : Slab{-1, -1, -1, nullptr, -1, -1, -1};
+                h_core<CPML>(a, C.coef(hk.cls(row, col - XO + CXO)), C.prof, L, ek.e(0, row, col), ek.e(1, row, col),
+                             ek.e(2, row, col), ek.e(1, row, col + 1), ek.e(2, row, col + 1), ek.e(0, row + 1, col),
+                             ek.e(2, row + 1, col), ek1.e(0, row, col), ek1.e(1, row, col), hk.h(0, row, col),
+                             hk.h(1, row, col), hk.h(2, row, col), hx, hy, hz);
+            }
+            *C.hn(hb, 0, row, col) = hx;
+            *C.hn(hb, 1, row, col) = hy;
+            *C.hn(hb, 2, row, col) = hz;
+        }
+        C.arrive(C.emptyH(R.h));    // a halo warp reads the slot in the H half step only
+        consumer_sync();            // H^{n+1/2} of plane k complete (tile + halo)
+        C.arrive(C.emptyE(R.e));    // E(k) is not read again
+        R.pass_e();
+        R.pass_h();
+        hb ^= 1u;
+    }
+    C.arrive(C.emptyE(R.e));        // plane kb (E only)
+    R.pass_e();
+}
+
+// the x-layer coefficients of an item's columns (identity outside the layer
+// and the grid), one value per consumer thread, and the identity profile row
+__device__ __forceinline__ void fill_xc(const StepArgs &a, const float *prof, float *xc, int x0, int tid)
+{
+    if (tid < 4) xc[6 * TX + tid] = tid == 2 ? 1.f : 0.f;
+    for (int q = tid; q < 6 * TX; q += NCONS) {
+        const int w = q / TX, i = x0 + q - w * TX, half = w / 3, comp = w - 3 * half;
+        const int s = i < a.nx ? slab_of(i, a.nx, a.d) : -1;
+        xc[q] = s >= 0 ? prof[((half * 2 * a.d + s) << 2) + comp] : (comp == 2 ? 1.f : 0.f);
+    }
 }
 
 // domain of global work item q: item_start[d] <= q < item_start[d + 1]
@@ -728,10 +949,79 @@ __device__ __forceinline__ int find_domain(const int *item_start, int n, int q)
     return lo;
 }
 
+// the items of a consumer warp, in the order the producer hands them out
+template <bool ROWS, bool ZL, int NH, bool BATCH, bool WIDE>
+__device__ __forceinline__ void consume(const Cons<NH> &C, const BatchArgs &B, StepArgs *sa, int *cons_e, int *cons_h)
+{
+    Ring<NH> R;
+    uint32_t ce = 0, ch = 0, hb = 0;    // planes of the items before the current one
+    uint32_t item_e = 0;                // E planes of the current item
+    int cur = -1;                   // domain whose arguments are staged
+    const int tid = threadIdx.x;
+    while (true) {
+        // first plane of the next item (or the end marker)
+        if (!mbar_wait(C.fullE(R.e), R.ep, C.abort)) *C.abort = 1;
+        consumer_sync();
+        if (*C.abort) break;
+        ce += item_e;
+        ch += max(item_e, 1u) - 1;
+        const int *hdr = C.ev(R.e).hdr();
+        const int item = hdr[0], dom = hdr[5];
+        if (item < 0) break;
+        if (BATCH && dom != cur) {
+            // stage this domain's image -- its arguments, coefficient
+            // table rows and CPML profile rows, which the host laid out
+            // exactly as their shared-memory copy -- in one round of
+            // independent 16-byte loads
+            const int2 ref = __ldg(B.img_ref + (dom * 2 + B.launch) * 2 + B.parity);
+            const int4 *src = B.img + ref.x;
+            int4 *dst = reinterpret_cast<int4 *>(sa);
+            for (int q = tid; q < ref.y; q += NCONS) dst[q] = __ldg(src + q);
+            cur = dom;
+            consumer_sync();
+        }
+        const StepArgs &a = *C.a;
+        const Item it = decode(a, item);
+        const bool layer = item_in_cpml(a, it);
+        if (layer) fill_xc(a, C.prof, C.xc, it.x0, tid);
+        const uint32_t n = R.e_next();
+        if (!mbar_wait(C.fullE(n), R.ep ^ (n == 0), C.abort)) *C.abort = 1;
+        consumer_sync();
+        if (*C.abort) break;
+        if constexpr (ROWS) {
+            // the layers its own cells meet (its planes: all or none of them)
+            const int d = a.d;
+            const bool lx = d > 0 && (it.x0 < d || min(it.x0 + TX, a.nx) > a.nx - d);
+            const bool ly = d > 0 && (it.y0 < d || min(it.y0 + TY, a.ny) > a.ny - d);
+            constexpr int Z = ZL ? LZ : 0;
+            if (lx && ly) run_rows<LX | LY | Z, NH, WIDE>(C, it, R, hb);
+            else if (lx) run_rows<LX | Z, NH, WIDE>(C, it, R, hb);
+            else if (ly) run_rows<LY | Z, NH, WIDE>(C, it, R, hb);
+            else run_rows<Z, NH, WIDE>(C, it, R, hb);
+        } else {
+            if (layer) run_halo<true, NH>(C, it, R, hb);
+            else run_halo<false, NH>(C, it, R, hb);
+        }
+        if (!BATCH && a.n_isrc > 0) {
+            // current sources on the item's edges, after all its E stores
+            const uint32_t m = item_sources(a, B.launch, item);
+            if (m) {
+                consumer_sync();
+                if (ROWS && tid == 0) add_sources(a, m);
+            }
+        }
+        item_e = (uint32_t)(it.kb - it.ka) + 2;
+    }
+    if (ROWS && tid == 0) {
+        *cons_e = (int)ce;
+        *cons_h = (int)ch;
+    }
+}
+
 // BATCH = false: one domain whose arguments and descriptors are the kernel's
 // own parameters (constant bank); BATCH = true: a table of domains in global
 // memory, the current domain's arguments staged in shared memory.
-template <int NH, bool BATCH, bool WIDE>
+template <bool ZL, int NH, bool BATCH, bool WIDE>
 __global__ void __launch_bounds__(NTHREADS, 2) step_tma_kernel(const __grid_constant__ SingleArgs S,
                                                               const BatchArgs B)
 {
@@ -744,13 +1034,14 @@ __global__ void __launch_bounds__(NTHREADS, 2) step_tma_kernel(const __grid_cons
     float *tab = reinterpret_cast<float *>(smem + Lo.tab + al128(sizeof(StepArgs)));
     float *prof = tab + B.max_classes * kTabStride;  // [axis][E, H][2d] x {b, c, 1/kappa, -}, slab entries only
     float *hnew = reinterpret_cast<float *>(smem + Lo.hnew);
+    float *xc = reinterpret_cast<float *>(smem + Lo.xc);
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + Lo.bar);
     volatile int *abort = reinterpret_cast<volatile int *>(smem + Lo.misc);
     int *cons_e = reinterpret_cast<int *>(smem + Lo.misc + 4);
     int *cons_h = reinterpret_cast<int *>(smem + Lo.misc + 8);
     int *iss_e = reinterpret_cast<int *>(smem + Lo.misc + 12);
     int *iss_h = reinterpret_cast<int *>(smem + Lo.misc + 16);
-    Cons<NH> C{BATCH ? sa : &S.a, smem, tab, prof, hnew, bars, abort, warp, lane, warp == NCW, Lo.hslot};
+    Cons<NH> C{BATCH ? sa : &S.a, smem, tab, prof, hnew, xc, bars, abort, warp, lane, Lo.hslot};
 
     if (!BATCH) {
         // the one domain's coefficient table and CPML profiles, once
@@ -772,11 +1063,11 @@ __global__ void __launch_bounds__(NTHREADS, 2) step_tma_kernel(const __grid_cons
     if (threadIdx.x == 0) {
         for (int q = 0; q < NE; ++q) {
             mbar_init(C.fullE(q), 1);
-            mbar_init(C.emptyE(q), NCW + 1);
+            mbar_init(C.emptyE(q), NCW + NHW);
         }
         for (int q = 0; q < NH; ++q) {
             mbar_init(C.fullH(q), 1);
-            mbar_init(C.emptyH(q), NCW + 1);
+            mbar_init(C.emptyH(q), NCW + NHW);
         }
         *abort = 0;
         *cons_e = *cons_h = *iss_e = *iss_h = 0;
@@ -784,149 +1075,131 @@ __global__ void __launch_bounds__(NTHREADS, 2) step_tma_kernel(const __grid_cons
     }
     __syncthreads();
 
-    if (warp == NCW + 1) {
+    if (warp >= NCW) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(AUX_REGS));
+    if (warp >= NCW + NHW) {
         // ------------------------------ producer ------------------------------
-        if (lane == 0) {
-            uint32_t qe = 0, qh = 0;
+        // The whole warp runs the loop, every value the same in all lanes
+        // (item numbers come from lane 0 by shuffle), and one elected lane
+        // issues the copies: addresses and coordinates stay in uniform
+        // registers.  A plane's copies are few, one per kind of array, and
+        // H(z) goes with E(z + 1): the consumers need both to start plane z.
+        if (warp == NCW + NHW) {
+            uint32_t qe = 0, qh = 0, se = 0, sh = 0, pe = 1, ph = 1;   // planes issued, slots, empty phases
             bool ok = true;
+            auto wait = [&](uint32_t bar, uint32_t parity) {
+                return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort));
+            };
+            auto next_e = [&]() {
+                ++qe;
+                se = (se + 1) % NE;
+                pe ^= se == 0;
+            };
+            int next = lane == 0 ? atomicAdd(B.work, 1) : 0;
             while (ok) {
-                const int gitem = atomicAdd(B.work, 1);
+                const int gitem = __shfl_sync(0xffffffffu, next, 0);
                 if (gitem >= B.nitems) break;
                 const int dom = BATCH ? find_domain(B.item_start, B.n_domains, gitem) : 0;
                 const StepArgs &a = BATCH ? B.doms[dom].a[B.launch][B.parity] : S.a;
                 const TmaMaps &m = BATCH ? B.doms[dom].m[B.parity] : S.m;
                 const int item = BATCH ? gitem - __ldg(B.item_start + dom) : gitem;
-                const Item it = decode(a, item);
-                for (int z = it.ka - 1; z <= it.kb; ++z) {
-                    const bool e_only = (z == it.kb);
-                    int f = 0, xs = 0, ys = 0;
-                    if (!e_only) staging(a, it.x0, it.y0, z, f, xs, ys);
-                    if (!mbar_wait(C.emptyE(qe), ((qe / NE) & 1) ^ 1, abort)) { ok = false; break; }
-                    char *es = smem + SM_EH + (qe % NE) * ESLOT;
-                    int *hdr = reinterpret_cast<int *>(es + OFF_HDR);
-                    hdr[0] = item;
-                    hdr[1] = z;
-                    hdr[2] = f;
-                    hdr[3] = xs;
-                    hdr[4] = ys;
-                    hdr[5] = dom;
-                    mbar_expect_tx(C.fullE(qe), TX_E);
-                    for (int c = 0; c < 3; ++c)
-                        tma_load_3d(smem_u32(es + c * E_COMP), &m.e[c], it.x0 - XO, it.y0 - 1, z, C.fullE(qe));
-                    ++qe;
-                    if (e_only) continue;
-                    if (!mbar_wait(C.emptyH(qh), ((qh / NH) & 1) ^ 1, abort)) { ok = false; break; }
-                    char *hs = smem + SM_HH + (qh % NH) * Lo.hslot;
-                    const uint32_t txb = TX_H + ((f & F_Z) ? TX_Z : 0u) +
-                                         ((f & F_X) ? 4u * a.pg.w * HBY * 4 : 0u) +
-                                         ((f & F_Y) ? 4u * HBX * a.pg.hy * 4 : 0u);
-                    const uint32_t fb = C.fullH(qh);
-                    mbar_expect_tx(fb, txb);
-                    for (int c = 0; c < 3; ++c)
-                        tma_load_3d(smem_u32(hs + OFF_H + c * H_COMP), &m.h[c], it.x0 - XO, it.y0 - 1, z, fb);
-                    tma_load_3d(smem_u32(hs + OFF_C), &m.c, it.x0 - CXO, it.y0 - 1, z, fb);
-                    char *ps = hs + OFF_PSI;
-                    if (f & F_Z) {
-                        for (int q = 0; q < 2; ++q) {
-                            const int sz = slab_of(z, a.nz, a.d);     // plane of the compact z arrays
-                            tma_load_3d(smem_u32(ps + q * H_COMP), &m.zh[q], it.x0 - XO, it.y0 - 1, sz, fb);
-                            tma_load_3d(smem_u32(ps + 2 * H_COMP + q * PE_BYTES), &m.ze[q], it.x0, it.y0, sz, fb);
-                        }
+                Item it = decode(a, item);
+                it.x0 = __shfl_sync(0xffffffffu, it.x0, 0);
+                it.y0 = __shfl_sync(0xffffffffu, it.y0, 0);
+                it.ka = __shfl_sync(0xffffffffu, it.ka, 0);
+                it.kb = __shfl_sync(0xffffffffu, it.kb, 0);
+                const int nz = a.nz, d = a.d, ox = a.ox, oy = a.oy;
+                // x / y boxes of the tile, and what they add to a plane
+                int fxy = 0, xs = 0, ys = 0;
+                if (d > 0) fxy = tile_boxes(a, it.x0, it.y0, xs, ys);
+                const uint32_t tx_xy = ((fxy & F_X) ? 4u * a.pg.w * HBY * 4 : 0u) +
+                                       ((fxy & F_Y) ? 4u * HBX * a.pg.hy * 4 : 0u);
+                const bool zxy = a.zxy;
+                // plane z's layers and E boxes; f: its staged-layer flags
+                auto flags = [&](int z) {
+                    if (d == 0 || z < 0 || z >= nz) return 0;
+                    const bool zs = z < d || z >= nz - d;
+                    return zs ? F_Z | (zxy ? fxy : 0) : fxy;
+                };
+                auto load_e = [&](int z) {
+                    char *es = smem + SM_EH + se * ESLOT;
+                    if (elect_one()) {
+                        int *hdr = reinterpret_cast<int *>(es + OFF_HDR);
+                        hdr[0] = item;
+                        hdr[2] = flags(z);
+                        hdr[3] = xs;
+                        hdr[4] = ys;
+                        hdr[5] = dom;
+                        mbar_expect_tx(C.fullE(se), TX_E);
+                        tma_load(smem_u32(es), &m.e, it.x0 - XO, it.y0 - 1, z, C.fullE(se));
                     }
-                    if (f & F_X) {
-                        for (int q = 0; q < 2; ++q) {
-                            tma_load_3d(smem_u32(ps + a.ox + q * a.pg.xb), &m.xh[q], xs, it.y0 - 1, z, fb);
-                            tma_load_3d(smem_u32(ps + a.ox + (2 + q) * a.pg.xb), &m.xe[q], xs, it.y0 - 1, z, fb);
+                    __syncwarp();
+                    next_e();
+                };
+                if (!wait(C.emptyE(se), pe)) { ok = false; break; }
+                load_e(it.ka - 1);
+                for (int z = it.ka - 1; z < it.kb; ++z) {
+                    if (!wait(C.emptyH(sh), ph) || !wait(C.emptyE(se), pe)) { ok = false; break; }
+                    const int f = flags(z);
+                    char *hs = smem + SM_HH + sh * Lo.hslot, *ps = hs + OFF_PSI;
+                    const uint32_t fb = C.fullH(sh);
+                    if (elect_one()) {
+                        mbar_expect_tx(fb, TX_H + ((f & F_Z) ? TX_Z : 0u) + ((f & (F_X | F_Y)) ? tx_xy : 0u));
+                        tma_load(smem_u32(hs + OFF_H), &m.h, it.x0 - XO, it.y0 - 1, z, fb);
+                        tma_load(smem_u32(hs + OFF_C), &m.c, it.x0 - CXO, it.y0 - 1, z, fb);
+                        if (f & F_Z) {
+                            const int sz = z < d ? z : z - (nz - 2 * d);     // plane of the compact z arrays
+                            tma_load(smem_u32(ps), &m.zh, it.x0 - XO, it.y0 - 1, sz, fb);
+                            tma_load(smem_u32(ps + OFF_ZE), &m.ze, it.x0, it.y0, sz, fb);
                         }
+                        if (f & F_X) tma_load(smem_u32(ps + ox), &m.x, xs, it.y0 - 1, z, fb);
+                        if (f & F_Y) tma_load(smem_u32(ps + oy), &m.y, it.x0 - XO, ys, z, fb);
                     }
-                    if (f & F_Y) {
-                        char *py = ps + a.oy;
-                        for (int q = 0; q < 2; ++q) {
-                            tma_load_3d(smem_u32(py + q * a.pg.yb), &m.yh[q], it.x0 - XO, ys, z, fb);
-                            tma_load_3d(smem_u32(py + (2 + q) * a.pg.yb), &m.ye[q], it.x0 - XO, ys, z, fb);
-                        }
-                    }
+                    __syncwarp();
                     ++qh;
+                    sh = sh + 1 == NH ? 0 : sh + 1;
+                    ph ^= sh == 0;
+                    load_e(z + 1);
+                    // the next item's number travels while this one's last planes are issued
+                    if (z == max(it.ka - 1, it.kb - 3) && lane == 0) next = atomicAdd(B.work, 1);
                 }
             }
             if (ok) {
                 // end marker: an E slot whose header carries item -1
-                if (mbar_wait(C.emptyE(qe), ((qe / NE) & 1) ^ 1, abort)) {
-                    int *hdr = reinterpret_cast<int *>(smem + SM_EH + (qe % NE) * ESLOT + OFF_HDR);
-                    hdr[0] = -1;
-                    hdr[1] = 0;
-                    hdr[2] = 0;
-                    hdr[5] = -1;
-                    mbar_arrive(C.fullE(qe));
-                    ++qe;
+                if (wait(C.emptyE(se), pe)) {
+                    if (elect_one()) {
+                        int *hdr = reinterpret_cast<int *>(smem + SM_EH + se * ESLOT + OFF_HDR);
+                        hdr[0] = -1;
+                        hdr[2] = 0;
+                        hdr[5] = -1;
+                        mbar_arrive(C.fullE(se));
+                    }
+                    __syncwarp();
+                    next_e();
                 } else {
                     ok = false;
                 }
             }
-            if (!ok) {
-                *abort = 1;
-                atomicExch(B.err, 1);
-            }
-            *iss_e = (int)qe;
-            *iss_h = (int)qh;
-            // the last CTA to finish handing out work resets the counters
-            __threadfence();
-            if (atomicAdd(B.work + 1, 1) == (int)gridDim.x - 1) {
-                B.work[0] = 0;
-                B.work[1] = 0;
+            if (lane == 0) {
+                if (!ok) {
+                    *abort = 1;
+                    atomicExch(B.err, 1);
+                }
+                *iss_e = (int)qe;
+                *iss_h = (int)qh;
+                // the last CTA to finish handing out work resets the counters
                 __threadfence();
-            }
-        }
-    } else {
-        // ------------------------- row warps and halo warp -------------------------
-        uint32_t ce = 0, ch = 0, hb = 0;
-        int cur = -1;                   // domain whose arguments are staged
-        const int tid = threadIdx.x;
-        while (true) {
-            // first plane of the next item (or the end marker)
-            bool ok = C.waitE(ce);
-            if (!ok) *abort = 1;
-            consumer_sync();
-            if (*abort) break;
-            const int *hdr = C.ev(ce).hdr();
-            const int item = hdr[0], dom = hdr[5];
-            if (item < 0) break;
-            if (BATCH && dom != cur) {
-                // stage this domain's image -- its arguments, coefficient
-                // table rows and CPML profile rows, which the host laid out
-                // exactly as their shared-memory copy -- in one round of
-                // independent 16-byte loads
-                const int2 ref = __ldg(B.img_ref + (dom * 2 + B.launch) * 2 + B.parity);
-                const int4 *src = B.img + ref.x;
-                int4 *dst = reinterpret_cast<int4 *>(sa);
-                for (int q = tid; q < ref.y; q += NCONS) dst[q] = __ldg(src + q);
-                cur = dom;
-                consumer_sync();
-            }
-            const StepArgs &a = *C.a;
-            const Item it = decode(a, item);
-            ok = C.waitE(ce + 1);
-            if (!ok) *abort = 1;
-            consumer_sync();
-            if (*abort) break;
-            const bool done = item_in_cpml(a, it) ? run_item<true, NH, WIDE>(C, it, ce, ch, hb)
-                                                  : run_item<false, NH, WIDE>(C, it, ce, ch, hb);
-            if (!done) break;
-            if (!BATCH && a.n_isrc > 0) {
-                // current sources on the item's edges, after all its E stores
-                const uint32_t m = item_sources(a, B.launch, item);
-                if (m) {
-                    consumer_sync();
-                    if (tid == 0) add_sources(a, m);
+                if (atomicAdd(B.work + 1, 1) == (int)gridDim.x - 1) {
+                    B.work[0] = 0;
+                    B.work[1] = 0;
+                    __threadfence();
                 }
             }
-            ce += (uint32_t)(it.kb - it.ka) + 2;
-            ch += (uint32_t)(it.kb - it.ka) + 1;
         }
-        if (threadIdx.x == 0) {
-            *cons_e = (int)ce;
-            *cons_h = (int)ch;
-        }
+    } else if (warp >= NCW) {
+        consume<false, ZL, NH, BATCH, WIDE>(C, B, sa, cons_e, cons_h);
+    } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(ROW_REGS));
+        consume<true, ZL, NH, BATCH, WIDE>(C, B, sa, cons_e, cons_h);
     }
     __syncthreads();
     // on an abort, wait (bounded) for copies still in flight before the
@@ -935,10 +1208,10 @@ __global__ void __launch_bounds__(NTHREADS, 2) step_tma_kernel(const __grid_cons
         atomicExch(B.err, 1);
         const unsigned long long t0 = gtimer();
         for (int q = *cons_e; q < *iss_e; ++q)
-            while (!mbar_try(C.fullE(q), (q / NE) & 1))
+            while (!mbar_try(C.fullE(q % NE), (q / NE) & 1))
                 if (gtimer() - t0 > kWaitNs) break;
         for (int q = *cons_h; q < *iss_h; ++q)
-            while (!mbar_try(C.fullH(q), (q / NH) & 1))
+            while (!mbar_try(C.fullH(q % NH), (q / NH) & 1))
                 if (gtimer() - t0 > kWaitNs) break;
     }
 }
@@ -976,8 +1249,8 @@ PsiGeom step_psi_geom(int d, int nx, int ny)
     }
     pg.w = w;
     pg.hy = hy;
-    pg.xb = al128(pg.w * HBY * 4);
-    pg.yb = al128(HBX * pg.hy * 4);
+    pg.xb = pg.w * HBY * 4;
+    pg.yb = HBX * pg.hy * 4;
     return pg;
 }
 
@@ -987,34 +1260,31 @@ void step_region(const PsiGeom &pg, int zxy, int *region, int *ox, int *oy)
         *region = *ox = *oy = 0;
     } else if (zxy) {
         *ox = Z_BYTES;
-        *oy = Z_BYTES + 4 * pg.xb;
-        *region = *oy + 4 * pg.yb;
+        *oy = *ox + al128(4 * pg.xb);
+        *region = *oy + al128(4 * pg.yb);
     } else {
         *ox = 0;
-        *oy = 4 * pg.xb;
-        *region = std::max(Z_BYTES, *oy + 4 * pg.yb);
+        *oy = al128(4 * pg.xb);
+        *region = std::max(Z_BYTES, *oy + al128(4 * pg.yb));
     }
 }
-const void *step_kernel_ptr(int nh, bool batch, bool wide)
+// the kernel of launch l (1: the z-layer planes)
+using StepKernel = void (*)(SingleArgs, BatchArgs);
+static StepKernel step_kernel(int l, int nh, bool batch, bool wide)
 {
-    if (batch) return nh == 2 ? (const void *)step_tma_kernel<2, true, false> : (const void *)step_tma_kernel<3, true, false>;
-    if (wide) return nh == 2 ? (const void *)step_tma_kernel<2, false, true> : (const void *)step_tma_kernel<3, false, true>;
-    return nh == 2 ? (const void *)step_tma_kernel<2, false, false> : (const void *)step_tma_kernel<3, false, false>;
+    static const StepKernel k[2][2][3] = {
+        {{step_tma_kernel<false, 2, false, false>, step_tma_kernel<false, 2, false, true>, step_tma_kernel<false, 2, true, false>},
+         {step_tma_kernel<false, 3, false, false>, step_tma_kernel<false, 3, false, true>, step_tma_kernel<false, 3, true, false>}},
+        {{step_tma_kernel<true, 2, false, false>, step_tma_kernel<true, 2, false, true>, step_tma_kernel<true, 2, true, false>},
+         {step_tma_kernel<true, 3, false, false>, step_tma_kernel<true, 3, false, true>, step_tma_kernel<true, 3, true, false>}}};
+    return k[l][nh == 3][batch ? 2 : (wide ? 1 : 0)];
 }
+const void *step_kernel_ptr(int l, int nh, bool batch, bool wide) { return (const void *)step_kernel(l, nh, batch, wide); }
 
 cudaError_t launch_step(const SingleArgs &one, const BatchArgs &b, int grid, cudaStream_t s)
 {
     const int smem = smem_bytes(b.max_classes, b.max_d, b.region, b.nh);
-    const bool batch = b.doms != nullptr;
-    if (b.nh == 2) {
-        if (batch) step_tma_kernel<2, true, false><<<grid, NTHREADS, smem, s>>>(one, b);
-        else if (b.wide) step_tma_kernel<2, false, true><<<grid, NTHREADS, smem, s>>>(one, b);
-        else step_tma_kernel<2, false, false><<<grid, NTHREADS, smem, s>>>(one, b);
-    } else {
-        if (batch) step_tma_kernel<3, true, false><<<grid, NTHREADS, smem, s>>>(one, b);
-        else if (b.wide) step_tma_kernel<3, false, true><<<grid, NTHREADS, smem, s>>>(one, b);
-        else step_tma_kernel<3, false, false><<<grid, NTHREADS, smem, s>>>(one, b);
-    }
+    step_kernel(b.launch, b.nh, b.doms != nullptr, b.wide)<<<grid, NTHREADS, smem, s>>>(one, b);
     return cudaGetLastError();
 }
 
