@@ -260,7 +260,8 @@ int fdtd_add_probe(fdtd_grid *g, int kind, int i, int j, int k, int axis, int n_
                    int *probe_id);
 
 /* Planes per work item of the step kernel (the depth of a 32x16 column
- * tile; 0 = the default 16).  Tuning only; results do not depend on it.
+ * tile; 0 = the default, chosen from the grid's size, or in a batch from all
+ * its domains together).  Tuning only; results do not depend on it.
  * Before fdtd_finalize(); FDTD_EINVAL outside 0..256. */
 int fdtd_set_block(fdtd_grid *g, int planes);
 

@@ -1227,6 +1227,79 @@ cudaError_t ensure_smem(const void *kernel, int bytes)
     return e;
 }
 
+// ---- depth of the work items --------------------------------------------
+// Column tiles and planes of one domain, for the choice of the depth.
+struct Columns {
+    int cols, planes, d;     // column tiles, planes between the z layers, layer thickness
+};
+struct Depth {
+    int kz, kz1;             // planes per item between the z layers, in them
+};
+int blocks(int n, int k) { return (n + k - 1) / k; }
+
+// Planes per work item for domains that run together on `sms` SMs with
+// `slots` resident CTAs in all.  An item's plane takes 0.6 to 1.2 us however
+// empty the chip is, so with few items the longest one is the step's time;
+// with many it is their sum plus about half an item at the end.  In planes,
+// with an item's start worth 1.5 of them (3 in a z layer):
+//  - shallow items while one CTA per SM holds them all: a second CTA slows
+//    both (64^3, 8-cell CPML: 4 and 3 planes, 12.6 us a step; 2 and 3 planes
+//    on more CTAs than SMs 15.7; 16 and 8 planes 25.6);
+//  - else one wave of all slots, the z layers whole (128^3 with 8 cells: 16
+//    planes, 38.0 us; 8 planes 38.3; 32 planes 53.9), or one wave of thin
+//    z-layer items and then one of the others, whichever is shorter
+//    (100x100x80 with 10 cells: 2 and 6 planes 27.5 us, 10 and 8 planes 30.1);
+//  - else the least of (columns x (planes + 1.5 per item)) / slots + half an
+//    item, within 8 .. 14 planes (160x160x200 with 10 cells: 10 planes 70.4
+//    us, 16 planes 74.0; 512x512x384 with 12 cells: 12 planes 901, 16 planes
+//    908, 24 planes 942, as deeper items leave the planes their neighbours
+//    share in L2 for too long).
+Depth pick_depth(const std::vector<Columns> &doms, int sms, int slots)
+{
+    int planes = 1, d = 0;
+    for (const Columns &c : doms) {
+        planes = std::max(planes, c.planes);
+        d = std::max(d, c.d);
+    }
+    auto items = [&](int kz) {
+        long long n = 0;
+        for (const Columns &c : doms) n += (long long)c.cols * blocks(c.planes, kz);
+        return n;
+    };
+    auto z_items = [&](int kz1) {
+        long long n = 0;
+        for (const Columns &c : doms)
+            if (c.d > 0) n += 2LL * c.cols * blocks(c.d, std::min(kz1, c.d));
+        return n;
+    };
+    for (int k = 1; k <= 8; ++k)
+        if (items(k) + z_items(std::max(1, k - 1)) <= sms) return Depth{std::min(k, planes), std::max(1, k - 1)};
+    const int full = std::max(d, 1);
+    Depth one{0, full}, two{0, 0};
+    for (int k = 1; k <= 16 && !one.kz; ++k)
+        if (items(k) + z_items(full) <= slots) one.kz = k;
+    for (int k = 1; k <= 16 && !two.kz; ++k)
+        if (items(k) <= slots) two.kz = k;
+    for (int k = 1; d > 0 && k < full && !two.kz1; ++k)
+        if (z_items(k) <= slots) two.kz1 = k;
+    const double t_one = std::max(one.kz + 1.5, d > 0 ? d + 3.0 : 0.0), t_two = two.kz + 1.5 + two.kz1 + 3.0;
+    if (one.kz || (two.kz && two.kz1)) {
+        const Depth b = one.kz && (!two.kz || !two.kz1 || t_one <= t_two) ? one : two;
+        return Depth{std::min(b.kz, planes), b.kz1};
+    }
+    int best = 12;
+    double best_t = 1e30;
+    for (int k = 8; k <= 14; ++k) {
+        double t = 0.5 * (k + 1);
+        for (const Columns &c : doms) t += c.cols * (c.planes + 1.5 * blocks(c.planes, k)) / slots;
+        if (t < best_t) {
+            best_t = t;
+            best = k;
+        }
+    }
+    return Depth{std::min(best, planes), full};
+}
+
 int setup_step_kernel(fdtd_grid *g)
 {
     using namespace fdtd::geom;
@@ -1270,19 +1343,15 @@ int setup_step_kernel(fdtd_grid *g)
         if (l == 0) {            // planes between the z layers (all planes without a CPML)
             L.zlo = d;
             L.zhi = g->nz - d;
-            L.kz = std::min(L.zhi - L.zlo, g->block > 0 ? g->block : 16);
             L.zxy = 0;
-        } else {                 // the two z layers, one block each
+        } else {                 // the two z layers
             if (d == 0) break;
             L.zlo = 0;
             L.zhi = d;
             L.zlo2 = g->nz - d;
             L.zhi2 = g->nz;
-            L.kz = d;
             L.zxy = 1;
         }
-        const int nzb = (L.zhi - L.zlo + L.kz - 1) / L.kz + (L.zhi2 - L.zlo2 + L.kz - 1) / L.kz;
-        L.nitems = cols * nzb;
         fdtd::step_region(g->pg, L.zxy, &L.region, &L.ox, &L.oy);
         // three H slots (two planes of lookahead) unless that costs the
         // second resident CTA per SM
@@ -1297,14 +1366,23 @@ int setup_step_kernel(fdtd_grid *g)
     for (int q = 0; q < 4 && e == cudaSuccess; ++q)
         e = ensure_smem(fdtd::step_kernel_ptr(q >> 1, 2 + (q & 1), false, wide), max_smem);
     if (e != cudaSuccess) return cuda_fail(g, e, "step kernel setup");
+    int occ[2] = {1, 1};
     for (int l = 0; l < g->n_launch; ++l) {
         auto &L = g->lc[l];
-        int occ = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fdtd::step_kernel_ptr(l, L.nh, false, wide), fdtd::step_threads(),
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[l], fdtd::step_kernel_ptr(l, L.nh, false, wide),
+                                                          fdtd::step_threads(),
                                                           fdtd::step_smem_bytes(g->n_classes, d, L.region, L.nh));
         if (e != cudaSuccess) return cuda_fail(g, e, "step kernel occupancy");
-        if (occ < 1) return fail(g, FDTD_ECUDA, "step kernel does not fit on an SM");
-        L.grid = std::max(1, std::min(sms * occ, L.nitems));
+        if (occ[l] < 1) return fail(g, FDTD_ECUDA, "step kernel does not fit on an SM");
+    }
+    // planes per item: the caller's, or from the grid's size
+    Depth dep{g->block, d};
+    if (g->block <= 0) dep = pick_depth({Columns{cols, g->nz - 2 * d, d}}, sms, sms * occ[0]);
+    for (int l = 0; l < g->n_launch; ++l) {
+        auto &L = g->lc[l];
+        L.kz = l == 0 ? std::min(dep.kz, L.zhi - L.zlo) : std::min(dep.kz1, d);
+        L.nitems = cols * (blocks(L.zhi - L.zlo, L.kz) + blocks(L.zhi2 - L.zlo2, L.kz));
+        L.grid = std::max(1, std::min(sms * occ[l], L.nitems));
     }
     g->sms = sms;
     return FDTD_OK;
@@ -2438,18 +2516,13 @@ int fdtd_batch_create(int n, fdtd_grid *const *grids, void *cuda_stream, fdtd_ba
     b->step = grids[0]->step;
     // launch sizing over all domains
     std::vector<int> starts[2];
-    for (int l = 0; l < 2; ++l) starts[l].push_back(0);
     for (fdtd_grid *g : b->grids) {
         b->max_classes = std::max(b->max_classes, g->n_classes);
         b->max_d = std::max(b->max_d, g->d);
         b->n_launch = std::max(b->n_launch, g->n_launch);
         b->has_edges = b->has_edges || has_edge_work(g);
         b->has_wires = b->has_wires || !g->osegs.empty();
-        for (int l = 0; l < 2; ++l) {
-            const int items = l < g->n_launch ? g->lc[l].nitems : 0;
-            starts[l].push_back(starts[l].back() + items);
-            if (l < g->n_launch) b->region[l] = std::max(b->region[l], g->lc[l].region);
-        }
+        for (int l = 0; l < g->n_launch; ++l) b->region[l] = std::max(b->region[l], g->lc[l].region);
     }
     int dev = 0, sms = 0, smem_per_sm = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -2457,7 +2530,6 @@ int fdtd_batch_create(int n, fdtd_grid *const *grids, void *cuda_stream, fdtd_ba
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&smem_per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
     int max_smem = 0;
     for (int l = 0; l < b->n_launch && e == cudaSuccess; ++l) {
-        b->nitems[l] = starts[l].back();
         b->nh[l] = 3;
         if (2 * (fdtd::step_smem_bytes(b->max_classes, b->max_d, b->region[l], 3) + 1024) > smem_per_sm &&
             2 * (fdtd::step_smem_bytes(b->max_classes, b->max_d, b->region[l], 2) + 1024) <= smem_per_sm)
@@ -2466,15 +2538,43 @@ int fdtd_batch_create(int n, fdtd_grid *const *grids, void *cuda_stream, fdtd_ba
     }
     for (int q = 0; q < 4 && e == cudaSuccess; ++q)
         e = ensure_smem(fdtd::step_kernel_ptr(q >> 1, 2 + (q & 1), true, false), max_smem);
+    int occ[2] = {1, 1};
     for (int l = 0; l < b->n_launch && e == cudaSuccess; ++l) {
-        int occ = 0;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &occ, fdtd::step_kernel_ptr(l, b->nh[l], true, false), fdtd::step_threads(),
+            &occ[l], fdtd::step_kernel_ptr(l, b->nh[l], true, false), fdtd::step_threads(),
             fdtd::step_smem_bytes(b->max_classes, b->max_d, b->region[l], b->nh[l]));
-        if (e == cudaSuccess && occ < 1) { delete b; return FDTD_ECUDA; }
-        b->grid[l] = std::max(1, std::min(sms * std::max(occ, 1), b->nitems[l]));
+        if (e == cudaSuccess && occ[l] < 1) { delete b; return FDTD_ECUDA; }
     }
     if (e != cudaSuccess) { delete b; return FDTD_ECUDA; }
+    // planes per item: the callers', or, for the domains whose caller set
+    // none, one choice from all of them together (a domain's own choice would
+    // fill the chip by itself)
+    std::vector<Columns> open;
+    for (fdtd_grid *g : b->grids)
+        if (g->block <= 0) open.push_back(Columns{g->ncx * g->ncy, g->nz - 2 * g->d, g->d});
+    const Depth dep = open.empty() ? Depth{1, 1} : pick_depth(open, sms, sms * occ[0]);
+    std::vector<fdtd::DomainSlot> slots;
+    for (int l = 0; l < 2; ++l) starts[l].push_back(0);
+    for (fdtd_grid *g : b->grids) {
+        slots.push_back(g->slot_h);
+        for (int l = 0; l < 2; ++l) {
+            int items = 0;
+            if (l < g->n_launch) {
+                const auto &L = g->lc[l];
+                const int kz = g->block > 0 ? L.kz : (l == 0 ? std::min(dep.kz, L.zhi - L.zlo) : std::min(dep.kz1, g->d));
+                items = g->ncx * g->ncy * (blocks(L.zhi - L.zlo, kz) + blocks(L.zhi2 - L.zlo2, kz));
+                for (fdtd::StepArgs &a : slots.back().a[l]) {
+                    a.kz = kz;
+                    a.nitems = items;
+                }
+            }
+            starts[l].push_back(starts[l].back() + items);
+        }
+    }
+    for (int l = 0; l < b->n_launch; ++l) {
+        b->nitems[l] = starts[l].back();
+        b->grid[l] = std::max(1, std::min(sms * occ[l], b->nitems[l]));
+    }
     // device tables
     const size_t nd = b->grids.size();
     // staging images: per domain, launch and input parity its StepArgs, then
@@ -2512,7 +2612,7 @@ int fdtd_batch_create(int n, fdtd_grid *const *grids, void *cuda_stream, fdtd_ba
             }
             for (int l = 0; l < 2; ++l)
                 for (int par = 0; par < 2; ++par) {
-                    std::memcpy(im.data(), &g->slot_h.a[l][par], sizeof(fdtd::StepArgs));
+                    std::memcpy(im.data(), &slots[q].a[l][par], sizeof(fdtd::StepArgs));
                     img_ref[(q * 2 + l) * 2 + par] = int2{(int)img.size(), (int)(im.size() / 16)};
                     const int4 *v = reinterpret_cast<const int4 *>(im.data());
                     img.insert(img.end(), v, v + im.size() / 16);
@@ -2539,10 +2639,8 @@ int fdtd_batch_create(int n, fdtd_grid *const *grids, void *cuda_stream, fdtd_ba
     b->errf = b->work + 4;
     b->img = (int4 *)(base + o_img);
     b->img_ref = (int2 *)(base + o_ref);
-    std::vector<fdtd::DomainSlot> slots(nd);
     std::vector<fdtd::EdgeArgs> edges(2 * nd);
     for (size_t q = 0; q < nd; ++q) {
-        slots[q] = b->grids[q]->slot_h;
         edges[2 * q] = b->grids[q]->edge_h[0];
         edges[2 * q + 1] = b->grids[q]->edge_h[1];
     }
