@@ -56,6 +56,13 @@ int fdtd_mlp_backward(const void *x, int x_is_bf16, const float *z, const float 
 int fdtd_mlp_adam(float *w, float *m, float *v, const float *g, void *w_bf16, int count, float lr, float beta1,
                   float beta2, float eps, float weight_decay, int t, void *cuda_stream);
 
+/* The same step on n parameter tensors in as few launches as possible: host
+ * arrays of n device pointers (w_bf16 may be NULL, or hold NULLs), counts and
+ * weight decays (weight_decay NULL = 0). */
+int fdtd_mlp_adam_multi(int n, float *const *w, float *const *m, float *const *v, const float *const *g,
+                        void *const *w_bf16, const int *count, const float *weight_decay, float lr, float beta1,
+                        float beta2, float eps, int t, void *cuda_stream);
+
 /* Weighted squared error over rows x cols (row-major): loss[0] += scale *
  * sum_r w_r sum_c (y - target)^2 (atomic; clear it first) and
  * dy = 2 scale w_r (y - target).  row_weight [rows] may be NULL (w_r = 1);

@@ -56,6 +56,7 @@ def load():
         lib = ctypes.CDLL(path)
         P, I, D, S = ctypes.c_void_p, ctypes.c_int, ctypes.c_double, ctypes.c_size_t
         ip = ctypes.POINTER(ctypes.c_int)
+        PP = ctypes.POINTER(P)
         sig = {
             "fdtd_create_grid": (I, [I, I, I, D, D, ctypes.POINTER(CpmlParams), P, ctypes.POINTER(P)]),
             "fdtd_set_materials": (I, [P, P, ctypes.POINTER(Material), I]),
@@ -104,6 +105,8 @@ def load():
             "fdtd_mlp_backward": (I, [P, I, P, P, I, I, I, I, P, P, P, P, P, P]),
             "fdtd_mlp_adam": (I, [P, P, P, P, P, I, ctypes.c_float, ctypes.c_float, ctypes.c_float,
                                   ctypes.c_float, ctypes.c_float, I, P]),
+            "fdtd_mlp_adam_multi": (I, [I, PP, PP, PP, PP, PP, ip, ctypes.POINTER(ctypes.c_float), ctypes.c_float,
+                                        ctypes.c_float, ctypes.c_float, ctypes.c_float, I, P]),
             "fdtd_mlp_mse": (I, [P, P, P, I, I, ctypes.c_float, P, P, P]),
             "fdtd_mlp_row_rel_err": (I, [P, P, I, I, P, P]),
             "fdtd_mlp_gather_rows": (I, [P, P, I, I, P, P]),

@@ -19,7 +19,9 @@
 
 #include <algorithm>
 #include <cstdint>
+#include <map>
 #include <mutex>
+#include <utility>
 
 #include "fdtd.h"
 #include "fdtd_mlp.h"
@@ -34,37 +36,127 @@ __device__ __forceinline__ float gelu_grad(float z)
 }
 
 struct Epi {
-    int mode;                 // 0: forward (bias, act, bf16 / f32 / z outputs); 1: plain FP32 store
     const float *bias;
     int act;
     __nv_bfloat16 *yb;
     float *yf;
     float *zf;
-    int ldc;
 };
 
-__global__ void act_grad_kernel(const float *__restrict__ dy, const float *__restrict__ z, float *__restrict__ dz,
-                                long long count, int act)
+__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+__device__ __forceinline__ uint32_t cluster_rank()
 {
-    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < count;
-         q += (long long)gridDim.x * blockDim.x)
-        dz[q] = act == FDTD_ACT_GELU ? dy[q] * gelu_grad(z[q]) : dy[q];
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
 }
 
-// db[n] = sum over rows of dz[row][n]
-__global__ void colsum_kernel(const float *__restrict__ dz, int rows, int n, float *__restrict__ db)
+__device__ __forceinline__ void cluster_sync()
 {
-    const int col = blockIdx.x * blockDim.x + threadIdx.x;
-    if (col >= n) return;
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// address of this CTA's shared-memory object p in the cluster's CTA `rank`
+__device__ __forceinline__ uint32_t peer(const void *p, uint32_t rank)
+{
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+    return a;
+}
+__device__ __forceinline__ float ld_peer(uint32_t a)
+{
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ float4 ld_peer4(uint32_t a)
+{
+    float4 v;
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "r"(a));
+    return v;
+}
+
+// dz = dy act'(z) and, with db, its column sums, in one pass.  A cluster of
+// CTAs takes ZB_COLS columns, each CTA every gridDim.y-th part of the rows: its
+// 32 row lanes keep ZB_ROWS loads in flight each, their sums meet in shared
+// memory and the CTAs' in rank 0 through distributed shared memory, always in
+// the same order.  Bound by latency at a minibatch (256 x 256: the two
+// passes of before, elementwise and then a serial column sum on two CTAs,
+// took 3 + 17 us; this one 4), by DRAM far above it.
+constexpr int ZB_COLS = 32, ZB_LANES = 8, ZB_ROWS = 4, ZB_MAX_SPLIT = 8;
+__global__ void __launch_bounds__(ZB_COLS * ZB_LANES)
+    act_grad_kernel(const float *__restrict__ dy, const float *__restrict__ z, float *__restrict__ dz, int rows, int n,
+                    int act, float *__restrict__ db)
+{
+    __shared__ float part[ZB_LANES][ZB_COLS];
+    __shared__ float total[ZB_COLS];
+    const int c = threadIdx.x % ZB_COLS, lane = threadIdx.x / ZB_COLS;
+    const int col = blockIdx.x * ZB_COLS + c;
+    const int per = (rows + gridDim.y - 1) / gridDim.y;
+    const int r0 = blockIdx.y * per, r1 = min(r0 + per, rows);
     float s = 0.f;
-    for (int r = 0; r < rows; ++r) s += dz[(long long)r * n + col];
-    db[col] = s;
+    if (col < n)
+        for (int r = r0 + lane; r < r1; r += ZB_LANES * ZB_ROWS) {
+            float d[ZB_ROWS], a[ZB_ROWS];
+#pragma unroll
+            for (int u = 0; u < ZB_ROWS; ++u) {
+                const int rr = r + u * ZB_LANES;
+                const long long at = (long long)rr * n + col;
+                d[u] = rr < r1 ? __ldg(dy + at) : 0.f;
+                a[u] = rr < r1 && act == FDTD_ACT_GELU ? __ldg(z + at) : 0.f;
+            }
+#pragma unroll
+            for (int u = 0; u < ZB_ROWS; ++u) {
+                const int rr = r + u * ZB_LANES;
+                const float v = act == FDTD_ACT_GELU ? d[u] * gelu_grad(a[u]) : d[u];
+                if (rr < r1) dz[(long long)rr * n + col] = v;
+                s += v;
+            }
+        }
+    if (!db) return;                // the same for every CTA of the cluster
+    part[lane][c] = s;
+    __syncthreads();
+    if (lane == 0) {
+        float t = 0.f;
+#pragma unroll
+        for (int l = 0; l < ZB_LANES; ++l) t += part[l][c];
+        total[c] = t;
+    }
+    cluster_sync();
+    if (cluster_rank() == 0 && lane == 0 && col < n) {
+        float t = 0.f;
+        for (uint32_t q = 0; q < gridDim.y; ++q) t += ld_peer(peer(&total[c], q));
+        db[col] = t;
+    }
+    cluster_sync();                 // no CTA leaves while rank 0 may still read it
 }
 
-__global__ void adam_kernel(float *w, float *m, float *v, const float *g, __nv_bfloat16 *wb, int count, float lr,
-                            float b1, float b2, float eps, float wd, float c1, float c2)
+// Adam on up to ADAM_MAX parameter tensors in one launch: a tensor's blocks
+// are blk[q] .. blk[q + 1] - 1
+constexpr int ADAM_MAX = 16;
+struct AdamArgs {
+    float *w[ADAM_MAX], *m[ADAM_MAX], *v[ADAM_MAX];
+    const float *g[ADAM_MAX];
+    __nv_bfloat16 *wb[ADAM_MAX];
+    int count[ADAM_MAX];
+    float wd[ADAM_MAX];
+    int blk[ADAM_MAX + 1];
+    int n;
+};
+__global__ void adam_kernel(const __grid_constant__ AdamArgs A, float lr, float b1, float b2, float eps, float c1,
+                            float c2)
 {
-    for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < count; q += gridDim.x * blockDim.x) {
+    int t = 0;
+    while (t + 1 < A.n && (int)blockIdx.x >= A.blk[t + 1]) ++t;
+    const int b0 = A.blk[t], nb = A.blk[t + 1] - b0;
+    float *w = A.w[t], *m = A.m[t], *v = A.v[t];
+    const float *g = A.g[t];
+    __nv_bfloat16 *wb = A.wb[t];
+    const float wd = A.wd[t];
+    for (int q = (blockIdx.x - b0) * blockDim.x + threadIdx.x; q < A.count[t]; q += nb * blockDim.x) {
         const float gq = g[q];
         const float mq = b1 * m[q] + (1.f - b1) * gq;
         const float vq = b2 * v[q] + (1.f - b2) * gq * gq;
@@ -158,8 +250,6 @@ constexpr int TC_SMEM = 1024 + 1024 + (TC_M + TC_N) * TC_KMAX * 2;
 constexpr unsigned long long TC_WAIT_NS = 1000000000ull;      // 1 s per wait
 
 __device__ int g_mlp_err;     // a bounded wait ran out (read and cleared by fdtd_mlp_check)
-
-__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 __device__ __forceinline__ unsigned long long gtimer()
 {
@@ -410,19 +500,20 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
     }
 }
 
-// ---- tcgen05 gradient GEMM ---------------------------------------------------
+// ---- tcgen05 GEMM on strided operands ----------------------------------------
 // C[M x N] (FP32, row pitch N) = sum_k A(m, k) B(k, n) with
 // A(m, k) = A[m sam + k sak] and B(k, n) = B[k sbk + n sbn], FP32 or BF16
 // operands with any element strides (the gradients dz^T x and dz wt read
-// their operands transposed).  One CTA per 128 x 64 output tile; the
-// reduction runs in chunks of GC_K: all threads stage a chunk of both
-// operands into the K-major core-matrix layout (rounded to BF16 in
-// registers; threads walk the operand's contiguous index so the loads
-// coalesce), one thread issues its MMA chain into the TMEM accumulator and
-// commits it to an mbarrier, and every thread waits (bounded) before the
-// next chunk overwrites the tiles.  The epilogue is the forward layer's.
+// their operands transposed).  One CTA per 128 x 64 output tile and part of
+// the reduction, which runs in chunks of GC_K: all threads fetch a chunk of
+// both operands into registers, every load in flight at once, round it to
+// BF16 into the K-major core-matrix layout, one thread issues its MMA chain
+// into the TMEM accumulator and commits it to an mbarrier; the next chunk is
+// fetched meanwhile, and stored once the chain has read the tiles (a bounded
+// wait).  Threads walk the operand's contiguous index, so the loads coalesce.
 constexpr int GC_K = 128;
 constexpr int GC_SMEM = 1024 + 1024 + (TC_M + TC_N) * GC_K * 2;
+constexpr int GC_SPLIT = 8;          // CTAs of a cluster that share a tile's reduction, at most
 
 template <typename T>
 __device__ __forceinline__ float elem(const T *p)
@@ -431,43 +522,135 @@ __device__ __forceinline__ float elem(const T *p)
     else return *reinterpret_cast<const float *>(p);
 }
 
-// rows r0 .. r0 + R - 1 (row index fast in memory when s_row == 1) and
-// reduction indices k0 .. k0 + GC_K - 1 of X(row, k) = X[row s_row + k s_k]
-// (zero outside rows x K) into the core-matrix layout of a GC_K chunk:
-// 8 elements of one row at (r / 8) (GC_K 16) + (k / 8) 128 + (r % 8) 16
-template <typename T>
-__device__ __forceinline__ void stage_strided(char *dst, const T *X, long long s_row, long long s_k, int rows,
-                                              int K, int r0, int R, int k0, int tid)
-{
-    constexpr int kgs = GC_K / 8;
-    for (int q = tid; q < R * kgs; q += TC_THREADS) {
-        int r, g;
-        if (s_row == 1) { r = q % R; g = q / R; }
-        else { r = q / kgs; g = q % kgs; }
-        const int row = r0 + r, k = k0 + g * 8;
-        float f[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-            f[j] = (row < rows && k + j < K) ? elem(X + row * s_row + (long long)(k + j) * s_k) : 0.f;
-        *reinterpret_cast<uint4 *>(dst + (r >> 3) * (GC_K * 16) + g * 128 + (r & 7) * 16) =
-            make_uint4(pack2(f[0], f[1]), pack2(f[2], f[3]), pack2(f[4], f[5]), pack2(f[6], f[7]));
+// A chunk of one operand, this thread's share: rows r0 .. r0 + R - 1 and
+// reduction indices k0 .. k0 + GC_K - 1 of X(row, k) = X[row s_row + k s_k],
+// zero outside rows x kend, in groups of 8 along k
+template <typename T, int R>
+struct Chunk {
+    static constexpr int KGS = GC_K / 8, G = R * KGS / TC_THREADS;
+    float f[G][8];
+    __device__ __forceinline__ static void place(int u, int tid, bool row_fast, int &r, int &g)
+    {
+        const int q = tid + u * TC_THREADS;
+        if (row_fast) { r = q % R; g = q / R; }
+        else { r = q / KGS; g = q % KGS; }
     }
+    // vec: 16-byte loads along k are valid (FP32, s_k = 1, rows on 16-byte
+    // boundaries, kend a multiple of 4)
+    __device__ __forceinline__ void fetch(const T *X, long long s_row, long long s_k, int rows, int kend, int r0,
+                                          int k0, bool vec, int tid)
+    {
+#pragma unroll
+        for (int u = 0; u < G; ++u) {
+            int r, g;
+            place(u, tid, s_row == 1, r, g);
+            const int row = r0 + r, k = k0 + g * 8;
+            const T *p = X + row * s_row + (long long)k * s_k;
+            if (sizeof(T) == 4 && vec) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (row < rows && k + 4 * h < kend) v = __ldg(reinterpret_cast<const float4 *>(p) + h);
+                    f[u][4 * h] = v.x;
+                    f[u][4 * h + 1] = v.y;
+                    f[u][4 * h + 2] = v.z;
+                    f[u][4 * h + 3] = v.w;
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) f[u][j] = (row < rows && k + j < kend) ? elem(p + j * s_k) : 0.f;
+            }
+        }
+    }
+    // into the core-matrix layout of a GC_K chunk: 8 elements of one row at
+    // (r / 8) (GC_K 16) + (k / 8) 128 + (r % 8) 16
+    __device__ __forceinline__ void store(char *dst, bool row_fast, int tid) const
+    {
+#pragma unroll
+        for (int u = 0; u < G; ++u) {
+            int r, g;
+            place(u, tid, row_fast, r, g);
+            *reinterpret_cast<uint4 *>(dst + (r >> 3) * (GC_K * 16) + g * 128 + (r & 7) * 16) =
+                make_uint4(pack2(f[u][0], f[u][1]), pack2(f[u][2], f[u][3]), pack2(f[u][4], f[u][5]),
+                           pack2(f[u][6], f[u][7]));
+        }
+    }
+};
+
+// one operand with its strides
+template <typename T>
+struct Operand {
+    const T *p;
+    long long s_row, s_k;
+    __device__ bool vec(int kend) const
+    {
+        return sizeof(T) == 4 && s_k == 1 && (s_row & 3) == 0 && (kend & 3) == 0 &&
+               (reinterpret_cast<uintptr_t>(p) & 15) == 0;
+    }
+};
+
+// the accumulator of tile (m0, n0) over the chunks c0 .. c1 - 1 of a reduction
+// of K indices (at least one chunk); false when a wait gave up
+template <typename TA, typename TB>
+__device__ __forceinline__ bool gemm_chunks(const Operand<TA> &A, const Operand<TB> &B, int M, int N, int K, int m0,
+                                            int n0, int c0, int c1, char *As, char *Bs, uint32_t tmem, uint32_t bar,
+                                            int tid)
+{
+    const uint32_t sbo = GC_K * 16;
+    const bool va = A.vec(K), vb = B.vec(K);
+    Chunk<TA, TC_M> a;
+    Chunk<TB, TC_N> b;
+    a.fetch(A.p, A.s_row, A.s_k, M, K, m0, c0 * GC_K, va, tid);
+    b.fetch(B.p, B.s_row, B.s_k, N, K, n0, c0 * GC_K, vb, tid);
+    bool ok = true;
+    for (int c = c0; c < c1 && ok; ++c) {
+        a.store(As, A.s_row == 1, tid);
+        b.store(Bs, B.s_row == 1, tid);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncthreads();
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        if (tid == 0) {
+            const uint32_t a0 = smem_u32(As), b0 = smem_u32(Bs);
+            for (int kk = 0; kk < GC_K; kk += 16) {
+                const uint64_t ad = smem_desc(a0 + kk * 16, 128, sbo), bd = smem_desc(b0 + kk * 16, 128, sbo);
+                const uint32_t acc = (c > c0 || kk > 0) ? 1u : 0u;
+                asm volatile(
+                    "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+                    " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
+                    "l"(ad), "l"(bd), "r"(TC_IDESC), "r"(acc)
+                    : "memory");
+            }
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
+                         : "memory");
+        }
+        if (c + 1 < c1) {           // travels while the chain runs
+            a.fetch(A.p, A.s_row, A.s_k, M, K, m0, (c + 1) * GC_K, va, tid);
+            b.fetch(B.p, B.s_row, B.s_k, N, K, n0, (c + 1) * GC_K, vb, tid);
+        }
+        // the tiles are free again (and, after the last chunk, the accumulator complete)
+        const uint32_t parity = (uint32_t)((c - c0) & 1);
+        ok = __syncthreads_and(mbar_wait_bounded(bar, parity));
+        if (!ok) {
+            if (tid == 0) atomicExch(&g_mlp_err, 1);
+            mbar_wait_bounded(bar, parity);   // the chain still in flight, bounded again
+        }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    }
+    return ok;
 }
 
-template <typename TA, typename TB>
-__global__ void __launch_bounds__(TC_THREADS, 2)
-    tc_grad_kernel(const TA *__restrict__ A, long long sam, long long sak, const TB *__restrict__ B, long long sbk,
-                   long long sbn, int M, int N, int K, Epi ep)
+// shared-memory views and TMEM of a GEMM CTA
+struct GemmCta {
+    char *As, *Bs;
+    uint32_t bar, tmem;
+};
+__device__ __forceinline__ GemmCta gemm_begin(char *smraw, int tid)
 {
-    extern __shared__ __align__(1024) char smraw[];
     char *sm = smraw + ((1024u - (smem_u32(smraw) & 1023u)) & 1023u);
     uint64_t *bar = reinterpret_cast<uint64_t *>(sm);
     uint32_t *tslot = reinterpret_cast<uint32_t *>(sm + 8);
-    char *As = sm + 1024;
-    char *Bs = As + TC_M * GC_K * 2;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = blockIdx.x * TC_M, n0 = blockIdx.y * TC_N;
-    if (warp == 0) {
+    if (tid < 32) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
                      "r"(TC_N));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -479,119 +662,206 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem = *tslot;
-    const uint32_t sbo = GC_K * 16;
-    bool ok = true;
-    const int nchunk = (K + GC_K - 1) / GC_K;
-    for (int c = 0; c < nchunk && ok; ++c) {
-        const int k0 = c * GC_K;
-        // A rows are m, B rows are n (B(k, n) read as row n of B^T)
-        stage_strided(As, A, sam, sak, M, K, m0, TC_M, k0, tid);
-        stage_strided(Bs, B, sbn, sbk, N, K, n0, TC_N, k0, tid);
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncthreads();
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        if (tid == 0) {
-            const uint32_t a0 = smem_u32(As), b0 = smem_u32(Bs);
-            for (int kk = 0; kk < GC_K; kk += 16) {
-                const uint64_t ad = smem_desc(a0 + kk * 16, 128, sbo), bd = smem_desc(b0 + kk * 16, 128, sbo);
-                const uint32_t acc = (c > 0 || kk > 0) ? 1u : 0u;
-                asm volatile(
-                    "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                    " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-                    "l"(ad), "l"(bd), "r"(TC_IDESC), "r"(acc)
-                    : "memory");
-            }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                             smem_u32(bar))
-                         : "memory");
-        }
-        // the tiles are free again (and, after the last chunk, the accumulator complete)
-        bool done = mbar_wait_bounded(smem_u32(bar), (uint32_t)(c & 1));
-        ok = __syncthreads_and(done);
-        if (!ok) {
-            if (tid == 0) atomicExch(&g_mlp_err, 1);
-            mbar_wait_bounded(smem_u32(bar), (uint32_t)(c & 1));   // the chain still in flight, bounded again
-        }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    }
-    if (ok) {
-        const int lg = warp & 3, cc = (warp >> 2) * 32;
-        float *T = reinterpret_cast<float *>(As) + warp * 32 * TC_TS;
-        const int mrow = m0 + lg * 32;
-        if (n0 + cc < N) {
-            uint32_t v[32];
-            tmem_ld32(tmem + ((uint32_t)(lg * 32) << 16) + (uint32_t)cc, v);
-            if (ep.mode == 1) {
-                float y[32];
-                for (int j = 0; j < 32; ++j) y[j] = __uint_as_float(v[j]);
-                store_f32(T, y, ep.yf, mrow, M, n0 + cc, N, lane);
-            } else {
-                float z[32], y[32];
-                for (int j = 0; j < 32; ++j) {
-                    const int n = n0 + cc + j;
-                    z[j] = __uint_as_float(v[j]) + ((ep.bias && n < N) ? __ldg(ep.bias + n) : 0.f);
-                    y[j] = ep.act == FDTD_ACT_GELU ? gelu(z[j]) : z[j];
-                }
-                if (ep.zf) store_f32(T, z, ep.zf, mrow, M, n0 + cc, N, lane);
-                if (ep.yf) store_f32(T, y, ep.yf, mrow, M, n0 + cc, N, lane);
-                if (ep.yb) store_bf16(T, y, ep.yb, mrow, M, n0 + cc, N, lane);
-            }
-        }
-    }
+    return GemmCta{sm + 1024, sm + 1024 + TC_M * GC_K * 2, smem_u32(bar), *tslot};
+}
+__device__ __forceinline__ void gemm_end(const GemmCta &G, int tid)
+{
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (warp == 0) {
+    if (tid < 32) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TC_N) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(G.tmem), "r"(TC_N) : "memory");
     }
+}
+
+// forward layer with a large K: bias, activation and up to three outputs
+template <typename TA>
+__global__ void __launch_bounds__(TC_THREADS, 1)
+    tc_long_kernel(const TA *__restrict__ X, const __nv_bfloat16 *__restrict__ Wt, int M, int N, int K, Epi ep)
+{
+    extern __shared__ __align__(1024) char smraw[];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int m0 = blockIdx.x * TC_M, n0 = blockIdx.y * TC_N;
+    const GemmCta G = gemm_begin(smraw, tid);
+    const bool ok = gemm_chunks(Operand<TA>{X, K, 1}, Operand<__nv_bfloat16>{Wt, K, 1}, M, N, K, m0, n0, 0,
+                                (K + GC_K - 1) / GC_K, G.As, G.Bs, G.tmem, G.bar, tid);
+    const int lg = warp & 3, cc = (warp >> 2) * 32;
+    if (ok && n0 + cc < N) {
+        float *T = reinterpret_cast<float *>(G.As) + warp * 32 * TC_TS;
+        const int mrow = m0 + lg * 32;
+        uint32_t v[32];
+        tmem_ld32(G.tmem + ((uint32_t)(lg * 32) << 16) + (uint32_t)cc, v);
+        float z[32], y[32];
+        for (int j = 0; j < 32; ++j) {
+            const int n = n0 + cc + j;
+            z[j] = __uint_as_float(v[j]) + ((ep.bias && n < N) ? __ldg(ep.bias + n) : 0.f);
+            y[j] = ep.act == FDTD_ACT_GELU ? gelu(z[j]) : z[j];
+        }
+        if (ep.zf) store_f32(T, z, ep.zf, mrow, M, n0 + cc, N, lane);
+        if (ep.yf) store_f32(T, y, ep.yf, mrow, M, n0 + cc, N, lane);
+        if (ep.yb) store_bf16(T, y, ep.yb, mrow, M, n0 + cc, N, lane);
+    }
+    gemm_end(G, tid);
+}
+
+// Both products of a layer's backward pass in one launch: dw = dz^T x
+// (n x k, over the rows) and dx = dz wt (rows x k, over n).  The first
+// dw_tiles clusters take a dw tile each: their CTAs share its reduction over
+// the rows by chunks and add their accumulators, kept in shared memory,
+// through distributed shared memory, each CTA a part of the tile's rows, in
+// rank order.  In the clusters after them every CTA takes a dx tile.  One
+// tile of dw is 128 x 64, so a 256 x 256 layer has eight: the split over the
+// rows is what gives a large minibatch more CTAs.  At a minibatch of 256 rows
+// the pass is a chain of latencies (fetch, MMA, epilogue; one chunk per CTA).
+// Measured with act_grad_kernel, a whole backward pass of a layer: 256 -> 256
+// at 256 rows 36.0 us in four launches before, 13.8 in two now; at 4096 rows
+// 317 before, 41; 256 -> 512 at 4096 rows 332 before, 65.
+constexpr int GP_PITCH = TC_N + 4;   // floats per row of a CTA's partial tile
+static_assert(TC_M * GP_PITCH * 4 <= (TC_M + TC_N) * GC_K * 2, "a partial tile fits the operand area");
+
+template <typename TX>
+__global__ void __launch_bounds__(TC_THREADS, 1)
+    tc_backward_kernel(const float *__restrict__ dz, const TX *__restrict__ x, const __nv_bfloat16 *__restrict__ wt,
+                       int rows, int k, int n, float *dw, float *dx, int dw_tiles, int dx_tiles, int split)
+{
+    extern __shared__ __align__(1024) char smraw[];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int cluster = blockIdx.x / split, rank = blockIdx.x - cluster * split;
+    const GemmCta G = gemm_begin(smraw, tid);
+    const int lg = warp & 3, cc = (warp >> 2) * 32;
+    if (cluster < dw_tiles) {
+        // A(o, r) = dz[r n + o], B(r, c) = x[r k + c]
+        const int mt = (n + TC_M - 1) / TC_M;
+        const int m0 = (cluster % mt) * TC_M, n0 = (cluster / mt) * TC_N;
+        const int nchunk = (rows + GC_K - 1) / GC_K;
+        const int c0 = nchunk * rank / split, c1 = nchunk * (rank + 1) / split;
+        const bool ok = gemm_chunks(Operand<float>{dz, 1, n}, Operand<TX>{x, 1, k}, n, k, rows, m0, n0, c0, c1, G.As,
+                                    G.Bs, G.tmem, G.bar, tid);
+        float *part = reinterpret_cast<float *>(G.As);
+        uint32_t v[32];
+        tmem_ld32(G.tmem + ((uint32_t)(lg * 32) << 16) + (uint32_t)cc, v);
+        for (int j = 0; j < 32; j += 4)
+            *reinterpret_cast<uint4 *>(part + (lg * 32 + lane) * GP_PITCH + cc + j) =
+                make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+        cluster_sync();
+        const int per = TC_M / split;            // this CTA's rows of the tile
+        const bool vec = (k & 3) == 0 && (reinterpret_cast<uintptr_t>(dw) & 15) == 0;
+        for (int q = tid; ok && q < per * (TC_N / 4); q += TC_THREADS) {
+            const int r = rank * per + q / (TC_N / 4), c = (q % (TC_N / 4)) * 4;
+            float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int p = 0; p < split; ++p) {
+                const float4 u = ld_peer4(peer(part + r * GP_PITCH + c, p));
+                t.x += u.x;
+                t.y += u.y;
+                t.z += u.z;
+                t.w += u.w;
+            }
+            const int o = m0 + r, col = n0 + c;
+            if (o >= n) continue;
+            float *d = dw + (size_t)o * k + col;
+            if (vec && col + 3 < k) {
+                *reinterpret_cast<float4 *>(d) = t;
+            } else {
+                const float e[4] = {t.x, t.y, t.z, t.w};
+                for (int u = 0; u < 4; ++u)
+                    if (col + u < k) d[u] = e[u];
+            }
+        }
+        cluster_sync();                          // no CTA leaves while another may still read it
+    } else {
+        const int tile = (cluster - dw_tiles) * split + rank;
+        if (tile < dx_tiles) {
+            // A(r, o) = dz[r n + o], B(o, c) = wt[o k + c]
+            const int mt = (rows + TC_M - 1) / TC_M;
+            const int m0 = (tile % mt) * TC_M, n0 = (tile / mt) * TC_N;
+            const bool ok = gemm_chunks(Operand<float>{dz, n, 1}, Operand<__nv_bfloat16>{wt, 1, k}, rows, k, n, m0, n0,
+                                        0, (n + GC_K - 1) / GC_K, G.As, G.Bs, G.tmem, G.bar, tid);
+            if (ok && n0 + cc < k) {
+                float *T = reinterpret_cast<float *>(G.As) + warp * 32 * TC_TS;
+                uint32_t v[32];
+                tmem_ld32(G.tmem + ((uint32_t)(lg * 32) << 16) + (uint32_t)cc, v);
+                float y[32];
+                for (int j = 0; j < 32; ++j) y[j] = __uint_as_float(v[j]);
+                store_f32(T, y, dx, m0 + lg * 32, rows, n0 + cc, k, lane);
+            }
+        }
+    }
+    gemm_end(G, tid);
 }
 
 static_assert(TC_THREADS / 32 * 32 * TC_TS * 4 <= (TC_M + TC_N) * GC_K * 2, "transpose buffers fit the tile area");
 
-template <typename TA, typename TB>
-cudaError_t tc_grad(const TA *A, long long sam, long long sak, const TB *B, long long sbk, long long sbn, int M, int N,
-                    int K, const Epi &ep, cudaStream_t s)
+// raise a kernel's dynamic shared-memory limit once per device
+cudaError_t allow_smem(const void *kernel, int bytes)
 {
     static std::mutex mu;
-    static bool ready[64] = {};
+    static std::map<std::pair<int, const void *>, int> set;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if (dev >= 64) return cudaErrorInvalidDevice;
-    {
-        std::lock_guard<std::mutex> lock(mu);
-        if (!ready[dev]) {
-            e = cudaFuncSetAttribute(tc_grad_kernel<TA, TB>, cudaFuncAttributeMaxDynamicSharedMemorySize, GC_SMEM);
-            if (e != cudaSuccess) return e;
-            ready[dev] = true;
-        }
-    }
-    dim3 grid((M + TC_M - 1) / TC_M, (N + TC_N - 1) / TC_N);
-    tc_grad_kernel<TA, TB><<<grid, TC_THREADS, GC_SMEM, s>>>(A, sam, sak, B, sbk, sbn, M, N, K, ep);
+    std::lock_guard<std::mutex> lock(mu);
+    int &cur = set[{dev, kernel}];
+    if (cur >= bytes) return cudaSuccess;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) cur = bytes;
+    return e;
+}
+
+// a launch in clusters of cx x cy CTAs
+cudaLaunchConfig_t cluster_launch(dim3 grid, int threads, size_t smem, cudaStream_t s, int cx, int cy,
+                                  cudaLaunchAttribute *attr)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = (unsigned)cx;
+    attr->val.clusterDim.y = (unsigned)cy;
+    attr->val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
+template <typename TA>
+cudaError_t tc_long(const TA *x, const __nv_bfloat16 *wt, int M, int N, int K, const Epi &ep, cudaStream_t s)
+{
+    cudaError_t e = allow_smem((const void *)tc_long_kernel<TA>, GC_SMEM);
+    if (e != cudaSuccess) return e;
+    const dim3 grid((M + TC_M - 1) / TC_M, (N + TC_N - 1) / TC_N);
+    tc_long_kernel<TA><<<grid, TC_THREADS, GC_SMEM, s>>>(x, wt, M, N, K, ep);
     return cudaGetLastError();
+}
+
+// dw and / or dx (see tc_backward_kernel).  The split of dw: as many CTAs as
+// the reduction has chunks, up to eight
+template <typename TX>
+cudaError_t tc_backward(const float *dz, const TX *x, const __nv_bfloat16 *wt, int rows, int k, int n, float *dw,
+                        float *dx, cudaStream_t s)
+{
+    const void *kern = (const void *)tc_backward_kernel<TX>;
+    cudaError_t e = allow_smem(kern, GC_SMEM);
+    if (e != cudaSuccess) return e;
+    const int kt = (k + TC_N - 1) / TC_N;
+    const int dw_tiles = dw ? ((n + TC_M - 1) / TC_M) * kt : 0;
+    const long long dx_tiles = dx ? (long long)((rows + TC_M - 1) / TC_M) * kt : 0;
+    int split = 1;
+    while (dw && 2 * split <= GC_SPLIT && 2 * split <= (rows + GC_K - 1) / GC_K) split *= 2;
+    const long long clusters = dw_tiles + (dx_tiles + split - 1) / split;
+    cudaLaunchAttribute attr[1];
+    const cudaLaunchConfig_t cfg =
+        cluster_launch(dim3((unsigned)(clusters * split)), TC_THREADS, GC_SMEM, s, split, 1, attr);
+    return cudaLaunchKernelEx(&cfg, tc_backward_kernel<TX>, dz, x, wt, rows, k, n, dw, dx, dw_tiles, (int)dx_tiles, split);
 }
 
 template <typename TA>
 cudaError_t tc_forward(const TA *x, int rows, int K, const __nv_bfloat16 *wt, const float *bias, int N, int act,
                        __nv_bfloat16 *yb, float *yf, float *zf, cudaStream_t s)
 {
-    static std::mutex mu;
-    static bool ready[2][64] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    const cudaError_t e = allow_smem((const void *)tc_forward_kernel<TA>, TC_SMEM);
     if (e != cudaSuccess) return e;
-    if (dev >= 64) return cudaErrorInvalidDevice;
-    {
-        std::lock_guard<std::mutex> lock(mu);
-        bool &r = ready[sizeof(TA) == 2][dev];
-        if (!r) {
-            e = cudaFuncSetAttribute(tc_forward_kernel<TA>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
-            if (e != cudaSuccess) return e;
-            r = true;
-        }
-    }
     const int Kp = (K + 15) / 16 * 16;
     const bool xvec = sizeof(TA) == 2 && K % 8 == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0;
     const bool wvec = K % 8 == 0 && (reinterpret_cast<uintptr_t>(wt) & 15) == 0;
@@ -657,18 +927,6 @@ __global__ void net_pack_kernel(const __nv_bfloat16 *__restrict__ wt, int n, int
         const __nv_bfloat16 v = (ng < n && kk < k) ? wt[(long long)ng * k + kk] : __float2bfloat16_rn(0.f);
         *reinterpret_cast<__nv_bfloat16 *>(dst + r * per * 2 + core_off(nl, kk, kp)) = v;
     }
-}
-
-__device__ __forceinline__ uint32_t cluster_rank()
-{
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-
-__device__ __forceinline__ void cluster_sync()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 __device__ __forceinline__ void tmem_ld8(uint32_t addr, uint32_t (&v)[8])
@@ -899,7 +1157,7 @@ int fdtd_mlp_forward(const void *x, int x_is_bf16, int rows, int k, const void *
 {
     if (!x || !wt || rows < 0 || k < 1 || n < 1 || (act != FDTD_ACT_NONE && act != FDTD_ACT_GELU)) return FDTD_EINVAL;
     if (rows == 0) return FDTD_OK;
-    Epi ep{0, bias, act, static_cast<__nv_bfloat16 *>(y_bf16), y_f32, z_f32, n};
+    Epi ep{bias, act, static_cast<__nv_bfloat16 *>(y_bf16), y_f32, z_f32};
     const auto *w = static_cast<const __nv_bfloat16 *>(wt);
     cudaStream_t s = (cudaStream_t)cuda_stream;
     if (k <= TC_KMAX) {       // tensor-core path (every layer of the surrogate networks)
@@ -909,10 +1167,9 @@ int fdtd_mlp_forward(const void *x, int x_is_bf16, int rows, int k, const void *
         return rc(tc_forward(static_cast<const float *>(x), rows, k, w, bias, n, act,
                              static_cast<__nv_bfloat16 *>(y_bf16), y_f32, z_f32, s));
     }
-    // larger k: the chunked tensor-core GEMM, B(k, n) = wt[n * k + k']
-    if (x_is_bf16)
-        return rc(tc_grad(static_cast<const __nv_bfloat16 *>(x), k, 1, w, 1, k, rows, n, k, ep, s));
-    return rc(tc_grad(static_cast<const float *>(x), k, 1, w, 1, k, rows, n, k, ep, s));
+    // larger k: the chunked tensor-core GEMM
+    if (x_is_bf16) return rc(tc_long(static_cast<const __nv_bfloat16 *>(x), w, rows, n, k, ep, s));
+    return rc(tc_long(static_cast<const float *>(x), w, rows, n, k, ep, s));
 }
 
 int fdtd_mlp_net_pack_bytes(const int *sizes, int n_layers, size_t *bytes)
@@ -962,31 +1219,11 @@ int fdtd_mlp_net_forward(const float *x, int rows, const int *sizes, int n_layer
     if (rows == 0) return FDTD_OK;
     P.image = static_cast<const char *>(image);
     P.out_scale = out_scale;
-    static std::mutex mu;
-    static int ready_smem[64] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess || dev >= 64) return FDTD_ECUDA;
-    {
-        std::lock_guard<std::mutex> lock(mu);
-        if (ready_smem[dev] < smem) {
-            e = cudaFuncSetAttribute(net_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, NF_SMEM_MAX);
-            if (e != cudaSuccess) return FDTD_ECUDA;
-            ready_smem[dev] = NF_SMEM_MAX;
-        }
-    }
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(((rows + TC_M - 1) / TC_M) * NF_CLUSTER));
-    cfg.blockDim = dim3(NF_THREADS);
-    cfg.dynamicSmemBytes = (size_t)smem;
-    cfg.stream = (cudaStream_t)cuda_stream;
+    if (allow_smem((const void *)net_forward_kernel, NF_SMEM_MAX) != cudaSuccess) return FDTD_ECUDA;
     cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = NF_CLUSTER;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    const cudaLaunchConfig_t cfg =
+        cluster_launch(dim3((unsigned)(((rows + TC_M - 1) / TC_M) * NF_CLUSTER)), NF_THREADS, (size_t)smem,
+                       (cudaStream_t)cuda_stream, NF_CLUSTER, 1, attr);
     return rc(cudaLaunchKernelEx(&cfg, net_forward_kernel, x, rows, P, y));
 }
 
@@ -1012,25 +1249,29 @@ int fdtd_mlp_backward(const void *x, int x_is_bf16, const float *z, const float 
     if ((dw && !x) || (dx && !wt)) return FDTD_EINVAL;
     if (rows == 0) return FDTD_OK;
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    const long long cnt = (long long)rows * n;
-    act_grad_kernel<<<grid1d(cnt), 256, 0, s>>>(dy, z, dz, cnt, act);
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess && db) {
-        colsum_kernel<<<(n + 127) / 128, 128, 0, s>>>(dz, rows, n, db);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess && dw) {
-        // dw[n x k] = dz^T x: A(m=o, kk=r) = dz[r * n + o]; B(kk=r, c) = x[r * k + c]
-        Epi ep{1, nullptr, 0, nullptr, dw, nullptr, k};
-        if (x_is_bf16)
-            e = tc_grad(dz, 1, n, static_cast<const __nv_bfloat16 *>(x), k, 1, n, k, rows, ep, s);
-        else
-            e = tc_grad(dz, 1, n, static_cast<const float *>(x), k, 1, n, k, rows, ep, s);
-    }
-    if (e == cudaSuccess && dx) {
-        // dx[rows x k] = dz wt: A(r, o) = dz[r * n + o]; B(o, c) = wt[o * k + c]
-        Epi ep{1, nullptr, 0, nullptr, dx, nullptr, k};
-        e = tc_grad(dz, n, 1, static_cast<const __nv_bfloat16 *>(wt), k, 1, rows, k, n, ep, s);
+    // dz and db: as many CTAs per column group as leave each 64 rows, up to eight
+    int split = 1;
+    while (db && 2 * split <= ZB_MAX_SPLIT && rows / (2 * split) >= 64) split *= 2;
+    if (!db) split = (int)std::min<long long>((rows + 63) / 64, 65535);
+    cudaLaunchAttribute attr[1];
+    const cudaLaunchConfig_t cfg = cluster_launch(dim3((unsigned)((n + ZB_COLS - 1) / ZB_COLS), (unsigned)split),
+                                                  ZB_COLS * ZB_LANES, 0, s, 1, db ? split : 1, attr);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, act_grad_kernel, dy, z, dz, rows, n, act, db);
+    if (e == cudaSuccess && (dw || dx)) {
+        const auto *w = static_cast<const __nv_bfloat16 *>(wt);
+        auto run = [&](float *dwp, float *dxp) {
+            return x_is_bf16 ? tc_backward(dz, static_cast<const __nv_bfloat16 *>(x), w, rows, k, n, dwp, dxp, s)
+                             : tc_backward(dz, static_cast<const float *>(x), w, rows, k, n, dwp, dxp, s);
+        };
+        // one launch for both, unless dx overwrites the x that dw reads
+        const size_t cells = (size_t)rows * k;
+        const char *x0 = static_cast<const char *>(x), *d0 = reinterpret_cast<const char *>(dx);
+        if (dw && dx && x0 < d0 + cells * 4 && d0 < x0 + cells * (x_is_bf16 ? 2 : 4)) {
+            e = run(dw, nullptr);
+            if (e == cudaSuccess) e = run(nullptr, dx);
+        } else {
+            e = run(dw, dx);
+        }
     }
     return rc(e);
 }
@@ -1038,12 +1279,37 @@ int fdtd_mlp_backward(const void *x, int x_is_bf16, const float *z, const float 
 int fdtd_mlp_adam(float *w, float *m, float *v, const float *g, void *w_bf16, int count, float lr, float beta1,
                   float beta2, float eps, float weight_decay, int t, void *cuda_stream)
 {
-    if (!w || !m || !v || !g || count < 0 || t < 1) return FDTD_EINVAL;
-    if (count == 0) return FDTD_OK;
+    if (!w || !m || !v || !g) return FDTD_EINVAL;
+    return fdtd_mlp_adam_multi(1, &w, &m, &v, &g, &w_bf16, &count, &weight_decay, lr, beta1, beta2, eps, t, cuda_stream);
+}
+
+int fdtd_mlp_adam_multi(int n, float *const *w, float *const *m, float *const *v, const float *const *g,
+                        void *const *w_bf16, const int *count, const float *weight_decay, float lr, float beta1,
+                        float beta2, float eps, int t, void *cuda_stream)
+{
+    if (n < 0 || t < 1 || (n > 0 && (!w || !m || !v || !g || !count))) return FDTD_EINVAL;
+    for (int q = 0; q < n; ++q)
+        if (count[q] < 0 || (count[q] > 0 && (!w[q] || !m[q] || !v[q] || !g[q]))) return FDTD_EINVAL;
     const float c1 = 1.f - powf(beta1, (float)t), c2 = 1.f - powf(beta2, (float)t);
-    adam_kernel<<<grid1d(count), 256, 0, (cudaStream_t)cuda_stream>>>(
-        w, m, v, g, static_cast<__nv_bfloat16 *>(w_bf16), count, lr, beta1, beta2, eps, weight_decay, c1, c2);
-    return rc(cudaGetLastError());
+    for (int q0 = 0; q0 < n; q0 += ADAM_MAX) {
+        AdamArgs A{};
+        A.n = std::min(ADAM_MAX, n - q0);
+        for (int q = 0; q < A.n; ++q) {
+            A.w[q] = w[q0 + q];
+            A.m[q] = m[q0 + q];
+            A.v[q] = v[q0 + q];
+            A.g[q] = g[q0 + q];
+            A.wb[q] = w_bf16 ? static_cast<__nv_bfloat16 *>(w_bf16[q0 + q]) : nullptr;
+            A.count[q] = count[q0 + q];
+            A.wd[q] = weight_decay ? weight_decay[q0 + q] : 0.f;
+            A.blk[q + 1] = A.blk[q] + (count[q0 + q] > 0 ? grid1d(count[q0 + q]) : 0);
+        }
+        if (A.blk[A.n] == 0) continue;
+        adam_kernel<<<A.blk[A.n], 256, 0, (cudaStream_t)cuda_stream>>>(A, lr, beta1, beta2, eps, c1, c2);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return FDTD_ECUDA;
+    }
+    return FDTD_OK;
 }
 
 int fdtd_mlp_mse(const float *y, const float *target, const float *row_weight, int rows, int cols, float scale,

@@ -48,6 +48,21 @@ def adam(w, m, v, g, w_bf16, lr, t, beta1=0.9, beta2=0.999, eps=1e-8, weight_dec
                              weight_decay, int(t), _stream()), "mlp_adam")
 
 
+def _ptrs(ts):
+    return (ctypes.c_void_p * len(ts))(*[(t.data_ptr() if t is not None else None) for t in ts])
+
+
+def adam_multi(ws, ms, vs, gs, ws_bf16, lr, t, beta1=0.9, beta2=0.999, eps=1e-8, weight_decays=None):
+    """adam on lists of parameter tensors (ws_bf16 may hold None), in one
+    launch for up to sixteen of them"""
+    lib = _lib.load()
+    n = len(ws)
+    wd = (ctypes.c_float * n)(*[float(d) for d in weight_decays]) if weight_decays is not None else None
+    _check(lib.fdtd_mlp_adam_multi(n, _ptrs(ws), _ptrs(ms), _ptrs(vs), _ptrs(gs), _ptrs(ws_bf16),
+                                   _ints([w.numel() for w in ws]), wd, lr, beta1, beta2, eps, int(t), _stream()),
+           "mlp_adam_multi")
+
+
 def mse(y, target, scale, dy, loss, row_weight=None):
     lib = _lib.load()
     rows, cols = y.shape

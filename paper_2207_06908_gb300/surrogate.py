@@ -161,10 +161,10 @@ class Network:
 
     def adam(self, lr, weight_decay=0.0):
         self.t += 1
-        for i, p in enumerate(self.params):
-            wb = self.Wb[i // 2] if i % 2 == 0 else None
-            self.mlp.adam(p, self.m[i], self.v[i], self.g[i], wb, lr, self.t,
-                          weight_decay=weight_decay if i % 2 == 0 else 0.0)
+        n = len(self.params)
+        self.mlp.adam_multi(self.params, self.m, self.v, self.g,
+                            [self.Wb[i // 2] if i % 2 == 0 else None for i in range(n)], lr, self.t,
+                            weight_decays=[weight_decay if i % 2 == 0 else 0.0 for i in range(n)])
 
     def host_weights(self):
         return [p.cpu().numpy() for p in self.params]
