@@ -5,9 +5,10 @@
 // Oblique thin wires (Sec. 2.3, the Guiffaut formalism read in
 // Holland-Simpson form): a separate kernel, concurrent with the step
 // kernels, takes the segment currents to t_{n+1/2} from E^n gathered along
-// each segment and the node potentials; this kernel, before the sources,
-// adds those currents to E^{n+1} through the same edge shares and takes the
-// node charges to t_{n+1}.
+// each segment and the node potentials; after the step kernels and before
+// the sources those currents are added to E^{n+1} through the same edge
+// shares and the node charges taken to t_{n+1}: by a kernel of its own on a
+// single grid, by this one in a batch.
 // One CTA per grid (one per domain in a batch, for the gather as well); a
 // device-side step counter indexes the source samples and the probe slots,
 // so the launches can be replayed inside a CUDA graph.
@@ -60,9 +61,43 @@ __device__ __forceinline__ void wire_gather_body(const EdgeArgs &a, long long n)
     }
 }
 
-// second half, after the step kernels: the segment currents in Ampere's law
-// at t_{n+1/2} (four coupled edges per thread per pass, their field loads in
-// flight together), then the node charges to t_{n+1}
+// second half, after the step kernels: node m's charge to t_{n+1} from the
+// segment currents cur(s)
+template <class Cur>
+__device__ __forceinline__ void wire_node(const EdgeArgs &a, int m, Cur cur)
+{
+    const WireArgs &w = a.w;
+    const ONode nd = w.node[m];
+    if (nd.grounded) {
+        w.Q[m] = 0.f;
+        w.V[m] = 0.f;
+        return;
+    }
+    float net = 0.f;
+    for (int q = nd.adj0; q < nd.adj0 + nd.nadj; ++q) {
+        const int t = w.adj[q];
+        net += (t & 1) ? cur(t >> 1) : -cur(t >> 1);
+    }
+    // V^{n+1} from K Q^{n+1} = e0 V^{n+1} + sum_p P_p^{n+1}, the charge
+    // and polarisation updates substituted
+    float *P = w.P + (size_t)m * 4;
+    const float V = w.V[m], Q = w.Q[m];
+    float spb = 0.f, spa = 0.f;
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+        spb += nd.pb[p];
+        spa += nd.pa[p] * P[p];
+    }
+    const float Vn = (nd.K * (Q + a.dt * net) - (nd.cs + spb) * V - spa) / (nd.e0 + spb + nd.cs);
+#pragma unroll
+    for (int p = 0; p < 4; ++p) P[p] = nd.pa[p] * P[p] + nd.pb[p] * (Vn + V);
+    w.Q[m] = Q + a.dt * net - nd.cs / nd.K * (Vn + V);
+    w.V[m] = Vn;
+}
+
+// the same second half by one CTA of a batch: the segment currents in
+// Ampere's law at t_{n+1/2} (four coupled edges per thread per pass, their
+// field loads in flight together), then the node charges
 __device__ __forceinline__ void wire_scatter_body(const EdgeArgs &a)
 {
     const WireArgs &w = a.w;
@@ -94,50 +129,51 @@ __device__ __forceinline__ void wire_scatter_body(const EdgeArgs &a)
             a.E[sc[k].comp][sc[k].idx] = ev[k] - sum;
         }
     }
-    for (int m = threadIdx.x; m < w.n_node; m += blockDim.x) {
-        const ONode nd = w.node[m];
-        if (nd.grounded) {
-            w.Q[m] = 0.f;
-            w.V[m] = 0.f;
-            continue;
-        }
-        float net = 0.f;
-        for (int q = nd.adj0; q < nd.adj0 + nd.nadj; ++q) {
-            const int t = w.adj[q];
-            net += (t & 1) ? cur(t >> 1) : -cur(t >> 1);
-        }
-        // V^{n+1} from K Q^{n+1} = e0 V^{n+1} + sum_p P_p^{n+1}, the charge
-        // and polarisation updates substituted
-        float *P = w.P + (size_t)m * 4;
-        const float V = w.V[m], Q = w.Q[m];
-        float spb = 0.f, spa = 0.f;
-#pragma unroll
-        for (int p = 0; p < 4; ++p) {
-            spb += nd.pb[p];
-            spa += nd.pa[p] * P[p];
-        }
-        const float Vn = (nd.K * (Q + a.dt * net) - (nd.cs + spb) * V - spa) / (nd.e0 + spb + nd.cs);
-#pragma unroll
-        for (int p = 0; p < 4; ++p) P[p] = nd.pa[p] * P[p] + nd.pb[p] * (Vn + V);
-        w.Q[m] = Q + a.dt * net - nd.cs / nd.K * (Vn + V);
-        w.V[m] = Vn;
-    }
+    for (int m = threadIdx.x; m < w.n_node; m += blockDim.x) wire_node(a, m, cur);
     __syncthreads();
 }
 
+// WIRES: the oblique wires' second half first
+template <bool WIRES>
 __device__ __forceinline__ void edge_body(const EdgeArgs &a)
 {
     __shared__ long long n_s;
     if (threadIdx.x == 0) n_s = __ldcg(a.step) + a.step_t;
     __syncthreads();
     const long long n = n_s;
-    if (a.w.n_seg > 0 && !a.wire_done) wire_scatter_body(a);
+    if (WIRES && a.w.n_seg > 0) wire_scatter_body(a);
     src_probe_body(a, n);
 }
 
-__global__ void edge_kernel(const EdgeArgs a) { edge_body(a); }
+__global__ void edge_kernel(const EdgeArgs a) { edge_body<false>(a); }
 
-__global__ void wire_finish_kernel(const EdgeArgs a) { wire_scatter_body(a); }
+// The second half on a single grid: a thread per coupled edge, then per node
+// (the charges read the currents only), over as many CTAs as that takes.  A
+// serial launch after the step kernels, so what counts is its chain of
+// dependent loads; one CTA's 1024 threads going round (wire_scatter_body)
+// took 11.5 us with the sources and probes on a 617-segment tower, this and
+// the probes beside the next step 3.
+constexpr int kWireThreads = 128;
+__global__ void __launch_bounds__(kWireThreads) wire_finish_kernel(const EdgeArgs a)
+{
+    const WireArgs &w = a.w;
+    auto cur = [&](int s) { return __ldg(w.I + s); };
+    const int u = blockIdx.x * kWireThreads + threadIdx.x;
+    if (u < w.n_scat) {
+        OScat sc = w.scat[u];
+        if (!in_bounds(sc.idx, a.plane * a.nz, 9, a.bounds)) sc.idx = 0;   // bounds-checked build only
+        float *e = a.E[sc.comp] + sc.idx;
+        const float old = *e;
+        float sum = 0.f;
+        for (int t = sc.t0; t < sc.t0 + sc.nt; ++t) {
+            const OTerm tm = w.term[t];
+            sum += tm.ws * cur(tm.seg);
+        }
+        *e = old - sum;
+    } else if (u - w.n_scat < w.n_node) {
+        wire_node(a, u - w.n_scat, cur);
+    }
+}
 
 __global__ void wire_gather_kernel(const EdgeArgs a)
 {
@@ -152,7 +188,7 @@ __global__ void edge_batch_kernel(const EdgeArgs *e, int parity)
     __shared__ EdgeArgs a;
     if (threadIdx.x == 0) a = e[2 * blockIdx.x + parity];
     __syncthreads();
-    if (a.n_src > 0 || a.n_probes > 0 || a.w.n_seg > 0) edge_body(a);
+    if (a.n_src > 0 || a.n_probes > 0 || a.w.n_seg > 0) edge_body<true>(a);
 }
 
 // one CTA per domain of a batch: the oblique wires' first half of the step
@@ -172,16 +208,14 @@ __global__ void wire_gather_batch_kernel(const EdgeArgs *e, int parity)
 
 cudaError_t launch_edges(const EdgeArgs &a, cudaStream_t s)
 {
-    // oblique wires are latency-bound loops over their segments and edges:
-    // a full CTA keeps enough loads in flight
-    const bool wires = a.w.n_seg > 0;
-    edge_kernel<<<1, wires ? 1024 : 128, wires ? kWireSegShared * sizeof(float) : 0, s>>>(a);
+    edge_kernel<<<1, 128, 0, s>>>(a);
     return cudaGetLastError();
 }
 
 cudaError_t launch_wire_finish(const EdgeArgs &a, cudaStream_t s)
 {
-    wire_finish_kernel<<<1, 1024, kWireSegShared * sizeof(float), s>>>(a);
+    const int n = a.w.n_scat + a.w.n_node;
+    wire_finish_kernel<<<(n + kWireThreads - 1) / kWireThreads, kWireThreads, 0, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -249,7 +249,6 @@ struct EdgeArgs {
     int npoles;
     const float *Ein[3];     // E^n, the step's input (oblique wires read it)
     WireArgs w;              // oblique wires (n_seg = 0: none)
-    int wire_done;           // the wires' scatter and charges ran before the Debye kernel
     int step_t;              // this launch serves step *step + step_t
     int advance;             // 1: set *step to that step + 1 when done
     int skip_src;            // the current sources ran in the step kernel
@@ -301,8 +300,9 @@ cudaError_t launch_edges(const EdgeArgs &a, cudaStream_t s);
 // oblique wires: segment currents to t_{n+1/2}; needs only the step's inputs,
 // so it may run concurrently with the step kernels, and before launch_edges
 cudaError_t launch_wire_gather(const EdgeArgs &a, cudaStream_t s);
-// oblique wires in Debye media: their scatter into E^{n+1} and node charges,
-// before the dispersive-media kernel (which then sees the wire currents)
+// oblique wires of a single grid: their scatter into E^{n+1} and node charges,
+// after the step kernels, before launch_edges and the dispersive-media kernel
+// (which then sees the wire currents)
 cudaError_t launch_wire_finish(const EdgeArgs &a, cudaStream_t s);
 cudaError_t launch_debye(const DebyeArgs &a, cudaStream_t s);
 // one CTA per domain: e[2 * d + parity]; wires: some domain has oblique wires

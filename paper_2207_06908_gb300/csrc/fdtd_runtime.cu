@@ -58,36 +58,50 @@ size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 // update disjoint planes from the previous step's buffers only, so one step
 // runs them concurrently: the z layers on a side stream forked from the
 // step's stream and joined back to it before the source / probe kernel.
+// Small launches that need only the step's inputs (the oblique wires'
+// gather, the probes of the step before) run on a second one: before the z
+// layers on theirs they would hold those back until the interior launch has
+// taken every SM (160x160x200 tower: 92 us a step so, 79 beside them).
 struct Fork {
-    cudaStream_t side = nullptr;
-    cudaEvent_t fork = nullptr, join = nullptr;
+    cudaStream_t side = nullptr, small = nullptr;
+    cudaEvent_t fork = nullptr, join = nullptr, join_small = nullptr;
     cudaError_t init()
     {
         cudaError_t e = cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking);
+        if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&small, cudaStreamNonBlocking);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&join, cudaEventDisableTiming);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&join_small, cudaEventDisableTiming);
         if (e != cudaSuccess) destroy();
         return e;
     }
     void destroy()
     {
         if (join) cudaEventDestroy(join);
+        if (join_small) cudaEventDestroy(join_small);
         if (fork) cudaEventDestroy(fork);
         if (side) cudaStreamDestroy(side);
-        side = nullptr;
-        fork = join = nullptr;
+        if (small) cudaStreamDestroy(small);
+        side = small = nullptr;
+        fork = join = join_small = nullptr;
     }
-    // launch_a on the side stream and launch_b on s, both after the work
-    // already queued on s; s continues after both
-    template <class A, class B>
-    cudaError_t run(cudaStream_t s, A launch_a, B launch_b) const
+    // launch_c on the small stream (with_c), launch_a on the side stream
+    // (with_a) and launch_b on s, all after the work already queued on s; s
+    // continues after all of them
+    template <class A, class B, class C>
+    cudaError_t run(cudaStream_t s, bool with_c, C launch_c, bool with_a, A launch_a, B launch_b) const
     {
-        cudaError_t e = cudaEventRecord(fork, s);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(side, fork, 0);
-        if (e == cudaSuccess) e = launch_a(side);
-        if (e == cudaSuccess) e = cudaEventRecord(join, side);
+        cudaError_t e = with_a || with_c ? cudaEventRecord(fork, s) : cudaSuccess;
+        auto branch = [&](cudaStream_t st, cudaEvent_t done, auto &launch) {
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(st, fork, 0);
+            if (e == cudaSuccess) e = launch(st);
+            if (e == cudaSuccess) e = cudaEventRecord(done, st);
+        };
+        if (with_c) branch(small, join_small, launch_c);
+        if (with_a) branch(side, join, launch_a);
         if (e == cudaSuccess) e = launch_b(s);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(s, join, 0);
+        if (e == cudaSuccess && with_a) e = cudaStreamWaitEvent(s, join, 0);
+        if (e == cudaSuccess && with_c) e = cudaStreamWaitEvent(s, join_small, 0);
         return e;
     }
 };
@@ -142,8 +156,8 @@ struct fdtd_grid {
     int *order_d = nullptr;               // column tiles in the order a z block hands them out
     std::vector<int> order_pos;           // position of each column tile in that order
     // single-grid steps apply the current sources in the step kernel and read
-    // the probes of step n beside step n + 1 (no Debye media, no oblique
-    // wires, no ideal voltage sources, at most 32 sources)
+    // the probes of step n beside step n + 1 (no Debye media, no ideal voltage
+    // sources, at most 32 sources, none beside oblique wires)
     bool fast = false;
     fdtd::DomainSlot slot_h;              // host copy (also read by batches)
     fdtd::EdgeArgs edge_h[2];             // edge-kernel arguments per input parity
@@ -1032,7 +1046,6 @@ fdtd::EdgeArgs edge_args(const fdtd_grid *g, int parity)
     e.w.Q = g->oQ_d;
     e.w.V = g->oV_d;
     e.w.P = g->oP_d;
-    e.wire_done = g->npoles > 0 && !g->osegs.empty();
     e.w.src = g->osrc_d;
     e.w.samples = g->osamp_d;
     e.step_t = 0;
@@ -1106,9 +1119,10 @@ fdtd::BatchArgs grid_launch(const fdtd_grid *g, int parity, int l, int *work, in
 // One step with the current sources in the step kernel (g->fast): step t of
 // a sequence whose first step is the device counter's value.  The probes of
 // the previous step (t > 0) read that step's output -- this step's input,
-// which nothing writes now -- on the side stream beside the step kernels;
-// the last step of the sequence (last) reads its own probes after its step
-// kernels and advances the counter by t + 1.
+// which nothing writes now -- beside the step kernels, before the oblique
+// wires' gather overwrites the segment currents; the last step of the
+// sequence (last) reads its own probes after its step kernels and advances
+// the counter by t + 1.
 cudaError_t enqueue_step_fast(fdtd_grid *g, int parity, cudaStream_t s, int t, bool last)
 {
     auto launch = [g, parity, t](int l) {
@@ -1117,25 +1131,31 @@ cudaError_t enqueue_step_fast(fdtd_grid *g, int parity, cudaStream_t s, int t, b
                                      grid_launch(g, parity, l, g->lc[l].work, g->err_d), g->lc[l].grid, st);
         };
     };
-    const bool prev = t > 0 && !g->probes.empty();
+    const bool prev = t > 0 && !g->probes.empty(), wires = !g->osegs.empty();
+    auto small = [g, parity, t, prev, wires](cudaStream_t st) {
+        cudaError_t r = cudaSuccess;
+        if (prev) {
+            fdtd::EdgeArgs pa = edge_args(g, parity ^ 1);     // step t - 1's output
+            pa.n_src = 0;
+            pa.skip_src = 1;
+            pa.step_t = t - 1;
+            pa.advance = 0;
+            r = fdtd::launch_edges(pa, st);
+        }
+        if (r == cudaSuccess && wires) {
+            fdtd::EdgeArgs ga = edge_args(g, parity);
+            ga.step_t = t;
+            r = fdtd::launch_wire_gather(ga, st);
+        }
+        return r;
+    };
     cudaError_t e = cudaSuccess;
-    if (g->fk.side && (g->n_launch == 2 || prev)) {
-        auto side = [g, parity, t, prev, &launch](cudaStream_t st) {
-            cudaError_t r = g->n_launch == 2 ? launch(1)(st) : cudaSuccess;
-            if (r == cudaSuccess && prev) {
-                fdtd::EdgeArgs pa = edge_args(g, parity ^ 1);     // step t - 1's output
-                pa.n_src = 0;
-                pa.skip_src = 1;
-                pa.step_t = t - 1;
-                pa.advance = 0;
-                r = fdtd::launch_edges(pa, st);
-            }
-            return r;
-        };
-        e = g->fk.run(s, side, launch(0));
+    if (g->fk.side) {
+        e = g->fk.run(s, prev || wires, small, g->n_launch == 2, launch(1), launch(0));
     } else {
         for (int l = 0; l < g->n_launch && e == cudaSuccess; ++l) e = launch(l)(s);
     }
+    if (e == cudaSuccess && wires) e = fdtd::launch_wire_finish(edge_args(g, parity), s);
     if (e == cudaSuccess && last) {
         fdtd::EdgeArgs pa = edge_args(g, parity);
         pa.n_src = 0;
@@ -1158,21 +1178,16 @@ cudaError_t enqueue_step(fdtd_grid *g, int parity, cudaStream_t s, int t = 0, bo
         };
     };
     const bool wires = !g->osegs.empty();
-    if (g->fk.side && (g->n_launch == 2 || wires)) {
-        // side stream: the oblique wires' gather, then the z-layer launch
-        auto side = [g, parity, wires, &launch](cudaStream_t st) {
-            cudaError_t r = wires ? fdtd::launch_wire_gather(edge_args(g, parity), st) : cudaSuccess;
-            if (r == cudaSuccess && g->n_launch == 2) r = launch(1)(st);
-            return r;
-        };
-        e = g->fk.run(s, side, launch(0));
+    if (g->fk.side) {
+        auto gather = [g, parity](cudaStream_t st) { return fdtd::launch_wire_gather(edge_args(g, parity), st); };
+        e = g->fk.run(s, wires, gather, g->n_launch == 2, launch(1), launch(0));
     } else {
         if (wires) e = fdtd::launch_wire_gather(edge_args(g, parity), s);
         for (int l = 0; l < g->n_launch && e == cudaSuccess; ++l) e = launch(l)(s);
     }
-    // in Debye media the wires' currents reach E^{n+1} before the polarisation
-    // currents advance from it
-    if (e == cudaSuccess && g->npoles && wires) e = fdtd::launch_wire_finish(edge_args(g, parity), s);
+    // the wires' currents reach E^{n+1} before the polarisation currents of
+    // Debye media advance from it
+    if (e == cudaSuccess && wires) e = fdtd::launch_wire_finish(edge_args(g, parity), s);
     if (e == cudaSuccess && g->npoles) e = fdtd::launch_debye(debye_args(g, parity), s);
     if (e != cudaSuccess) return e;
     if (has_edge_work(g)) e = fdtd::launch_edges(edge_args(g, parity), s);
@@ -1487,8 +1502,7 @@ int step_with_scratch(fdtd_grid *g, int n, int *scratch, int scratch_ints)
         for (int l = 0; l < g->n_launch && e == cudaSuccess; ++l)
             e = launch_step(single_args(g, g->parity, l), grid_launch(g, g->parity, l, scratch + 2 * l, g->noalloc_err),
                             g->lc[l].grid, g->stream);
-        if (e == cudaSuccess && g->npoles && !g->osegs.empty())
-            e = launch_wire_finish(edge_args(g, g->parity), g->stream);
+        if (e == cudaSuccess && !g->osegs.empty()) e = launch_wire_finish(edge_args(g, g->parity), g->stream);
         if (e == cudaSuccess && g->npoles) e = launch_debye(debye_args(g, g->parity), g->stream);
         if (e == cudaSuccess && has_edge_work(g))
             e = launch_edges(edge_args(g, g->parity), g->stream);
@@ -2073,7 +2087,9 @@ int fdtd_finalize(fdtd_grid *g, int probe_capacity, void *arena, size_t arena_by
         if (e != cudaSuccess) return cuda_fail(g, e, "upload of the column order");
     }
     // current sources in the step kernel: each source's launch and work item
-    g->fast = g->npoles == 0 && g->osegs.empty() && g->srcs.size() <= 32 && has_edge_work(g);
+    // (with oblique wires, whose currents come before the sources', only
+    // without sources)
+    g->fast = g->npoles == 0 && (g->osegs.empty() || g->srcs.empty()) && g->srcs.size() <= 32 && has_edge_work(g);
     for (const Source &src : g->srcs) g->fast = g->fast && !src.hard;
     if (g->fast && !g->srcs.empty()) {
         using namespace fdtd::geom;
@@ -2430,13 +2446,8 @@ cudaError_t batch_enqueue(fdtd_batch *b, int parity, cudaStream_t s)
         };
     };
     if (b->fk.side) {
-        // side stream: the oblique wires' gather, then the z-layer launch
-        auto side = [b, parity, nd, &launch](cudaStream_t st) {
-            cudaError_t r = b->has_wires ? fdtd::launch_wire_gather_batch(b->edges, nd, parity, st) : cudaSuccess;
-            if (r == cudaSuccess) r = launch(1)(st);
-            return r;
-        };
-        e = b->fk.run(s, side, launch(0));
+        auto gather = [b, parity, nd](cudaStream_t st) { return fdtd::launch_wire_gather_batch(b->edges, nd, parity, st); };
+        e = b->fk.run(s, b->has_wires, gather, b->n_launch == 2 && b->nitems[1] > 0, launch(1), launch(0));
     } else {
         if (b->has_wires) e = fdtd::launch_wire_gather_batch(b->edges, nd, parity, s);
         for (int l = 0; l < b->n_launch && e == cudaSuccess; ++l) e = launch(l)(s);
