@@ -252,18 +252,6 @@ int debye_extent(const fdtd_grid *g, int *z0, int *z1)
     return P;
 }
 
-// a grid whose field arrays hold 2^31 elements or more needs 64-bit indices;
-// FDTD_WIDE_INDEX=1 in the environment selects them for any single grid
-// (the tests compare both instantiations on small grids)
-bool grid_is_wide(const fdtd_grid *g)
-{
-    static const bool forced = [] {
-        const char *v = std::getenv("FDTD_WIDE_INDEX");
-        return v && v[0] == '1';
-    }();
-    return (double)g->plane * g->nz >= 2147483647.0 || forced;
-}
-
 // compact auxiliaries: only their axis's two layers (fdtd_internal.h)
 int psi_px(const fdtd_grid *g) { return (2 * g->d + 3) / 4 * 4; }
 size_t psi_elems(const fdtd_grid *g, int q)
@@ -1112,7 +1100,6 @@ fdtd::BatchArgs grid_launch(const fdtd_grid *g, int parity, int l, int *work, in
     b.max_d = g->d;
     b.region = g->lc[l].region;
     b.nh = g->lc[l].nh;
-    b.wide = grid_is_wide(g);
     return b;
 }
 
@@ -1377,14 +1364,13 @@ int setup_step_kernel(fdtd_grid *g)
         max_smem = std::max(max_smem, fdtd::step_smem_bytes(g->n_classes, d, L.region, L.nh));
         g->n_launch = l + 1;
     }
-    const bool wide = grid_is_wide(g);
     for (int q = 0; q < 4 && e == cudaSuccess; ++q)
-        e = ensure_smem(fdtd::step_kernel_ptr(q >> 1, 2 + (q & 1), false, wide), max_smem);
+        e = ensure_smem(fdtd::step_kernel_ptr(q >> 1, 2 + (q & 1), false), max_smem);
     if (e != cudaSuccess) return cuda_fail(g, e, "step kernel setup");
     int occ[2] = {1, 1};
     for (int l = 0; l < g->n_launch; ++l) {
         auto &L = g->lc[l];
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[l], fdtd::step_kernel_ptr(l, L.nh, false, wide),
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[l], fdtd::step_kernel_ptr(l, L.nh, false),
                                                           fdtd::step_threads(),
                                                           fdtd::step_smem_bytes(g->n_classes, d, L.region, L.nh));
         if (e != cudaSuccess) return cuda_fail(g, e, "step kernel occupancy");
@@ -2548,11 +2534,11 @@ int fdtd_batch_create(int n, fdtd_grid *const *grids, void *cuda_stream, fdtd_ba
         max_smem = std::max(max_smem, fdtd::step_smem_bytes(b->max_classes, b->max_d, b->region[l], b->nh[l]));
     }
     for (int q = 0; q < 4 && e == cudaSuccess; ++q)
-        e = ensure_smem(fdtd::step_kernel_ptr(q >> 1, 2 + (q & 1), true, false), max_smem);
+        e = ensure_smem(fdtd::step_kernel_ptr(q >> 1, 2 + (q & 1), true), max_smem);
     int occ[2] = {1, 1};
     for (int l = 0; l < b->n_launch && e == cudaSuccess; ++l) {
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &occ[l], fdtd::step_kernel_ptr(l, b->nh[l], true, false), fdtd::step_threads(),
+            &occ[l], fdtd::step_kernel_ptr(l, b->nh[l], true), fdtd::step_threads(),
             fdtd::step_smem_bytes(b->max_classes, b->max_d, b->region[l], b->nh[l]));
         if (e == cudaSuccess && occ[l] < 1) { delete b; return FDTD_ECUDA; }
     }

@@ -28,14 +28,20 @@
 //     none runs without any CPML code, the others without a branch per cell.
 // What bounds it: DRAM on grids that fill the chip, otherwise the latency of
 // a plane's chain (copies landed, H, barrier, E), which a CTA cannot
-// overlap with more than the ring holds.  Hence few and wide instructions
-// per plane, registers split by role (setmaxnreg), and few copies issued by
-// a converged warp.  With four cells per lane (16-byte accesses) the plane
-// loop has fewer instructions but half the warps to hide its latency, and
-// measured slower.  Measured (us per step, one cell per lane and fifteen
-// copies a plane before): 256^3 PEC 136.3 -> 130.1 (0.93 of the measured copy
-// bandwidth), 256^3 with a 10-cell CPML 175.9 -> 164.6, 512x512x384 with 12
-// cells 956 -> 908, 128^3 with 8 cells 42.7 -> 38.4.
+// overlap with more than the ring holds: 1300 cycles alone on an SM without a
+// layer, 2000 with one.  Hence few and wide instructions per plane, values
+// the same for a warp in uniform registers (item by shuffle, one base
+// pointer per array and plane, one 32-bit offset per lane), no choice inside
+// the plane loop, registers split by role (setmaxnreg) so that nothing
+// spills, and few copies issued by a converged warp.  With four cells per
+// lane (16-byte accesses) the plane loop has fewer instructions but half the
+// warps to hide its latency, and measured slower (197 us on the 256^3 CPML
+// grid at the same stage as 171); running 64-bit pointers per lane in place
+// of offsets took 11 % more instructions (256^3 PEC 134 us).  Measured (us
+// per step; one cell per lane, fifteen copies a plane and 16 planes per item
+// before): 256^3 PEC 136.3 -> 129.8, 256^3 with a 10-cell CPML 175.9 ->
+// 162.8, 512x512x384 with 12 cells 956 -> 909, 128^3 with 8 cells 42.7 ->
+// 33.6, 64^3 with 8 cells 25.6 -> 10.4.
 // DRAM traffic per cell and step: 6 FP32 reads + 6 writes + 1 class byte
 // (49 B) plus the CPML auxiliaries in the layer; every halo read is an L2
 // hit.  Every wait is bounded; on a timeout the kernel records an error
@@ -61,11 +67,17 @@ constexpr int NHW = 2;                 // halo warps: low-y row, low-x column
 constexpr int NCONS = (NCW + NHW) * 32;  // row warps + halo warps
 constexpr int NTHREADS = (NCW + 4) * 32;   // + the producer warp, one warp idle: whole warpgroups
 // registers: the row warps (the first warpgroups) hold their cells' state and
-// take ROW_REGS each, the halo warps and the producer AUX_REGS; together
+// take row_regs each, the halo warps and the producer aux_regs; together
 // what the block is launched with (two blocks per SM)
-constexpr int ROW_REGS = 96, AUX_REGS = 48, LAUNCH_REGS = 80;
+// (the split that leaves no spills: a batch's row warps read their arguments
+// from shared memory and need fewer, its producer more)
+constexpr int LAUNCH_REGS = 80;
+constexpr int row_regs(bool batch) { return batch ? 88 : 96; }
+constexpr int aux_regs(bool batch) { return batch ? 64 : 48; }
 static_assert(NCW % 4 == 0, "row warps fill warpgroups");
-static_assert(NCW * ROW_REGS + 4 * AUX_REGS <= (NCW + 4) * LAUNCH_REGS, "the shares of the launch's registers");
+static_assert(NCW * row_regs(false) + 4 * aux_regs(false) <= (NCW + 4) * LAUNCH_REGS &&
+              NCW * row_regs(true) + 4 * aux_regs(true) <= (NCW + 4) * LAUNCH_REGS,
+              "the shares of the launch's registers");
 constexpr int NE = 4;                  // E-plane ring: planes k, k+1 in use, two ahead
 constexpr int NH_MAX = 3;              // H / class / CPML ring: plane k in use, up to two ahead
                                        // (a launch whose auxiliary region is large uses 2)
@@ -125,9 +137,9 @@ constexpr int HNEW_PLANE = HBY * HBX;
 constexpr int HNEW_BYTES = 2 * 3 * HNEW_PLANE * 4;     // [2][3][HBY][HBX]
 constexpr int NBAR = 2 * NE + 2 * NH_MAX;             // fullE, emptyE, fullH, emptyH
 // x-layer coefficients of the current item's columns: {b, c, 1/kappa} at E,
-// then at H positions, TX floats each (identity outside the layer), and an
-// identity profile row
-constexpr int XC_BYTES = 6 * TX * 4 + 16;
+// then at H positions, TX floats each (identity outside the layer), an
+// identity profile row and three zero coefficient rows
+constexpr int XC_BYTES = (6 * TX + 4 + 12) * 4;
 struct Layout {
     int hslot, hnew, xc, bar, misc, tab;
     __host__ __device__ Layout(int region, int nh)
@@ -282,10 +294,6 @@ __device__ __forceinline__ int psi_y(const StepArgs &a, int i, int sy, int k)
 {
     return (k * (2 * a.d) + sy) * a.pitch + i;
 }
-__device__ __forceinline__ int psi_z(const StepArgs &a, int i, int j, int sz)
-{
-    return (sz * a.ny + j) * a.pitch + i;
-}
 // elements of the compact x, y, z arrays (extents for the bounds-checked build)
 __device__ __forceinline__ long long psi_n(const StepArgs &a, int u)
 {
@@ -368,32 +376,30 @@ __device__ __forceinline__ F2 sub2(F2 a, F2 b) { return fma2(b, pk(-1.f, -1.f), 
 // pair), of this one and the one before (w)
 __device__ __forceinline__ F2 next_diff(F2 x, float e) { return pk(hi2(x) - lo2(x), e - hi2(x)); }
 __device__ __forceinline__ F2 prev_diff(F2 x, float w) { return pk(lo2(x) - w, hi2(x) - lo2(x)); }
-// the cells m (bit c: cell c) of a pair at element g of base to global
-// memory.  all: both or none (every tile that lies wholly in the grid; the
-// same for the whole warp)
-template <typename Idx>
-__device__ __forceinline__ void put2(float *base, Idx g, F2 x, int m, bool all, long long n, int site, int *bounds)
+// a pair into a plane of an array (element `plane` on; the same for the
+// whole warp) at the lane's element off of the plane, if `on`.  The second
+// cell of a side of odd length falls into the row's padding (rows are padded
+// to 16 elements), where it is zero for a field (its coefficients are) and
+// never read.  n: the array's elements, for the bounds-checked build
+template <typename Off>
+__device__ __forceinline__ void put2(float *base, long long plane, Off off, F2 x, bool on, long long n, int site,
+                                     int *bounds)
 {
-    if (all) {
-        if (m && in_bounds(g, n, site, bounds) && in_bounds(g + 1, n, site, bounds)) st2(base + g, x);
-    } else {
-        if ((m & 1) && in_bounds(g, n, site, bounds)) base[g] = lo2(x);
-        if ((m & 2) && in_bounds(g + 1, n, site, bounds)) base[g + 1] = hi2(x);
-    }
+    float *p = base + plane;
+    if (on && in_bounds(plane + off, n, site, bounds) && in_bounds(plane + off + 1, n, site, bounds)) st2(p + off, x);
 }
 
 // what a lane's pair of cells is to the layers of its item, formed once per item
+enum { IN0 = 1, IN1 = 2, XM0 = 4, XM1 = 8, XM = 12, YM = 16 };
 struct Pair {
-    int i, j;                // first cell
-    int m;                   // bit c: cell c lies inside the grid
-    bool all;                // every cell of the tile does (uniform)
-    int xm;                  // bit c: cell c lies in an x layer
-    int xe;                  // slab entry of the first cell (of the layer the members lie in)
-    int xo;                  // float offset of that entry in the first x box
-    int sy;                  // slab row or -1
+    int fl;                  // IN0, IN1: the first, second cell lies inside the grid; XM0, XM1: in an x layer;
+                             // YM: the row lies in a y layer
+    int xo;                  // float offset of the first cell's entry in the first x box
     int yo;                  // float offset of the pair in the first y box (of the lane's column, outside the layer)
     const float4 *py;        // its y profile row at E positions (the identity outside the layer)
     int ph;                  // rows from there to the one at H positions
+    unsigned off;            // its element in a plane of the fields and z auxiliaries
+    int xoff, yoff;          // of the x, y auxiliaries (a lane outside the layer: not used)
 };
 
 // one plane's auxiliaries for a pair
@@ -418,71 +424,94 @@ __device__ __forceinline__ F2 cpmlx(F2 &dif, const PX &q, F2 o)
     return p;
 }
 
-// The x layer.  VEC: every pair lies wholly in a layer or outside and its
-// entries start on an 8-byte boundary (d and nx - 2 d even).  A pair never
-// has members in both layers (they are two cells apart at least).  Cells
-// outside the layer read 0.
-__device__ __forceinline__ F2 x_psi(const Pair &G, const float *box, bool vec)
+// Both differences of the x layer at E (h = 0) or H (h = 1) positions.  VEC:
+// every pair lies wholly in a layer or outside and its entries start on an
+// 8-byte boundary (d and nx even); otherwise cell by cell (a choice made
+// inside the plane loop costs more than the layer's arithmetic).  A pair
+// never has members in both layers (they are two cells apart at least).
+// Cells outside the layer read 0.
+template <bool VEC>
+__device__ __forceinline__ void cpml_x(const StepArgs &a, const Pair &G, const PlaneX &P, int h, int k, F2 &d0, F2 &d1)
 {
-    F2 o = 0;
-    if (vec) {
-        if (G.xm) o = ld2(box + G.xo);
-    } else {
-        float a = 0.f, b = 0.f;
-        if (G.xm & 1) a = box[G.xo];
-        if (G.xm & 2) b = box[G.xo + 1];
-        o = pk(a, b);
-    }
-    return o;
-}
-// both differences of the x layer at E (h = 0) or H (h = 1) positions
-__device__ __forceinline__ void cpml_x(const StepArgs &a, const Pair &G, const PlaneX &P, int h, bool vec, int k,
-                                       F2 &d0, F2 &d1)
-{
-    const int q = a.pg.xb >> 2, g = psi_x(a, G.xe, G.j, k), at = h ? PSI_HY_X : PSI_EY_X;
-    const float *b = P.base + (h ? 0 : 2 * q);
+    const int q = a.pg.xb >> 2, at = h ? 0 : 2;
+    const float *b = P.base + at * q + G.xo;
     const PX pr = profx(P.xc + (h ? 3 * TX : 0));
-    const F2 p0 = cpmlx(d0, pr, x_psi(G, b, vec)), p1 = cpmlx(d1, pr, x_psi(G, b + q, vec));
-    put2(a.psi_out[at], g, p0, G.xm, vec, psi_n(a, 0), 3, a.bounds);
-    put2(a.psi_out[at + 1], g, p1, G.xm, vec, psi_n(a, 0), 3, a.bounds);
+    F2 o0 = 0, o1 = 0;
+    if (VEC) {
+        if (G.fl & XM) {
+            o0 = ld2(b);
+            o1 = ld2(b + q);
+        }
+    } else {
+        float f[4] = {0.f, 0.f, 0.f, 0.f};
+        if (G.fl & XM0) {
+            f[0] = b[0];
+            f[1] = b[q];
+        }
+        if (G.fl & XM1) {
+            f[2] = b[1];
+            f[3] = b[q + 1];
+        }
+        o0 = pk(f[0], f[2]);
+        o1 = pk(f[1], f[3]);
+    }
+    const F2 p0 = cpmlx(d0, pr, o0), p1 = cpmlx(d1, pr, o1);
+    const int pl = k * (a.ny * a.px);
+    float *u0 = a.psi_out[h ? PSI_HY_X : PSI_EY_X], *u1 = a.psi_out[h ? PSI_HZ_X : PSI_EZ_X];
+    const long long n = psi_n(a, 0);
+    if (VEC) {
+        put2(u0, pl, G.xoff, p0, G.fl & XM, n, 3, a.bounds);
+        put2(u1, pl, G.xoff, p1, G.fl & XM, n, 3, a.bounds);
+    } else {
+        u0 += pl;
+        u1 += pl;
+        if ((G.fl & XM0) && in_bounds(pl + G.xoff, n, 3, a.bounds)) {
+            u0[G.xoff] = lo2(p0);
+            u1[G.xoff] = lo2(p1);
+        }
+        if ((G.fl & XM1) && in_bounds(pl + G.xoff + 1, n, 3, a.bounds)) {
+            u0[G.xoff + 1] = hi2(p0);
+            u1[G.xoff + 1] = hi2(p1);
+        }
+    }
 }
 // of the y layer
 __device__ __forceinline__ void cpml_y(const StepArgs &a, const Pair &G, const PlaneX &P, int h, int k, F2 &d0, F2 &d1)
 {
-    const int q = a.pg.yb >> 2, g = psi_y(a, G.i, G.sy, k), at = h ? PSI_HX_Y : PSI_EX_Y;
-    const float *b = P.base + G.yo + (h ? 0 : 2 * q);
+    const int q = a.pg.yb >> 2, at = h ? 0 : 2;
+    const float *b = P.base + G.yo + at * q;
     const PX pr = profx(G.py[h ? G.ph : 0]);
     const F2 p0 = cpmlx(d0, pr, ld2(b)), p1 = cpmlx(d1, pr, ld2(b + q));
-    const int m = G.sy >= 0 ? G.m : 0;
-    put2(a.psi_out[at], g, p0, m, G.all, psi_n(a, 1), 3, a.bounds);
-    put2(a.psi_out[at + 1], g, p1, m, G.all, psi_n(a, 1), 3, a.bounds);
+    const int pl = k * (2 * a.d * a.pitch);
+    put2(a.psi_out[h ? PSI_HX_Y : PSI_EX_Y], pl, G.yoff, p0, G.fl & YM, psi_n(a, 1), 3, a.bounds);
+    put2(a.psi_out[h ? PSI_HZ_Y : PSI_EZ_Y], pl, G.yoff, p1, G.fl & YM, psi_n(a, 1), 3, a.bounds);
 }
 // of the z layer
 __device__ __forceinline__ void cpml_z(const StepArgs &a, const Pair &G, const PlaneX &P, const float *prof, int h,
                                        F2 &d0, F2 &d1)
 {
-    const int g = psi_z(a, G.i, G.j, P.sz), at = h ? PSI_HX_Z : PSI_EX_Z;
     const float *b = P.base + (h ? P.zo : P.zeo);
     const PX pr = profx(prow(prof, 2, h, 2 * a.d)[P.sz]);
     const F2 p0 = cpmlx(d0, pr, ld2(b)), p1 = cpmlx(d1, pr, ld2(b + (h ? H_COMP : PE_BYTES) / 4));
-    put2(a.psi_out[at], g, p0, G.m, G.all, psi_n(a, 2), 3, a.bounds);
-    put2(a.psi_out[at + 1], g, p1, G.m, G.all, psi_n(a, 2), 3, a.bounds);
+    const int pl = P.sz * (a.ny * a.pitch);
+    put2(a.psi_out[h ? PSI_HX_Z : PSI_EX_Z], pl, G.off, p0, G.fl & IN0, psi_n(a, 2), 3, a.bounds);
+    put2(a.psi_out[h ? PSI_HY_Z : PSI_EY_Z], pl, G.off, p1, G.fl & IN0, psi_n(a, 2), 3, a.bounds);
 }
 
 // layers met by the cells an item updates (template bits)
-constexpr int LX = 1, LY = 2, LZ = 4;
+constexpr int LX = 1, LY = 2, LZ = 4, LXS = 8;     // LX, LXS: the x layer in whole pairs, cell by cell
 
 // H^{n+1/2} of a pair (h_core) from H^{n-1/2} in place; t0, t1: its cells'
 // coefficient rows.
 template <int L>
 __device__ __forceinline__ void h_corex(const StepArgs &a, const Pair &G, const PlaneX &P, const float *prof, int k,
-                                        bool vec, F2 ex, F2 ey, F2 ez, F2 ex_y1, F2 ez_y1, float ey_e, float ez_e,
+                                        F2 ex, F2 ey, F2 ez, F2 ex_y1, F2 ez_y1, float ey_e, float ez_e,
                                         F2 ex_z1, F2 ey_z1, const float4 *t0, const float4 *t1, F2 &hx, F2 &hy, F2 &hz)
 {
     F2 hx_z = sub2(ey_z1, ey), hx_y = sub2(ez_y1, ez);
     F2 hy_x = next_diff(ez, ez_e), hy_z = sub2(ex_z1, ex);
     F2 hz_y = sub2(ex_y1, ex), hz_x = next_diff(ey, ey_e);
-    if constexpr (L & LX) cpml_x(a, G, P, 1, vec, k, hy_x, hz_x);
+    if constexpr (L & (LX | LXS)) cpml_x<(L & LX) != 0>(a, G, P, 1, k, hy_x, hz_x);
     if constexpr (L & LY) cpml_y(a, G, P, 1, k, hx_y, hz_y);
     if constexpr (L & LZ) cpml_z(a, G, P, prof, 1, hx_z, hy_z);
     const F2 dx = sub2(hx_z, hx_y), dy = sub2(hy_x, hy_z), dz = sub2(hz_y, hz_x);
@@ -494,9 +523,9 @@ __device__ __forceinline__ void h_corex(const StepArgs &a, const Pair &G, const 
 
 // Hx and Hy^{n+1/2} of a pair of the plane below an item, which the item
 // reads but does not update, in place; x / y auxiliaries that are not staged
-// there (flags f) come from global memory.
+// there (flags f) come from global memory, elements gx, gy.
 __device__ __forceinline__ void h_belowx(const StepArgs &a, const Pair &G, const PlaneX &P, const float *prof, int f,
-                                         int k, F2 ex, F2 ey, F2 ez, F2 ez_y1, float ez_e, F2 ex_z1, F2 ey_z1,
+                                         int gx, int gy, F2 ex, F2 ey, F2 ez, F2 ez_y1, float ez_e, F2 ex_z1, F2 ey_z1,
                                          const float4 *t0, const float4 *t1, F2 &hx, F2 &hy)
 {
     F2 hx_z = sub2(ey_z1, ey), hx_y = sub2(ez_y1, ez);
@@ -507,12 +536,14 @@ __device__ __forceinline__ void h_belowx(const StepArgs &a, const Pair &G, const
         if ((m & 2) && in_bounds(g + 1, psi_n(a, u), 4, a.bounds)) o1 = __ldg(arr + g + 1);
         return pk(o0, o1);
     };
-    if (G.xm)
-        cpmlx(hy_x, profx(P.xc + 3 * TX), (f & F_X) ? x_psi(G, P.base, false)
-                                                    : far(a.psi_in[PSI_HY_X], psi_x(a, G.xe, G.j, k), G.xm, 0));
-    if (G.sy >= 0)
-        cpmlx(hx_y, profx(G.py[G.ph]), (f & F_Y) ? ld2(P.base + G.yo)
-                                                    : far(a.psi_in[PSI_HX_Y], psi_y(a, G.i, G.sy, k), G.m, 1));
+    if (G.fl & XM) {
+        F2 o;
+        if (f & F_X) o = pk(G.fl & XM0 ? P.base[G.xo] : 0.f, G.fl & XM1 ? P.base[G.xo + 1] : 0.f);
+        else o = far(a.psi_in[PSI_HY_X], gx, (G.fl & XM) / XM0, 0);
+        cpmlx(hy_x, profx(P.xc + 3 * TX), o);
+    }
+    if (G.fl & YM)
+        cpmlx(hx_y, profx(G.py[G.ph]), (f & F_Y) ? ld2(P.base + G.yo) : far(a.psi_in[PSI_HX_Y], gy, G.fl & 3, 1));
     if (P.sz >= 0) {
         const PX q = profx(prow(prof, 2, 1, 2 * a.d)[P.sz]);
         cpmlx(hx_z, q, ld2(P.base + P.zo));
@@ -529,13 +560,13 @@ __device__ __forceinline__ void h_belowx(const StepArgs &a, const Pair &G, const
 // the pair along x.
 template <int L>
 __device__ __forceinline__ void e_corex(const StepArgs &a, const Pair &G, const PlaneX &P, const float *prof, int k,
-                                        bool vec, F2 hx, F2 hy, F2 hz, F2 hz_ym, F2 hx_ym, float hz_w, float hy_w,
+                                        F2 hx, F2 hy, F2 hz, F2 hz_ym, F2 hx_ym, float hz_w, float hy_w,
                                         F2 hx_zm, F2 hy_zm, const float4 *t0, const float4 *t1, F2 &ex, F2 &ey, F2 &ez)
 {
     F2 ex_y = sub2(hz, hz_ym), ex_z = sub2(hy, hy_zm);
     F2 ey_z = sub2(hx, hx_zm), ey_x = prev_diff(hz, hz_w);
     F2 ez_x = prev_diff(hy, hy_w), ez_y = sub2(hx, hx_ym);
-    if constexpr (L & LX) cpml_x(a, G, P, 0, vec, k, ey_x, ez_x);
+    if constexpr (L & (LX | LXS)) cpml_x<(L & LX) != 0>(a, G, P, 0, k, ey_x, ez_x);
     if constexpr (L & LY) cpml_y(a, G, P, 0, k, ex_y, ez_y);
     if constexpr (L & LZ) cpml_z(a, G, P, prof, 0, ex_z, ey_z);
     const F2 dx = sub2(ex_y, ex_z), dy = sub2(ey_z, ey_x), dz = sub2(ez_x, ez_y);
@@ -674,6 +705,14 @@ __device__ __forceinline__ Item decode(const StepArgs &a, int item)
     return it;
 }
 
+// the same item with its values in uniform registers
+__device__ __forceinline__ Item uniform(const Item &it)
+{
+    const unsigned all = 0xffffffffu;
+    return Item{__shfl_sync(all, it.x0, 0), __shfl_sync(all, it.y0, 0), __shfl_sync(all, it.ka, 0),
+                __shfl_sync(all, it.kb, 0)};
+}
+
 // does any cell the item updates or recomputes lie in a CPML layer
 __device__ __forceinline__ bool item_in_cpml(const StepArgs &a, const Item &it)
 {
@@ -742,61 +781,53 @@ struct Cons {
     }
 };
 
-// a lane's pairs of three field components to global memory at element g
-template <typename Idx>
-__device__ __forceinline__ void put_fields(float *const *out, Idx g, F2 x, F2 y, F2 z, const Pair &G, long long n,
-                                           int site, int *bounds)
-{
-    put2(out[0], g, x, G.m, G.all, n, site, bounds);
-    put2(out[1], g, y, G.m, G.all, n, site, bounds);
-    put2(out[2], g, z, G.m, G.all, n, site, bounds);
-}
-
 // One work item in a row warp.  R is at the item's first plane, ka-1, on
 // entry and at the next item's on return.  A wait that gives up sets *abort;
 // the warp then goes through the item's remaining barriers without touching
 // the slots, so no other warp is left waiting, and the CTA leaves at the
 // item's end.
-// WIDE: 64-bit element indices for the field stores (grids of 2^31
-// elements or more); 32-bit otherwise, fewer registers in the plane loop
 // L: the layers the item's own cells meet
-template <int L, int NH, bool WIDE>
+template <int L, int NH>
 __device__ __forceinline__ void run_rows(const Cons<NH> &C, const Item &it, Ring<NH> &R, uint32_t &hb)
 {
-    using Idx = typename std::conditional<WIDE, long long, int>::type;
     const StepArgs &a = *C.a;
     const int lane = C.lane, d = a.d;
     // the lane's pair of cells
     const int row = 1 + C.warp + (lane / LPR) * NCW, gx = GX * (lane % LPR);
     const int lx = XO + gx, clx = CXO + gx;
-    const bool vec = ((d | a.nx) & 1) == 0;
+    const int i = it.x0 + gx, j = it.y0 + row - 1;
+    const int nv = j < a.ny ? max(0, min(GX, a.nx - i)) : 0;
     Pair G;
-    G.i = it.x0 + gx;
-    G.j = it.y0 + row - 1;
-    const int nv = G.j < a.ny ? max(0, min(GX, a.nx - G.i)) : 0;
-    G.m = (1 << nv) - 1;
-    G.all = it.x0 + TX <= a.nx && it.y0 + TY <= a.ny;
-    G.xm = G.xe = G.xo = 0;
-    G.sy = -1;
+    G.fl = (1 << nv) - 1;
+    G.xo = 0;
     G.yo = 0;
     G.py = reinterpret_cast<const float4 *>(C.xc + 6 * TX);      // the identity
     G.ph = 0;
+    // slab entry of the pair's first cell, in the layer its members lie in, and of its row
+    const int xe = i < d ? i : i - (a.nx - 2 * d), sy = d > 0 && nv > 0 ? slab_of(j, a.ny, d) : -1;
     if (d > 0) {
         Stg tb(0, 0, 0);                // the tile's x / y layer boxes
         tb.f = tile_boxes(a, it.x0, it.y0, tb.xs, tb.ys);
 #pragma unroll
         for (int c = 0; c < GX; ++c)
-            if (c < nv && slab_of(G.i + c, a.nx, d) >= 0) G.xm |= 1 << c;
-        G.xe = G.i < d ? G.i : G.i - (a.nx - 2 * d);
-        G.xo = a.ox / 4 + row * a.pg.w + G.xe - tb.xs;
-        if (nv > 0) G.sy = slab_of(G.j, a.ny, d);
-        G.yo = a.oy / 4 + (G.sy >= 0 ? G.sy - tb.ys : 0) * HBX + lx;
-        if (G.sy >= 0) {
-            G.py = prow(C.prof, 1, 0, 2 * d) + G.sy;
+            if (c < nv && slab_of(i + c, a.nx, d) >= 0) G.fl |= XM0 << c;
+        G.xo = a.ox / 4 + row * a.pg.w + xe - tb.xs;
+        G.yo = a.oy / 4 + (sy >= 0 ? sy - tb.ys : 0) * HBX + lx;
+        if (sy >= 0) {
+            G.fl |= YM;
+            G.py = prow(C.prof, 1, 0, 2 * d) + sy;
             G.ph = 2 * d;
         }
     }
-    auto row_of = [&](uint32_t cls) { return reinterpret_cast<const float4 *>(C.tab + (cls & 255u) * kTabStride); };
+    G.off = (unsigned)j * a.pitch + i;
+    G.xoff = j * a.px + xe;
+    G.yoff = sy * a.pitch + i;
+    // coefficient rows of the pair's cells (a second cell outside the grid: zeros)
+    const float4 *const zero = reinterpret_cast<const float4 *>(C.xc + 6 * TX + 4);
+    auto row0 = [&](uint32_t cls) { return reinterpret_cast<const float4 *>(C.tab + (cls & 255u) * kTabStride); };
+    auto row1 = [&](uint32_t cls) {
+        return (G.fl & 3) == IN0 ? zero : reinterpret_cast<const float4 *>(C.tab + (cls >> 8) * kTabStride);
+    };
     bool ok = __all_sync(0xffffffffu, mbar_wait(C.fullH(R.h), R.hp, C.abort));
     if (!ok) *C.abort = 1;
     // Hx, Hy of the plane below, kept where that plane's would be: the lane's
@@ -811,9 +842,9 @@ __device__ __forceinline__ void run_rows(const Cons<NH> &C, const Item &it, Ring
         const uint32_t cls = h0.cls2(row, clx);
         hx = ld2(h0.at(0, row, lx));
         hy = ld2(h0.at(1, row, lx));
-        h_belowx(a, G, P, C.prof, Stg(e0.hdr()).f, k, ld2(e0.at(0, row, lx)), ld2(e0.at(1, row, lx)),
+        h_belowx(a, G, P, C.prof, Stg(e0.hdr()).f, psi_x(a, xe, j, k), psi_y(a, i, sy, k), ld2(e0.at(0, row, lx)), ld2(e0.at(1, row, lx)),
                  ld2(e0.at(2, row, lx)), ld2(e0.at(2, row + 1, lx)), e0.e(2, row, lx + GX), ld2(e1.at(0, row, lx)),
-                 ld2(e1.at(1, row, lx)), row_of(cls), row_of(cls >> 8), hx, hy);
+                 ld2(e1.at(1, row, lx)), row0(cls), row1(cls), hx, hy);
     }
     st2(own + (hb ^ 1) * (3 * HNEW_PLANE), hx);
     st2(own + (hb ^ 1) * (3 * HNEW_PLANE) + HNEW_PLANE, hy);
@@ -821,16 +852,15 @@ __device__ __forceinline__ void run_rows(const Cons<NH> &C, const Item &it, Ring
     C.arrive(C.emptyH(R.h));
     R.pass_e();
     R.pass_h();
-    Idx g = (Idx)it.ka * (Idx)a.plane + (Idx)G.j * a.pitch + G.i;
-    const long long n = (long long)a.plane * a.nz;
 #pragma unroll 1
-    for (int k = it.ka; k < it.kb; ++k, g += (Idx)a.plane) {
+    for (int k = it.ka; k < it.kb; ++k) {
         ok = ok && C.wait_plane(R);
         if (!ok) *C.abort = 1;
         const EView ek = C.ev(R.e), ek1 = C.ev(R.e_next());
         const HView hk = C.hv(R.h);
         const PlaneX P{hk.psi(), (L & LZ) ? slab_of(k, a.nz, d) : -1, row * HBX + lx,
                        OFF_ZE / 4 + (row - 1) * TX + gx, C.xc + gx};
+        const long long pl = k * a.plane, n = a.plane * a.nz;
         float *const cur = own + hb * (3 * HNEW_PLANE), *const old = own + (hb ^ 1) * (3 * HNEW_PLANE);
         F2 ex, ey, ez;
         uint32_t cls = 0;
@@ -842,9 +872,9 @@ __device__ __forceinline__ void run_rows(const Cons<NH> &C, const Item &it, Ring
             hx = ld2(hk.at(0, row, lx));
             hy = ld2(hk.at(1, row, lx));
             hz = ld2(hk.at(2, row, lx));
-            h_corex<L>(a, G, P, C.prof, k, vec, ex, ey, ez, ld2(ek.at(0, row + 1, lx)), ld2(ek.at(2, row + 1, lx)),
+            h_corex<L>(a, G, P, C.prof, k, ex, ey, ez, ld2(ek.at(0, row + 1, lx)), ld2(ek.at(2, row + 1, lx)),
                        ek.e(1, row, lx + GX), ek.e(2, row, lx + GX), ld2(ek1.at(0, row, lx)),
-                       ld2(ek1.at(1, row, lx)), row_of(cls), row_of(cls >> 8), hx, hy, hz);
+                       ld2(ek1.at(1, row, lx)), row0(cls), row1(cls), hx, hy, hz);
             st2(cur, hx);
             st2(cur + HNEW_PLANE, hy);
             st2(cur + 2 * HNEW_PLANE, hz);
@@ -852,11 +882,15 @@ __device__ __forceinline__ void run_rows(const Cons<NH> &C, const Item &it, Ring
         consumer_sync();            // H^{n+1/2} of plane k complete (tile + halo)
         C.arrive(C.emptyE(R.e));    // E(k) is not read again
         if (ok) {
-            put_fields(a.Hout, g, hx, hy, hz, G, n, 1, a.bounds);
-            e_corex<L>(a, G, P, C.prof, k, vec, hx, hy, hz, ld2(cur + 2 * HNEW_PLANE - HBX), ld2(cur - HBX),
-                       cur[2 * HNEW_PLANE - 1], cur[HNEW_PLANE - 1], ld2(old), ld2(old + HNEW_PLANE), row_of(cls),
-                       row_of(cls >> 8), ex, ey, ez);
-            put_fields(a.Eout, g, ex, ey, ez, G, n, 2, a.bounds);
+            put2(a.Hout[0], pl, G.off, hx, G.fl & IN0, n, 1, a.bounds);
+            put2(a.Hout[1], pl, G.off, hy, G.fl & IN0, n, 1, a.bounds);
+            put2(a.Hout[2], pl, G.off, hz, G.fl & IN0, n, 1, a.bounds);
+            e_corex<L>(a, G, P, C.prof, k, hx, hy, hz, ld2(cur + 2 * HNEW_PLANE - HBX), ld2(cur - HBX),
+                       cur[2 * HNEW_PLANE - 1], cur[HNEW_PLANE - 1], ld2(old), ld2(old + HNEW_PLANE), row0(cls),
+                       row1(cls), ex, ey, ez);
+            put2(a.Eout[0], pl, G.off, ex, G.fl & IN0, n, 2, a.bounds);
+            put2(a.Eout[1], pl, G.off, ey, G.fl & IN0, n, 2, a.bounds);
+            put2(a.Eout[2], pl, G.off, ez, G.fl & IN0, n, 2, a.bounds);
         }
         C.arrive(C.emptyH(R.h));    // this warp is done with plane k's H slot
         R.pass_e();
@@ -926,10 +960,9 @@ __device__ __forceinline__ void run_halo(const Cons<NH> &C, const Item &it, Ring
 }
 
 // the x-layer coefficients of an item's columns (identity outside the layer
-// and the grid), one value per consumer thread, and the identity profile row
+// and the grid), one value per consumer thread
 __device__ __forceinline__ void fill_xc(const StepArgs &a, const float *prof, float *xc, int x0, int tid)
 {
-    if (tid < 4) xc[6 * TX + tid] = tid == 2 ? 1.f : 0.f;
     for (int q = tid; q < 6 * TX; q += NCONS) {
         const int w = q / TX, i = x0 + q - w * TX, half = w / 3, comp = w - 3 * half;
         const int s = i < a.nx ? slab_of(i, a.nx, a.d) : -1;
@@ -950,7 +983,7 @@ __device__ __forceinline__ int find_domain(const int *item_start, int n, int q)
 }
 
 // the items of a consumer warp, in the order the producer hands them out
-template <bool ROWS, bool ZL, int NH, bool BATCH, bool WIDE>
+template <bool ROWS, bool ZL, int NH, bool BATCH>
 __device__ __forceinline__ void consume(const Cons<NH> &C, const BatchArgs &B, StepArgs *sa, int *cons_e, int *cons_h)
 {
     Ring<NH> R;
@@ -981,7 +1014,7 @@ __device__ __forceinline__ void consume(const Cons<NH> &C, const BatchArgs &B, S
             consumer_sync();
         }
         const StepArgs &a = *C.a;
-        const Item it = decode(a, item);
+        const Item it = uniform(decode(a, item));
         const bool layer = item_in_cpml(a, it);
         if (layer) fill_xc(a, C.prof, C.xc, it.x0, tid);
         const uint32_t n = R.e_next();
@@ -994,10 +1027,18 @@ __device__ __forceinline__ void consume(const Cons<NH> &C, const BatchArgs &B, S
             const bool lx = d > 0 && (it.x0 < d || min(it.x0 + TX, a.nx) > a.nx - d);
             const bool ly = d > 0 && (it.y0 < d || min(it.y0 + TY, a.ny) > a.ny - d);
             constexpr int Z = ZL ? LZ : 0;
-            if (lx && ly) run_rows<LX | LY | Z, NH, WIDE>(C, it, R, hb);
-            else if (lx) run_rows<LX | Z, NH, WIDE>(C, it, R, hb);
-            else if (ly) run_rows<LY | Z, NH, WIDE>(C, it, R, hb);
-            else run_rows<Z, NH, WIDE>(C, it, R, hb);
+            const bool vec = ((d | a.nx) & 1) == 0;
+            if (lx && ly) {
+                if (vec) run_rows<LX | LY | Z, NH>(C, it, R, hb);
+                else run_rows<LXS | LY | Z, NH>(C, it, R, hb);
+            } else if (lx) {
+                if (vec) run_rows<LX | Z, NH>(C, it, R, hb);
+                else run_rows<LXS | Z, NH>(C, it, R, hb);
+            } else if (ly) {
+                run_rows<LY | Z, NH>(C, it, R, hb);
+            } else {
+                run_rows<Z, NH>(C, it, R, hb);
+            }
         } else {
             if (layer) run_halo<true, NH>(C, it, R, hb);
             else run_halo<false, NH>(C, it, R, hb);
@@ -1021,14 +1062,14 @@ __device__ __forceinline__ void consume(const Cons<NH> &C, const BatchArgs &B, S
 // BATCH = false: one domain whose arguments and descriptors are the kernel's
 // own parameters (constant bank); BATCH = true: a table of domains in global
 // memory, the current domain's arguments staged in shared memory.
-template <bool ZL, int NH, bool BATCH, bool WIDE>
+template <bool ZL, int NH, bool BATCH>
 __global__ void __launch_bounds__(NTHREADS, 2) step_tma_kernel(const __grid_constant__ SingleArgs S,
                                                               const BatchArgs B)
 {
     extern __shared__ __align__(128) char smem_raw[];
     // TMA destinations are kept 128-byte aligned
     char *smem = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const Layout Lo(B.region, NH);
     StepArgs *sa = reinterpret_cast<StepArgs *>(smem + Lo.tab);          // current domain's arguments
     float *tab = reinterpret_cast<float *>(smem + Lo.tab + al128(sizeof(StepArgs)));
@@ -1060,6 +1101,7 @@ __global__ void __launch_bounds__(NTHREADS, 2) step_tma_kernel(const __grid_cons
             }
         }
     }
+    if (threadIdx.x < 16) xc[6 * TX + threadIdx.x] = threadIdx.x == 2 ? 1.f : 0.f;
     if (threadIdx.x == 0) {
         for (int q = 0; q < NE; ++q) {
             mbar_init(C.fullE(q), 1);
@@ -1075,7 +1117,7 @@ __global__ void __launch_bounds__(NTHREADS, 2) step_tma_kernel(const __grid_cons
     }
     __syncthreads();
 
-    if (warp >= NCW) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(AUX_REGS));
+    if (warp >= NCW) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(aux_regs(BATCH)));
     if (warp >= NCW + NHW) {
         // ------------------------------ producer ------------------------------
         // The whole warp runs the loop, every value the same in all lanes
@@ -1102,11 +1144,7 @@ __global__ void __launch_bounds__(NTHREADS, 2) step_tma_kernel(const __grid_cons
                 const StepArgs &a = BATCH ? B.doms[dom].a[B.launch][B.parity] : S.a;
                 const TmaMaps &m = BATCH ? B.doms[dom].m[B.parity] : S.m;
                 const int item = BATCH ? gitem - __ldg(B.item_start + dom) : gitem;
-                Item it = decode(a, item);
-                it.x0 = __shfl_sync(0xffffffffu, it.x0, 0);
-                it.y0 = __shfl_sync(0xffffffffu, it.y0, 0);
-                it.ka = __shfl_sync(0xffffffffu, it.ka, 0);
-                it.kb = __shfl_sync(0xffffffffu, it.kb, 0);
+                const Item it = uniform(decode(a, item));
                 const int nz = a.nz, d = a.d, ox = a.ox, oy = a.oy;
                 // x / y boxes of the tile, and what they add to a plane
                 int fxy = 0, xs = 0, ys = 0;
@@ -1196,10 +1234,10 @@ __global__ void __launch_bounds__(NTHREADS, 2) step_tma_kernel(const __grid_cons
             }
         }
     } else if (warp >= NCW) {
-        consume<false, ZL, NH, BATCH, WIDE>(C, B, sa, cons_e, cons_h);
+        consume<false, ZL, NH, BATCH>(C, B, sa, cons_e, cons_h);
     } else {
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(ROW_REGS));
-        consume<true, ZL, NH, BATCH, WIDE>(C, B, sa, cons_e, cons_h);
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(row_regs(BATCH)));
+        consume<true, ZL, NH, BATCH>(C, B, sa, cons_e, cons_h);
     }
     __syncthreads();
     // on an abort, wait (bounded) for copies still in flight before the
@@ -1270,21 +1308,20 @@ void step_region(const PsiGeom &pg, int zxy, int *region, int *ox, int *oy)
 }
 // the kernel of launch l (1: the z-layer planes)
 using StepKernel = void (*)(SingleArgs, BatchArgs);
-static StepKernel step_kernel(int l, int nh, bool batch, bool wide)
+static StepKernel step_kernel(int l, int nh, bool batch)
 {
-    static const StepKernel k[2][2][3] = {
-        {{step_tma_kernel<false, 2, false, false>, step_tma_kernel<false, 2, false, true>, step_tma_kernel<false, 2, true, false>},
-         {step_tma_kernel<false, 3, false, false>, step_tma_kernel<false, 3, false, true>, step_tma_kernel<false, 3, true, false>}},
-        {{step_tma_kernel<true, 2, false, false>, step_tma_kernel<true, 2, false, true>, step_tma_kernel<true, 2, true, false>},
-         {step_tma_kernel<true, 3, false, false>, step_tma_kernel<true, 3, false, true>, step_tma_kernel<true, 3, true, false>}}};
-    return k[l][nh == 3][batch ? 2 : (wide ? 1 : 0)];
+    static const StepKernel k[2][2][2] = {{{step_tma_kernel<false, 2, false>, step_tma_kernel<false, 2, true>},
+                                           {step_tma_kernel<false, 3, false>, step_tma_kernel<false, 3, true>}},
+                                          {{step_tma_kernel<true, 2, false>, step_tma_kernel<true, 2, true>},
+                                           {step_tma_kernel<true, 3, false>, step_tma_kernel<true, 3, true>}}};
+    return k[l][nh == 3][batch];
 }
-const void *step_kernel_ptr(int l, int nh, bool batch, bool wide) { return (const void *)step_kernel(l, nh, batch, wide); }
+const void *step_kernel_ptr(int l, int nh, bool batch) { return (const void *)step_kernel(l, nh, batch); }
 
 cudaError_t launch_step(const SingleArgs &one, const BatchArgs &b, int grid, cudaStream_t s)
 {
     const int smem = smem_bytes(b.max_classes, b.max_d, b.region, b.nh);
-    step_kernel(b.launch, b.nh, b.doms != nullptr, b.wide)<<<grid, NTHREADS, smem, s>>>(one, b);
+    step_kernel(b.launch, b.nh, b.doms != nullptr)<<<grid, NTHREADS, smem, s>>>(one, b);
     return cudaGetLastError();
 }
 
