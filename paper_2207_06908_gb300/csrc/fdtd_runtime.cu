@@ -1454,6 +1454,103 @@ int step_queue(fdtd_grid *g, int n)
     return FDTD_OK;
 }
 
+// Page-locked staging blocks for small read-backs, shared by every grid of
+// the process and handed to one call at a time; at most kKept stay allocated
+// while unused (they are freed with the process).
+class Staging {
+public:
+    static constexpr size_t kBytes = 64 << 10;
+    static constexpr size_t kKept = 8;
+    Staging()
+    {
+        std::lock_guard<std::mutex> lock(mu());
+        if (!pool().empty()) {
+            p_ = pool().back();
+            pool().pop_back();
+        }
+        if (!p_ && cudaHostAlloc(&p_, kBytes, cudaHostAllocPortable) != cudaSuccess) {
+            p_ = nullptr;
+            cudaGetLastError();
+        }
+    }
+    ~Staging()
+    {
+        if (!p_) return;
+        {
+            std::lock_guard<std::mutex> lock(mu());
+            if (pool().size() < kKept) {
+                pool().push_back(p_);
+                return;
+            }
+        }
+        cudaFreeHost(p_);
+    }
+    Staging(const Staging &) = delete;
+    Staging &operator=(const Staging &) = delete;
+    char *data() const { return static_cast<char *>(p_); }
+
+private:
+    static std::mutex &mu()
+    {
+        static std::mutex m;
+        return m;
+    }
+    static std::vector<void *> &pool()
+    {
+        static auto *v = new std::vector<void *>;
+        return *v;
+    }
+    void *p_ = nullptr;
+};
+
+// Wait for the grid's queued work, report what its flags hold and bring
+// `count` floats from src to dst (NULL, 0: none).  The flags and the first
+// floats travel behind the work on the grid's stream, so the call waits once:
+// with a blocking copy each for the two flags and the data a probe read took
+// about 30 us.  On an error the floats are not delivered.
+int finish(fdtd_grid *g, const float *src, size_t count, float *dst)
+{
+    cudaStream_t s = g->stream;
+    const Staging st;
+    const size_t room = st.data() ? (Staging::kBytes - 64) / sizeof(float) : 0, head = std::min(count, room);
+    int pageable[3] = {0, 0, 0};
+    // the step kernel's and the watchdog's flags are neighbours (err_d, div_d)
+    int *flag = st.data() ? reinterpret_cast<int *>(st.data()) : pageable;
+    flag[0] = flag[1] = flag[2] = 0;
+    cudaError_t e = cudaSuccess;
+    if (g->finalized) {
+        e = cudaMemcpyAsync(flag, g->err_d, 2 * sizeof(int), cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess && g->noalloc_err)
+            e = cudaMemcpyAsync(flag + 2, g->noalloc_err, sizeof(int), cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess && head)
+            e = cudaMemcpyAsync(st.data() + 64, src, head * sizeof(float), cudaMemcpyDeviceToHost, s);
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) return cuda_fail(g, e, "synchronize");
+    auto clear = [&](int *dev) {
+        cudaError_t c = cudaMemsetAsync(dev, 0, sizeof(int), s);
+        return c == cudaSuccess ? cudaStreamSynchronize(s) : c;
+    };
+    if (flag[0]) return fail(g, FDTD_ETIMEOUT, "a bounded wait in the step kernel gave up");
+    if (flag[1]) {
+        // reported once per detection; a later check finds it again if the fields still diverge
+        if ((e = clear(g->div_d)) != cudaSuccess) return cuda_fail(g, e, "watchdog flag clear");
+        return fail(g, FDTD_EDIVERGED, "the watchdog found a NaN or an infinity in the fields");
+    }
+    if (flag[2]) {
+        // the shared flag of fdtd_step_noalloc(): read and cleared on this
+        // grid's stream (it never holds a work counter)
+        if ((e = clear(g->noalloc_err)) != cudaSuccess) return cuda_fail(g, e, "error flag clear");
+        return fail(g, FDTD_ETIMEOUT, "a bounded wait in the step kernel gave up (fdtd_step_noalloc)");
+    }
+    if (head) std::memcpy(dst, st.data() + 64, head * sizeof(float));
+    if (count > head) {
+        e = cudaMemcpy(dst + head, src + head, (count - head) * sizeof(float), cudaMemcpyDeviceToHost);
+        if (e != cudaSuccess) return cuda_fail(g, e, "probe copy");
+    }
+    return FDTD_OK;
+}
+
 int check_open(fdtd_grid *g, bool want_finalized)
 {
     if (!g) return FDTD_EINVAL;
@@ -2134,37 +2231,7 @@ int fdtd_step(fdtd_grid *g, int n)
 int fdtd_synchronize(fdtd_grid *g)
 {
     if (!g) return FDTD_EINVAL;
-    cudaError_t e = cudaStreamSynchronize(g->stream);
-    if (e != cudaSuccess) return cuda_fail(g, e, "synchronize");
-    if (g->finalized) {
-        int flag = 0;
-        e = cudaMemcpy(&flag, g->err_d, sizeof flag, cudaMemcpyDeviceToHost);
-        if (e != cudaSuccess) return cuda_fail(g, e, "error flag read");
-        if (flag) return fail(g, FDTD_ETIMEOUT, "a bounded wait in the step kernel gave up");
-        e = cudaMemcpy(&flag, g->div_d, sizeof flag, cudaMemcpyDeviceToHost);
-        if (e != cudaSuccess) return cuda_fail(g, e, "watchdog flag read");
-        if (flag) {
-            // reported once per detection; a later check finds it again if the fields still diverge
-            e = cudaMemsetAsync(g->div_d, 0, sizeof flag, g->stream);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
-            if (e != cudaSuccess) return cuda_fail(g, e, "watchdog flag clear");
-            return fail(g, FDTD_EDIVERGED, "the watchdog found a NaN or an infinity in the fields");
-        }
-        if (g->noalloc_err) {
-            // the shared flag of fdtd_step_noalloc(): read and cleared on this
-            // grid's stream (it never holds a work counter)
-            e = cudaMemcpyAsync(&flag, g->noalloc_err, sizeof flag, cudaMemcpyDeviceToHost, g->stream);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
-            if (e != cudaSuccess) return cuda_fail(g, e, "error flag read");
-            if (flag) {
-                e = cudaMemsetAsync(g->noalloc_err, 0, sizeof flag, g->stream);
-                if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
-                if (e != cudaSuccess) return cuda_fail(g, e, "error flag clear");
-                return fail(g, FDTD_ETIMEOUT, "a bounded wait in the step kernel gave up (fdtd_step_noalloc)");
-            }
-        }
-    }
-    return FDTD_OK;
+    return finish(g, nullptr, 0, nullptr);
 }
 
 int fdtd_read_probes(fdtd_grid *g, int probe_id, int first_step, int count, float *host_out)
@@ -2173,12 +2240,7 @@ int fdtd_read_probes(fdtd_grid *g, int probe_id, int first_step, int count, floa
     if (probe_id < 0 || probe_id >= (int)g->probes.size() || first_step < 0 || count < 0 ||
         (long long)first_step + count > g->capacity || (count > 0 && !host_out))
         return fail(g, FDTD_EINVAL, "probe range outside the recorded window");
-    if (int rc = fdtd_synchronize(g)) return rc;
-    if (count == 0) return FDTD_OK;
-    cudaError_t e = cudaMemcpy(host_out, g->probe_out + (size_t)probe_id * g->capacity + first_step,
-                               (size_t)count * sizeof(float), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return cuda_fail(g, e, "probe copy");
-    return FDTD_OK;
+    return finish(g, g->probe_out + (size_t)probe_id * g->capacity + first_step, (size_t)count, host_out);
 }
 
 int fdtd_get_field(fdtd_grid *g, int component, float *host_out)
@@ -2674,11 +2736,12 @@ int fdtd_batch_step(fdtd_batch *b, int n)
 int fdtd_batch_synchronize(fdtd_batch *b)
 {
     if (!b) return FDTD_EINVAL;
-    cudaError_t e = cudaStreamSynchronize(b->stream);
+    const Staging st;
+    int pageable = 0, *flag_h = st.data() ? reinterpret_cast<int *>(st.data()) : &pageable;
+    cudaError_t e = cudaMemcpyAsync(flag_h, b->errf, sizeof(int), cudaMemcpyDeviceToHost, b->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) return bfail(b, FDTD_ECUDA, std::string("synchronize: ") + cudaGetErrorString(e));
-    int flag = 0;
-    e = cudaMemcpy(&flag, b->errf, sizeof flag, cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return bfail(b, FDTD_ECUDA, "error flag read");
+    const int flag = *flag_h;
     if (flag) return bfail(b, FDTD_ETIMEOUT, "a bounded wait in the step kernel gave up");
     return FDTD_OK;
 }
