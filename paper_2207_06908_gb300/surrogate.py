@@ -183,8 +183,13 @@ def features(params):
     input is mapped affinely (radius logarithmically) onto about [-1, 1] over
     its sampled range."""
     p = np.asarray(params, dtype=np.float64).reshape(-1, N_IN)
-    cells = np.array([W.grounding_cells(l, d) for l, d in p[:, [2, 4]]], dtype=np.float64).reshape(-1, 2)
-    length, depth = cells[:, 0] * W.GROUND_DX, cells[:, 1] * W.GROUND_DX
+    # W.grounding_cells for all rows at once (rint and round are both half to
+    # even; a row at a time took 8.1 ms for 4096 rows, this 0.1)
+    if not np.isfinite(p[:, [2, 4]]).all():
+        for l, d in p[:, [2, 4]]:
+            W.grounding_cells(l, d)             # raises for the first such value
+    length = np.maximum(np.rint(p[:, 2] / W.GROUND_DX), 1.0) * W.GROUND_DX
+    depth = np.rint(p[:, 4] / W.GROUND_DX) * W.GROUND_DX
     return np.stack([(p[:, 0] - 22.0) / 18.0,
                      (p[:, 1] + 2.5) / 1.5,
                      (length - 5.0) / 4.0,
