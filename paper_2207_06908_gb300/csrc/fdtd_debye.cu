@@ -40,6 +40,7 @@ __global__ void __launch_bounds__(256) debye_kernel(const DebyeArgs a)
                 if (tab[r * kDebyeRec + c * kMaxPoles * 3 + 3 * p + 2] != 0.f) m |= 1 << c;
         mask[r] = m;
     }
+    step_chain();
     __syncthreads();
     const uchar4 *__restrict__ dcls4 = reinterpret_cast<const uchar4 *>(a.dcls);
     const long long n4 = a.jstride / 4;
@@ -54,7 +55,7 @@ __global__ void __launch_bounds__(256) debye_kernel(const DebyeArgs a)
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             if (!(comps >> c & 1)) continue;
-            e0[c] = __ldg(reinterpret_cast<const float4 *>(a.Ein[c] + g));
+            e0[c] = *reinterpret_cast<const float4 *>(a.Ein[c] + g);
             e1[c] = *reinterpret_cast<const float4 *>(a.Eout[c] + g);
 #pragma unroll
             for (int p = 0; p < np; ++p)

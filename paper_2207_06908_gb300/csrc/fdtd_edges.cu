@@ -145,7 +145,11 @@ __device__ __forceinline__ void edge_body(const EdgeArgs &a)
     src_probe_body(a, n);
 }
 
-__global__ void edge_kernel(const EdgeArgs a) { edge_body<false>(a); }
+__global__ void edge_kernel(const EdgeArgs a)
+{
+    step_chain();
+    edge_body<false>(a);
+}
 
 // The second half on a single grid: a thread per coupled edge, then per node
 // (the charges read the currents only), over as many CTAs as that takes.  A
@@ -157,7 +161,8 @@ constexpr int kWireThreads = 128;
 __global__ void __launch_bounds__(kWireThreads) wire_finish_kernel(const EdgeArgs a)
 {
     const WireArgs &w = a.w;
-    auto cur = [&](int s) { return __ldg(w.I + s); };
+    step_chain();
+    auto cur = [&](int s) { return __ldcg(w.I + s); };
     const int u = blockIdx.x * kWireThreads + threadIdx.x;
     if (u < w.n_scat) {
         OScat sc = w.scat[u];
@@ -178,7 +183,8 @@ __global__ void __launch_bounds__(kWireThreads) wire_finish_kernel(const EdgeArg
 __global__ void wire_gather_kernel(const EdgeArgs a)
 {
     __shared__ long long n_s;
-    if (threadIdx.x == 0) n_s = *a.step + a.step_t;
+    step_chain();
+    if (threadIdx.x == 0) n_s = __ldcg(a.step) + a.step_t;
     __syncthreads();
     wire_gather_body(a, n_s);
 }
@@ -187,6 +193,7 @@ __global__ void edge_batch_kernel(const EdgeArgs *e, int parity)
 {
     __shared__ EdgeArgs a;
     if (threadIdx.x == 0) a = e[2 * blockIdx.x + parity];
+    step_chain();
     __syncthreads();
     if (a.n_src > 0 || a.n_probes > 0 || a.w.n_seg > 0) edge_body<true>(a);
 }
@@ -196,6 +203,7 @@ __global__ void wire_gather_batch_kernel(const EdgeArgs *e, int parity)
 {
     __shared__ EdgeArgs a;
     __shared__ long long n_s;
+    step_chain();
     if (threadIdx.x == 0) {
         a = e[2 * blockIdx.x + parity];
         if (a.w.n_seg > 0) n_s = __ldcg(a.step) + a.step_t;

@@ -273,6 +273,20 @@ __device__ __forceinline__ bool in_bounds(long long idx, long long n, int site, 
 __device__ __forceinline__ bool in_bounds(long long, long long, int, int *) { return true; }
 #endif
 
+#ifdef __CUDACC__
+// Every kernel of a time step begins with this: wait until the launches it
+// depends on have finished and their stores are visible, then let the ones
+// that depend on it start.  In a captured graph, where those dependencies are
+// programmatic (runtime), a kernel's CTAs are then placed and its constant
+// data read while the kernels before it end.  What runs before it must not
+// touch anything a time step writes.  Without such a dependency it does nothing.
+__device__ __forceinline__ void step_chain()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+#endif
+
 // the six field arrays of one state (Ex Ey Ez Hx Hy Hz)
 struct FieldPtrs {
     const float *p[6];

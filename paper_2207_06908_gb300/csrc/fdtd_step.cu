@@ -110,9 +110,9 @@ constexpr int H_COMP = HBX * HBY * 4;
 constexpr int C_BYTES = al128(CBX * CBY);
 constexpr int PE_BYTES = TX * TY * 4;                // E-type psi box: the tile itself
 // E slot: three E boxes and a header: item, -, staged-layer flags of the
-// plane, x-box start, y-box start, domain
+// plane, x-box start, y-box start, domain, the item's x0, y0, ka, kb
 constexpr int OFF_HDR = 3 * E_COMP;
-constexpr int ESLOT = al128(OFF_HDR + 32);
+constexpr int ESLOT = al128(OFF_HDR + 40);
 // H slot: three H boxes, the class box, then the staged-auxiliary region
 // (grid dependent size).  In a z-layer plane the region holds the z boxes
 // (2 H-type with the H box, 2 E-type with the tile box); elsewhere the x
@@ -532,8 +532,8 @@ __device__ __forceinline__ void h_belowx(const StepArgs &a, const Pair &G, const
     F2 hy_x = next_diff(ez, ez_e), hy_z = sub2(ex_z1, ex);
     auto far = [&](const float *arr, int g, int m, int u) {
         float o0 = 0.f, o1 = 0.f;
-        if ((m & 1) && in_bounds(g, psi_n(a, u), 4, a.bounds)) o0 = __ldg(arr + g);
-        if ((m & 2) && in_bounds(g + 1, psi_n(a, u), 4, a.bounds)) o1 = __ldg(arr + g + 1);
+        if ((m & 1) && in_bounds(g, psi_n(a, u), 4, a.bounds)) o0 = __ldcg(arr + g);
+        if ((m & 2) && in_bounds(g + 1, psi_n(a, u), 4, a.bounds)) o1 = __ldcg(arr + g + 1);
         return pk(o0, o1);
     };
     if (G.fl & XM) {
@@ -1014,7 +1014,7 @@ __device__ __forceinline__ void consume(const Cons<NH> &C, const BatchArgs &B, S
             consumer_sync();
         }
         const StepArgs &a = *C.a;
-        const Item it = uniform(decode(a, item));
+        const Item it = uniform(Item{hdr[6], hdr[7], hdr[8], hdr[9]});
         const bool layer = item_in_cpml(a, it);
         if (layer) fill_xc(a, C.prof, C.xc, it.x0, tid);
         const uint32_t n = R.e_next();
@@ -1136,7 +1136,12 @@ __global__ void __launch_bounds__(NTHREADS, 2) step_tma_kernel(const __grid_cons
                 se = (se + 1) % NE;
                 pe ^= se == 0;
             };
-            int next = lane == 0 ? atomicAdd(B.work, 1) : 0;
+            // The CTA's first item is its own number (the grid has no more
+            // CTAs than items), the counter hands out the ones after those:
+            // nothing has to travel before the first copies but the wait for
+            // the step before, and that comes when all else is ready.
+            int next = blockIdx.x;
+            bool first = true;
             while (ok) {
                 const int gitem = __shfl_sync(0xffffffffu, next, 0);
                 if (gitem >= B.nitems) break;
@@ -1167,12 +1172,18 @@ __global__ void __launch_bounds__(NTHREADS, 2) step_tma_kernel(const __grid_cons
                         hdr[3] = xs;
                         hdr[4] = ys;
                         hdr[5] = dom;
+                        hdr[6] = it.x0;
+                        hdr[7] = it.y0;
+                        hdr[8] = it.ka;
+                        hdr[9] = it.kb;
                         mbar_expect_tx(C.fullE(se), TX_E);
                         tma_load(smem_u32(es), &m.e, it.x0 - XO, it.y0 - 1, z, C.fullE(se));
                     }
                     __syncwarp();
                     next_e();
                 };
+                if (first) step_chain();
+                first = false;
                 if (!wait(C.emptyE(se), pe)) { ok = false; break; }
                 load_e(it.ka - 1);
                 for (int z = it.ka - 1; z < it.kb; ++z) {
@@ -1198,7 +1209,7 @@ __global__ void __launch_bounds__(NTHREADS, 2) step_tma_kernel(const __grid_cons
                     ph ^= sh == 0;
                     load_e(z + 1);
                     // the next item's number travels while this one's last planes are issued
-                    if (z == max(it.ka - 1, it.kb - 3) && lane == 0) next = atomicAdd(B.work, 1);
+                    if (z == max(it.ka - 1, it.kb - 3) && lane == 0) next = gridDim.x + atomicAdd(B.work, 1);
                 }
             }
             if (ok) {
