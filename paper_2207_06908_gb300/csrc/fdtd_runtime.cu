@@ -156,8 +156,8 @@ struct fdtd_grid {
     int *order_d = nullptr;               // column tiles in the order a z block hands them out
     std::vector<int> order_pos;           // position of each column tile in that order
     // single-grid steps apply the current sources in the step kernel and read
-    // the probes of step n beside step n + 1 (no Debye media, no ideal voltage
-    // sources, at most 32 sources, none beside oblique wires)
+    // the probes of step n beside step n + 1 (no ideal voltage sources, at most
+    // 32 sources, none on a dispersive edge or beside oblique wires)
     bool fast = false;
     fdtd::DomainSlot slot_h;              // host copy (also read by batches)
     fdtd::EdgeArgs edge_h[2];             // edge-kernel arguments per input parity
@@ -1143,6 +1143,7 @@ cudaError_t enqueue_step_fast(fdtd_grid *g, int parity, cudaStream_t s, int t, b
         for (int l = 0; l < g->n_launch && e == cudaSuccess; ++l) e = launch(l)(s);
     }
     if (e == cudaSuccess && wires) e = fdtd::launch_wire_finish(edge_args(g, parity), s);
+    if (e == cudaSuccess && g->npoles) e = fdtd::launch_debye(debye_args(g, parity), s);
     if (e == cudaSuccess && last) {
         fdtd::EdgeArgs pa = edge_args(g, parity);
         pa.n_src = 0;
@@ -2202,7 +2203,11 @@ int fdtd_finalize(fdtd_grid *g, int probe_capacity, void *arena, size_t arena_by
     // current sources in the step kernel: each source's launch and work item
     // (with oblique wires, whose currents come before the sources', only
     // without sources)
-    g->fast = g->npoles == 0 && (g->osegs.empty() || g->srcs.empty()) && g->srcs.size() <= 32 && has_edge_work(g);
+    g->fast = (g->osegs.empty() || g->srcs.empty()) && g->srcs.size() <= 32 && has_edge_work(g);
+    // a source on a dispersive edge comes after the polarisation currents and
+    // moves them too (100x100x80 array over three Debye layers, sources in
+    // air: the serial source / probe launch was 5 of 46 us a step)
+    for (const fdtd::SourceDesc &d : sd) g->fast = g->fast && d.jidx < 0;
     for (const Source &src : g->srcs) g->fast = g->fast && !src.hard;
     if (g->fast && !g->srcs.empty()) {
         using namespace fdtd::geom;
