@@ -19,13 +19,21 @@
 namespace fdtd {
 namespace {
 
-__device__ __forceinline__ float &el(float4 &v, int t) { return reinterpret_cast<float *>(&v)[t]; }
+// V consecutive floats (V = 2, 4) as one access
+template <int V>
+struct __align__(4 * V) Vec {
+    float v[V];
+};
 
-// Each thread takes four consecutive elements of the box (16-byte aligned:
-// the plane is a multiple of 16 elements), issues every load of its
-// dispersive components first (E^n, E^{n+1}, the currents, all float4),
-// then updates and stores them.
-template <int NP>
+// Each thread takes V consecutive elements of the box (aligned to them: the
+// plane is a multiple of 16 elements), issues every load of its dispersive
+// components first (E^n, E^{n+1}, the currents), then updates and stores
+// them.  Bound by DRAM.  With two to four poles V = 4 holds 96 to 167
+// registers and leaves few threads per SM; V = 2 takes 64 to 96 (256^3 with
+// half of it soil and four poles, whole step: 331.9 us against 343.5; 128^3
+// 54.7 against 57.4, with two poles 43.8 against 45.5).  With one pole the
+// wider accesses win (236.2 us against 237.8; 100x100x80 24.1 against 24.6).
+template <int NP, int V>
 __global__ void __launch_bounds__(256) debye_kernel(const DebyeArgs a)
 {
     extern __shared__ float tab[];          // [n_rec][kDebyeRec], then a component mask per record
@@ -42,46 +50,66 @@ __global__ void __launch_bounds__(256) debye_kernel(const DebyeArgs a)
     }
     step_chain();
     __syncthreads();
-    const uchar4 *__restrict__ dcls4 = reinterpret_cast<const uchar4 *>(a.dcls);
-    const long long n4 = a.jstride / 4;
-    for (long long q4 = (long long)blockIdx.x * blockDim.x + threadIdx.x; q4 < n4;
-         q4 += (long long)gridDim.x * blockDim.x) {
-        const uchar4 rv = __ldg(dcls4 + q4);
-        const int rec[4] = {rv.x, rv.y, rv.z, rv.w};
-        const int comps = mask[rec[0]] | mask[rec[1]] | mask[rec[2]] | mask[rec[3]];
+    using F = Vec<V>;
+    struct __align__(V) Recs {
+        uint8_t r[V];
+    };
+    const Recs *__restrict__ dcls = reinterpret_cast<const Recs *>(a.dcls);
+    const long long nv = a.jstride / V;
+    for (long long qv = (long long)blockIdx.x * blockDim.x + threadIdx.x; qv < nv;
+         qv += (long long)gridDim.x * blockDim.x) {
+        const Recs rec = dcls[qv];
+        int comps = 0;
+#pragma unroll
+        for (int t = 0; t < V; ++t) comps |= mask[rec.r[t]];
         if (!comps) continue;
-        const long long q = 4 * q4, g = a.off + q;
-        float4 e0[3], e1[3], jv[3][NP];
+        const long long q = V * qv, g = a.off + q;
+        F e0[3], e1[3], jv[3][NP];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             if (!(comps >> c & 1)) continue;
-            e0[c] = *reinterpret_cast<const float4 *>(a.Ein[c] + g);
-            e1[c] = *reinterpret_cast<const float4 *>(a.Eout[c] + g);
+            e0[c] = *reinterpret_cast<const F *>(a.Ein[c] + g);
+            e1[c] = *reinterpret_cast<const F *>(a.Eout[c] + g);
 #pragma unroll
             for (int p = 0; p < np; ++p)
-                jv[c][p] = *reinterpret_cast<const float4 *>(a.J + (long long)(c * np + p) * a.jstride + q);
+                jv[c][p] = *reinterpret_cast<const F *>(a.J + (long long)(c * np + p) * a.jstride + q);
         }
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             if (!(comps >> c & 1)) continue;
-            float4 e = e1[c];
+            F e = e1[c];
 #pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                const float *rc = tab + rec[t] * kDebyeRec + c * kMaxPoles * 3;
-                float v = el(e, t);
+            for (int t = 0; t < V; ++t) {
+                const float *rc = tab + rec.r[t] * kDebyeRec + c * kMaxPoles * 3;
+                float v = e.v[t];
 #pragma unroll
-                for (int p = 0; p < np; ++p) v += rc[3 * p] * el(jv[c][p], t);
+                for (int p = 0; p < np; ++p) v += rc[3 * p] * jv[c][p].v[t];
 #pragma unroll
                 for (int p = 0; p < np; ++p)
-                    el(jv[c][p], t) = rc[3 * p + 1] * el(jv[c][p], t) + rc[3 * p + 2] * (v - el(e0[c], t));
-                el(e, t) = v;
+                    jv[c][p].v[t] = rc[3 * p + 1] * jv[c][p].v[t] + rc[3 * p + 2] * (v - e0[c].v[t]);
+                e.v[t] = v;
             }
 #pragma unroll
             for (int p = 0; p < np; ++p)
-                *reinterpret_cast<float4 *>(a.J + (long long)(c * np + p) * a.jstride + q) = jv[c][p];
-            *reinterpret_cast<float4 *>(a.Eout[c] + g) = e;
+                *reinterpret_cast<F *>(a.J + (long long)(c * np + p) * a.jstride + q) = jv[c][p];
+            *reinterpret_cast<F *>(a.Eout[c] + g) = e;
         }
     }
+}
+
+template <int NP, int V>
+cudaError_t run_debye(const DebyeArgs &a, int sms, cudaStream_t s)
+{
+    const long long blocks = std::min<long long>((a.jstride / V + 255) / 256, 8LL * sms);
+    const size_t smem = (size_t)a.n_rec * (kDebyeRec * sizeof(float) + sizeof(int));
+    debye_kernel<NP, V><<<(unsigned)std::max<long long>(blocks, 1), 256, smem, s>>>(a);
+    return cudaGetLastError();
+}
+
+template <int NP>
+cudaError_t run_debye(const DebyeArgs &a, int sms, cudaStream_t s)
+{
+    return run_debye<NP, (NP >= 2 ? 2 : 4)>(a, sms, s);
 }
 
 }  // namespace
@@ -95,17 +123,13 @@ cudaError_t launch_debye(const DebyeArgs &a, cudaStream_t s)
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
             sms = 148;
     }
-    const long long blocks = std::min<long long>((a.jstride / 4 + 255) / 256, 8LL * sms);
-    const dim3 grid((unsigned)std::max<long long>(blocks, 1));
-    const size_t smem = (size_t)a.n_rec * (kDebyeRec * sizeof(float) + sizeof(int));
     switch (a.npoles) {
-    case 1: debye_kernel<1><<<grid, 256, smem, s>>>(a); break;
-    case 2: debye_kernel<2><<<grid, 256, smem, s>>>(a); break;
-    case 3: debye_kernel<3><<<grid, 256, smem, s>>>(a); break;
-    case 4: debye_kernel<4><<<grid, 256, smem, s>>>(a); break;
+    case 1: return run_debye<1>(a, sms, s);
+    case 2: return run_debye<2>(a, sms, s);
+    case 3: return run_debye<3>(a, sms, s);
+    case 4: return run_debye<4>(a, sms, s);
     default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 }  // namespace fdtd
