@@ -614,7 +614,7 @@ def main():
                 "ms_per_step": ms / K, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
                 "dtype": "f32", "data": "synthetic", "config": workload_config(sc, K),
                 "roofline": roofline, "cpu_baseline": cpu, "e2e": e2e, "clocks": clocks,
-                "gpu_launches": (3 + bool(getattr(sc, "debye", None)) + bool(getattr(sc, "owires", None))) * K,
+                "gpu_launches": (3 + bool(getattr(sc, "debye", None)) + 2 * bool(getattr(sc, "owires", None))) * K,
                 "finite": finite}
         line.update(sub)
         print(json.dumps(line), flush=True)

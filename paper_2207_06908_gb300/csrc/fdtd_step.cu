@@ -40,8 +40,9 @@
 // of offsets took 11 % more instructions (256^3 PEC 134 us).  Measured (us
 // per step; one cell per lane, fifteen copies a plane and 16 planes per item
 // before): 256^3 PEC 136.3 -> 129.8, 256^3 with a 10-cell CPML 175.9 ->
-// 162.8, 512x512x384 with 12 cells 956 -> 909, 128^3 with 8 cells 42.7 ->
-// 33.6, 64^3 with 8 cells 25.6 -> 10.4.
+// 160.8, 512x512x384 with 12 cells 956 -> 905, 128^3 with 8 cells 42.7 ->
+// 31.9, 64^3 with 8 cells 25.6 -> 9.3 (programmatic dependencies between the
+// steps' kernels, fdtd_runtime.cu, included).
 // DRAM traffic per cell and step: 6 FP32 reads + 6 writes + 1 class byte
 // (49 B) plus the CPML auxiliaries in the layer; every halo read is an L2
 // hit.  Every wait is bounded; on a timeout the kernel records an error
