@@ -12,6 +12,7 @@
 #include <cstring>
 #include <map>
 #include <mutex>
+#include <new>
 #include <array>
 #include <string>
 #include <thread>
@@ -106,7 +107,73 @@ struct Fork {
     }
 };
 
+// Page-locked staging blocks for small read-backs, shared by every grid and
+// batch of the process and handed to one call at a time.  At most kKept stay
+// allocated while unused, and only while a grid or batch lives (each holds a
+// User): the last one gives them back.
+class Staging {
+public:
+    static constexpr size_t kBytes = 64 << 10;
+    Staging()
+    {
+        {
+            std::lock_guard<std::mutex> lock(pool().mu);
+            if (pool().n) p_ = pool().kept[--pool().n];
+        }
+        if (!p_ && cudaHostAlloc(&p_, kBytes, cudaHostAllocPortable) != cudaSuccess) {
+            p_ = nullptr;
+            cudaGetLastError();
+        }
+    }
+    ~Staging()
+    {
+        if (!p_) return;
+        {
+            std::lock_guard<std::mutex> lock(pool().mu);
+            if (pool().n < kKept) {
+                pool().kept[pool().n++] = p_;
+                return;
+            }
+        }
+        cudaFreeHost(p_);
+    }
+    Staging(const Staging &) = delete;
+    Staging &operator=(const Staging &) = delete;
+    char *data() const { return static_cast<char *>(p_); }
+
+    struct User {
+        User()
+        {
+            std::lock_guard<std::mutex> lock(pool().mu);
+            ++pool().users;
+        }
+        ~User()
+        {
+            std::lock_guard<std::mutex> lock(pool().mu);
+            if (--pool().users) return;
+            while (pool().n) cudaFreeHost(pool().kept[--pool().n]);
+        }
+        User(const User &) = delete;
+        User &operator=(const User &) = delete;
+    };
+
+private:
+    static constexpr int kKept = 8;
+    struct Pool {
+        std::mutex mu;
+        void *kept[kKept];
+        int n, users;
+    };
+    static Pool &pool()
+    {
+        static Pool v{};
+        return v;
+    }
+    void *p_ = nullptr;
+};
+
 struct fdtd_grid {
+    Staging::User staging_user;
     int nx = 0, ny = 0, nz = 0;
     double dx = 0, dt = 0, courant = 0;
     fdtd_cpml cpml{};
@@ -1404,7 +1471,7 @@ cudaError_t enqueue_watch(fdtd_grid *g, cudaStream_t s)
 // while these end.  Measured per step, with the step kernel's first items
 // fixed: 48^3 PEC 6.1 -> 5.6 us, 64^3 with an 8-cell CPML 10.4 -> 9.3, 256^3
 // with 10 cells 162.8 -> 160.8, eight 64^3 domains 46.1 -> 38.6.
-cudaError_t make_programmatic(cudaGraph_t graph)
+cudaError_t make_programmatic(cudaGraph_t graph) try
 {
     size_t n = 0;
     cudaError_t e = cudaGraphGetEdges(graph, nullptr, nullptr, nullptr, &n);
@@ -1432,6 +1499,8 @@ cudaError_t make_programmatic(cudaGraph_t graph)
     data.assign(m, prog);
     if (e == cudaSuccess) e = cudaGraphAddDependencies(graph, from.data(), to.data(), data.data(), m);
     return e;
+} catch (const std::bad_alloc &) {
+    return cudaErrorMemoryAllocation;
 }
 
 // Which graphs of 2^k steps (bit k, k = 1 .. 5) a call with n steps left
@@ -1499,55 +1568,6 @@ int step_queue(fdtd_grid *g, int n)
     return FDTD_OK;
 }
 
-// Page-locked staging blocks for small read-backs, shared by every grid of
-// the process and handed to one call at a time; at most kKept stay allocated
-// while unused (they are freed with the process).
-class Staging {
-public:
-    static constexpr size_t kBytes = 64 << 10;
-    static constexpr size_t kKept = 8;
-    Staging()
-    {
-        std::lock_guard<std::mutex> lock(mu());
-        if (!pool().empty()) {
-            p_ = pool().back();
-            pool().pop_back();
-        }
-        if (!p_ && cudaHostAlloc(&p_, kBytes, cudaHostAllocPortable) != cudaSuccess) {
-            p_ = nullptr;
-            cudaGetLastError();
-        }
-    }
-    ~Staging()
-    {
-        if (!p_) return;
-        {
-            std::lock_guard<std::mutex> lock(mu());
-            if (pool().size() < kKept) {
-                pool().push_back(p_);
-                return;
-            }
-        }
-        cudaFreeHost(p_);
-    }
-    Staging(const Staging &) = delete;
-    Staging &operator=(const Staging &) = delete;
-    char *data() const { return static_cast<char *>(p_); }
-
-private:
-    static std::mutex &mu()
-    {
-        static std::mutex m;
-        return m;
-    }
-    static std::vector<void *> &pool()
-    {
-        static auto *v = new std::vector<void *>;
-        return *v;
-    }
-    void *p_ = nullptr;
-};
-
 // Wait for the grid's queued work, report what its flags hold and bring
 // `count` floats from src to dst (NULL, 0: none).  The flags and the first
 // floats travel behind the work on the grid's stream, so the call waits once:
@@ -1570,7 +1590,9 @@ int finish(fdtd_grid *g, const float *src, size_t count, float *dst)
         if (e == cudaSuccess && head)
             e = cudaMemcpyAsync(st.data() + 64, src, head * sizeof(float), cudaMemcpyDeviceToHost, s);
     }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    // also after a failure: the staging block goes back with no copy in flight
+    const cudaError_t e_sync = cudaStreamSynchronize(s);
+    if (e == cudaSuccess) e = e_sync;
     if (e != cudaSuccess) return cuda_fail(g, e, "synchronize");
     auto clear = [&](int *dev) {
         cudaError_t c = cudaMemsetAsync(dev, 0, sizeof(int), s);
@@ -2482,6 +2504,7 @@ void fdtd_destroy(fdtd_grid *g)
 // over their z-layer planes when they have a CPML), then one source / probe
 // launch with a CTA per domain.  fdtd_batch_step replays a captured graph.
 struct fdtd_batch {
+    Staging::User staging_user;
     std::vector<fdtd_grid *> grids;
     cudaStream_t stream = nullptr;
     void *mem = nullptr;
@@ -2789,7 +2812,8 @@ int fdtd_batch_synchronize(fdtd_batch *b)
     const Staging st;
     int pageable = 0, *flag_h = st.data() ? reinterpret_cast<int *>(st.data()) : &pageable;
     cudaError_t e = cudaMemcpyAsync(flag_h, b->errf, sizeof(int), cudaMemcpyDeviceToHost, b->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+    const cudaError_t e_sync = cudaStreamSynchronize(b->stream);
+    if (e == cudaSuccess) e = e_sync;
     if (e != cudaSuccess) return bfail(b, FDTD_ECUDA, std::string("synchronize: ") + cudaGetErrorString(e));
     const int flag = *flag_h;
     if (flag) return bfail(b, FDTD_ETIMEOUT, "a bounded wait in the step kernel gave up");
