@@ -419,6 +419,17 @@ void fdtd_batch_destroy(fdtd_batch *b);
  * FDTD_ECUDA on a CUDA error.  The context stays usable afterwards. */
 int fdtd_selftest_wait(double seconds, void *cuda_stream);
 
+/* Self-test of a CTA leaving together (a library addition).  When a wait of
+ * the step kernel gives up, all consumer warps of its CTA must leave at the
+ * same barrier: one that went on would wait for the others without a limit.
+ * This call runs the routine that decides it in `ctas` CTAs (1..65535), each
+ * for at most `rounds` rounds (1..1000000), while a further warp raises the
+ * abort flag at some moment.  *spread receives the largest difference of the
+ * rounds after which two warps of a CTA left (0 as designed), *early the CTAs
+ * that left before their rounds were up.  Synchronises cuda_stream.
+ * FDTD_EINVAL for bad arguments, FDTD_ECUDA on a CUDA error. */
+int fdtd_selftest_leave(int ctas, int rounds, int *spread, int *early, void *cuda_stream);
+
 /* Checkpoint / resume of a finalized grid (a library addition; the paper's
  * solver has no counterpart).  The state is everything the step reads that
  * changes while stepping: the six fields, the twelve CPML auxiliaries (when

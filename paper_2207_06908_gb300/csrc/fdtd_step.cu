@@ -236,6 +236,7 @@ __global__ void wait_selftest_kernel(unsigned long long limit_ns, int *flag)
 }
 
 __device__ int g_selftest_flag;
+__device__ int g_selftest_leave[2];
 
 // box at (x, y, z) of every array of the map
 __device__ __forceinline__ void tma_load(uint32_t dst, const CUtensorMap *map, int x, int y, int z, uint32_t bar)
@@ -258,6 +259,55 @@ __device__ __forceinline__ bool elect_one()
 __device__ __forceinline__ void consumer_sync()
 {
     asm volatile("bar.sync 1, %0;" ::"n"(NCONS) : "memory");
+}
+
+// The same barrier, telling every consumer thread whether any of them gave p:
+// what they decide together (to leave a CTA whose waits gave up) comes out of
+// the barrier.  Each reading the abort flag for itself after a plain barrier
+// could differ, as the producer may set the flag between two warps' reads,
+// and the warps that stay would wait for those that left without a limit.
+__device__ __forceinline__ bool consumer_any(bool p)
+{
+    uint32_t any;
+    asm volatile(
+        "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.or.pred q, 1, %2, p;\n selp.u32 %0, 1, 0, q;\n}\n"
+        : "=r"(any)
+        : "r"((uint32_t)p), "n"(NCONS)
+        : "memory");
+    return any != 0;
+}
+
+// Self-test of leaving together: the consumer warps of a CTA go round
+// consumer_any on an abort flag that the warp after them sets at some moment,
+// or until `rounds` are up.  out[0]: the largest difference, over the CTAs, of
+// the rounds after which two warps left; out[1]: CTAs that left early.
+__global__ void __launch_bounds__(NCONS + 32) leave_selftest_kernel(int rounds, int *out)
+{
+    __shared__ int abort_flag, first, last;
+    if (threadIdx.x == 0) {
+        abort_flag = 0;
+        first = rounds;
+        last = 0;
+    }
+    __syncthreads();
+    volatile int *abort = &abort_flag;
+    if (threadIdx.x < NCONS) {
+        int r = 0;
+        while (r < rounds && !consumer_any(*abort != 0)) ++r;
+        if ((threadIdx.x & 31) == 0) {
+            atomicMin(&first, r);
+            atomicMax(&last, r);
+        }
+    } else if (threadIdx.x == NCONS) {
+        const unsigned long long t0 = gtimer(), t = 1000ull + 37ull * blockIdx.x;
+        while (gtimer() - t0 < t) {}
+        *abort = 1;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        atomicMax(out, last - first);
+        if (last < rounds) atomicAdd(out + 1, 1);
+    }
 }
 
 // ---- stencil cores ----------------------------------------------------------
@@ -995,8 +1045,7 @@ __device__ __forceinline__ void consume(const Cons<NH> &C, const BatchArgs &B, S
     while (true) {
         // first plane of the next item (or the end marker)
         if (!mbar_wait(C.fullE(R.e), R.ep, C.abort)) *C.abort = 1;
-        consumer_sync();
-        if (*C.abort) break;
+        if (consumer_any(*C.abort != 0)) break;
         ce += item_e;
         ch += max(item_e, 1u) - 1;
         const int *hdr = C.ev(R.e).hdr();
@@ -1020,8 +1069,7 @@ __device__ __forceinline__ void consume(const Cons<NH> &C, const BatchArgs &B, S
         if (layer) fill_xc(a, C.prof, C.xc, it.x0, tid);
         const uint32_t n = R.e_next();
         if (!mbar_wait(C.fullE(n), R.ep ^ (n == 0), C.abort)) *C.abort = 1;
-        consumer_sync();
-        if (*C.abort) break;
+        if (consumer_any(*C.abort != 0)) break;
         if constexpr (ROWS) {
             // the layers its own cells meet (its planes: all or none of them)
             const int d = a.d;
@@ -1355,4 +1403,23 @@ extern "C" int fdtd_selftest_wait(double seconds, void *cuda_stream)
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return FDTD_ECUDA;
     return v == 1 ? FDTD_ETIMEOUT : (v == 2 ? FDTD_OK : FDTD_ECUDA);
+}
+
+extern "C" int fdtd_selftest_leave(int ctas, int rounds, int *spread, int *early, void *cuda_stream)
+{
+    if (ctas < 1 || ctas > 65535 || rounds < 1 || rounds > 1000000 || !spread || !early) return FDTD_EINVAL;
+    int *out = nullptr;
+    cudaError_t e = cudaGetSymbolAddress(reinterpret_cast<void **>(&out), fdtd::g_selftest_leave);
+    cudaStream_t s = (cudaStream_t)cuda_stream;
+    if (e == cudaSuccess) e = cudaMemsetAsync(out, 0, 2 * sizeof(int), s);
+    if (e == cudaSuccess) {
+        fdtd::leave_selftest_kernel<<<ctas, fdtd::NCONS + 32, 0, s>>>(rounds, out);
+        e = cudaGetLastError();
+    }
+    int v[2] = {0, 0};
+    if (e == cudaSuccess) e = cudaMemcpyAsync(v, out, sizeof v, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    *spread = v[0];
+    *early = v[1];
+    return e == cudaSuccess ? FDTD_OK : FDTD_ECUDA;
 }
