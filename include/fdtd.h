@@ -430,6 +430,14 @@ int fdtd_selftest_wait(double seconds, void *cuda_stream);
  * FDTD_EINVAL for bad arguments, FDTD_ECUDA on a CUDA error. */
 int fdtd_selftest_leave(int ctas, int rounds, int *spread, int *early, void *cuda_stream);
 
+/* Self-test of the step kernel's register split (host arithmetic only).  Its
+ * row warps take registers that its other warps give back; a launch with too
+ * few would wait for them without a limit, so grids and batches are checked
+ * against the compiled kernel when they are set up (FDTD_ECUDA).  FDTD_OK if
+ * a kernel compiled for `regs` registers a thread passes that check,
+ * FDTD_ECUDA if not, FDTD_EINVAL outside 1..255. */
+int fdtd_selftest_registers(int regs);
+
 /* Checkpoint / resume of a finalized grid (a library addition; the paper's
  * solver has no counterpart).  The state is everything the step reads that
  * changes while stepping: the six fields, the twelve CPML auxiliaries (when

@@ -88,6 +88,7 @@ def load():
             "fdtd_batch_destroy": (None, [P]),
             "fdtd_selftest_wait": (I, [ctypes.c_double, P]),
             "fdtd_selftest_leave": (I, [I, I, ip, ip, P]),
+            "fdtd_selftest_registers": (I, [I]),
             "fdtd_set_debye": (I, [P, I, I, P, P]),
             "fdtd_add_voltage_source": (I, [P, I, I, I, I, ctypes.c_double, P, I, P]),
             "fdtd_add_lumped": (I, [P, I, I, I, I, ctypes.c_double, ctypes.c_double, P]),

@@ -308,6 +308,9 @@ PsiGeom step_psi_geom(int d, int nx, int ny);
 // (zxy = 0) or z together with the x / y layers (zxy = 1)
 void step_region(const PsiGeom &pg, int zxy, int *region, int *ox, int *oy);
 const void *step_kernel_ptr(int launch, int nh, bool batch);
+// whether the kernel was compiled for as many registers as its roles share
+// (before its first launch; cudaErrorLaunchOutOfResources if not)
+cudaError_t check_step_kernel(int launch, int nh, bool batch);
 // fdtd_edges.cu
 cudaError_t launch_edges(const EdgeArgs &a, cudaStream_t s);
 // oblique wires: segment currents to t_{n+1/2}; needs only the step's inputs,

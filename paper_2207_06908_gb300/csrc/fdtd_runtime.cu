@@ -1432,8 +1432,10 @@ int setup_step_kernel(fdtd_grid *g)
         max_smem = std::max(max_smem, fdtd::step_smem_bytes(g->n_classes, d, L.region, L.nh));
         g->n_launch = l + 1;
     }
-    for (int q = 0; q < 4 && e == cudaSuccess; ++q)
-        e = ensure_smem(fdtd::step_kernel_ptr(q >> 1, 2 + (q & 1), false), max_smem);
+    for (int q = 0; q < 4 && e == cudaSuccess; ++q) {
+        e = fdtd::check_step_kernel(q >> 1, 2 + (q & 1), false);
+        if (e == cudaSuccess) e = ensure_smem(fdtd::step_kernel_ptr(q >> 1, 2 + (q & 1), false), max_smem);
+    }
     if (e != cudaSuccess) return cuda_fail(g, e, "step kernel setup");
     int occ[2] = {1, 1};
     for (int l = 0; l < g->n_launch; ++l) {
@@ -2668,8 +2670,10 @@ int fdtd_batch_create(int n, fdtd_grid *const *grids, void *cuda_stream, fdtd_ba
             b->nh[l] = 2;
         max_smem = std::max(max_smem, fdtd::step_smem_bytes(b->max_classes, b->max_d, b->region[l], b->nh[l]));
     }
-    for (int q = 0; q < 4 && e == cudaSuccess; ++q)
-        e = ensure_smem(fdtd::step_kernel_ptr(q >> 1, 2 + (q & 1), true), max_smem);
+    for (int q = 0; q < 4 && e == cudaSuccess; ++q) {
+        e = fdtd::check_step_kernel(q >> 1, 2 + (q & 1), true);
+        if (e == cudaSuccess) e = ensure_smem(fdtd::step_kernel_ptr(q >> 1, 2 + (q & 1), true), max_smem);
+    }
     int occ[2] = {1, 1};
     for (int l = 0; l < b->n_launch && e == cudaSuccess; ++l) {
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(

@@ -1378,6 +1378,20 @@ static StepKernel step_kernel(int l, int nh, bool batch)
 }
 const void *step_kernel_ptr(int l, int nh, bool batch) { return (const void *)step_kernel(l, nh, batch); }
 
+// A launch with `regs` registers a thread holds both roles' shares: a
+// setmaxnreg.inc beyond what the launch was given would wait without a limit.
+static bool split_fits(int regs, bool batch)
+{
+    return (NCW + 4) * regs >= NCW * row_regs(batch) + 4 * aux_regs(batch);
+}
+cudaError_t check_step_kernel(int l, int nh, bool batch)
+{
+    cudaFuncAttributes at;
+    const cudaError_t e = cudaFuncGetAttributes(&at, step_kernel_ptr(l, nh, batch));
+    if (e != cudaSuccess) return e;
+    return split_fits(at.numRegs, batch) ? cudaSuccess : cudaErrorLaunchOutOfResources;
+}
+
 cudaError_t launch_step(const SingleArgs &one, const BatchArgs &b, int grid, cudaStream_t s)
 {
     const int smem = smem_bytes(b.max_classes, b.max_d, b.region, b.nh);
@@ -1422,4 +1436,10 @@ extern "C" int fdtd_selftest_leave(int ctas, int rounds, int *spread, int *early
     *spread = v[0];
     *early = v[1];
     return e == cudaSuccess ? FDTD_OK : FDTD_ECUDA;
+}
+
+extern "C" int fdtd_selftest_registers(int regs)
+{
+    if (regs < 1 || regs > 255) return FDTD_EINVAL;
+    return fdtd::split_fits(regs, false) && fdtd::split_fits(regs, true) ? FDTD_OK : FDTD_ECUDA;
 }
