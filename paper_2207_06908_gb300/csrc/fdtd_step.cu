@@ -138,9 +138,9 @@ constexpr int HNEW_PLANE = HBY * HBX;
 constexpr int HNEW_BYTES = 2 * 3 * HNEW_PLANE * 4;     // [2][3][HBY][HBX]
 constexpr int NBAR = 2 * NE + 2 * NH_MAX;             // fullE, emptyE, fullH, emptyH
 // x-layer coefficients of the current item's columns: {b, c, 1/kappa} at E,
-// then at H positions, TX floats each (identity outside the layer), an
-// identity profile row and three zero coefficient rows
-constexpr int XC_BYTES = (6 * TX + 4 + 12) * 4;
+// then at H positions, TX floats each (zero outside the layer, where nothing
+// uses them), and three zero coefficient rows
+constexpr int XC_BYTES = (6 * TX + 12) * 4;
 struct Layout {
     int hslot, hnew, xc, bar, misc, tab;
     __host__ __device__ Layout(int region, int nh)
@@ -394,7 +394,7 @@ __device__ __forceinline__ void h_core(const StepArgs &a, const float4 *t, const
 // with another, the index arithmetic and the barriers are paid once per two
 // cells, and the differences and layer sums run two cells to an instruction
 // (packed FP32 pairs).  The layers an item meets are template arguments and
-// the lanes outside them run along with identity coefficients, so the plane
+// the lanes outside them run along and leave out the last sum, so the plane
 // loop has no branches to wait on.  Every sum is written as explicit products
 // and fused multiply-adds, so every instantiation of the kernel rounds alike.
 using F2 = unsigned long long;           // two FP32 values
@@ -447,8 +447,8 @@ struct Pair {
                              // YM: the row lies in a y layer
     int xo;                  // float offset of the first cell's entry in the first x box
     int yo;                  // float offset of the pair in the first y box (of the lane's column, outside the layer)
-    const float4 *py;        // its y profile row at E positions (the identity outside the layer)
-    int ph;                  // rows from there to the one at H positions
+    const float4 *py;        // its y profile row at E positions, 2d rows before the one at H positions
+                             // (outside the layer: any)
     unsigned off;            // its element in a plane of the fields and z auxiliaries
     int xoff, yoff;          // of the x, y auxiliaries (a lane outside the layer: not used)
 };
@@ -473,6 +473,35 @@ __device__ __forceinline__ F2 cpmlx(F2 &dif, const PX &q, F2 o)
     const F2 p = fma2(q.b, o, mul2(q.c, dif));
     dif = fma2(dif, q.ki, p);
     return p;
+}
+// The same for a lane that may lie outside the layer (in: inside); outside,
+// the difference stays as it is.  Coefficients of zero and one would not do
+// that: times an infinite difference, or an infinite auxiliary of the row
+// that a lane outside the layer reads, zero is a NaN.  Written so it costs
+// -0.3 to 0.6 % (20 steps of 256^3 with 10 cells 3338 -> 3336 us, 32 of
+// 160x160x200 2345 -> 2357); selects or inline PTX predicates spilled (1 to 4 %).
+__device__ __forceinline__ F2 cpmlx(F2 &dif, const PX &q, F2 o, bool in)
+{
+    const F2 p = fma2(q.b, o, mul2(q.c, dif));
+    if (in) dif = fma2(dif, q.ki, p);
+    return p;
+}
+// both differences of a pair cut by the layer: in0, in1 for its two cells
+__device__ __forceinline__ void cpmlx_cut(F2 &d0, F2 &d1, const PX &q, F2 o0, F2 o1, bool in0, bool in1, F2 &p0, F2 &p1)
+{
+    p0 = fma2(q.b, o0, mul2(q.c, d0));
+    p1 = fma2(q.b, o1, mul2(q.c, d1));
+    float l0 = lo2(d0), h0 = hi2(d0), l1 = lo2(d1), h1 = hi2(d1);
+    if (in0) {
+        l0 = __fmaf_rn(l0, lo2(q.ki), lo2(p0));
+        l1 = __fmaf_rn(l1, lo2(q.ki), lo2(p1));
+    }
+    if (in1) {
+        h0 = __fmaf_rn(h0, hi2(q.ki), hi2(p0));
+        h1 = __fmaf_rn(h1, hi2(q.ki), hi2(p1));
+    }
+    d0 = pk(l0, h0);
+    d1 = pk(l1, h1);
 }
 
 // Both differences of the x layer at E (h = 0) or H (h = 1) positions.  VEC:
@@ -506,7 +535,13 @@ __device__ __forceinline__ void cpml_x(const StepArgs &a, const Pair &G, const P
         o0 = pk(f[0], f[2]);
         o1 = pk(f[1], f[3]);
     }
-    const F2 p0 = cpmlx(d0, pr, o0), p1 = cpmlx(d1, pr, o1);
+    F2 p0, p1;
+    if (VEC) {
+        p0 = cpmlx(d0, pr, o0, G.fl & XM);
+        p1 = cpmlx(d1, pr, o1, G.fl & XM);
+    } else {
+        cpmlx_cut(d0, d1, pr, o0, o1, G.fl & XM0, G.fl & XM1, p0, p1);
+    }
     const int pl = k * (a.ny * a.px);
     float *u0 = a.psi_out[h ? PSI_HY_X : PSI_EY_X], *u1 = a.psi_out[h ? PSI_HZ_X : PSI_EZ_X];
     const long long n = psi_n(a, 0);
@@ -531,8 +566,8 @@ __device__ __forceinline__ void cpml_y(const StepArgs &a, const Pair &G, const P
 {
     const int q = a.pg.yb >> 2, at = h ? 0 : 2;
     const float *b = P.base + G.yo + at * q;
-    const PX pr = profx(G.py[h ? G.ph : 0]);
-    const F2 p0 = cpmlx(d0, pr, ld2(b)), p1 = cpmlx(d1, pr, ld2(b + q));
+    const PX pr = profx(G.py[h ? 2 * a.d : 0]);
+    const F2 p0 = cpmlx(d0, pr, ld2(b), G.fl & YM), p1 = cpmlx(d1, pr, ld2(b + q), G.fl & YM);
     const int pl = k * (2 * a.d * a.pitch);
     put2(a.psi_out[h ? PSI_HX_Y : PSI_EX_Y], pl, G.yoff, p0, G.fl & YM, psi_n(a, 1), 3, a.bounds);
     put2(a.psi_out[h ? PSI_HZ_Y : PSI_EZ_Y], pl, G.yoff, p1, G.fl & YM, psi_n(a, 1), 3, a.bounds);
@@ -591,10 +626,11 @@ __device__ __forceinline__ void h_belowx(const StepArgs &a, const Pair &G, const
         F2 o;
         if (f & F_X) o = pk(G.fl & XM0 ? P.base[G.xo] : 0.f, G.fl & XM1 ? P.base[G.xo + 1] : 0.f);
         else o = far(a.psi_in[PSI_HY_X], gx, (G.fl & XM) / XM0, 0);
-        cpmlx(hy_x, profx(P.xc + 3 * TX), o);
+        F2 none = 0, p0, p1;
+        cpmlx_cut(hy_x, none, profx(P.xc + 3 * TX), o, none, G.fl & XM0, G.fl & XM1, p0, p1);
     }
     if (G.fl & YM)
-        cpmlx(hx_y, profx(G.py[G.ph]), (f & F_Y) ? ld2(P.base + G.yo) : far(a.psi_in[PSI_HX_Y], gy, G.fl & 3, 1));
+        cpmlx(hx_y, profx(G.py[2 * a.d]), (f & F_Y) ? ld2(P.base + G.yo) : far(a.psi_in[PSI_HX_Y], gy, G.fl & 3, 1));
     if (P.sz >= 0) {
         const PX q = profx(prow(prof, 2, 1, 2 * a.d)[P.sz]);
         cpmlx(hx_z, q, ld2(P.base + P.zo));
@@ -852,8 +888,7 @@ __device__ __forceinline__ void run_rows(const Cons<NH> &C, const Item &it, Ring
     G.fl = (1 << nv) - 1;
     G.xo = 0;
     G.yo = 0;
-    G.py = reinterpret_cast<const float4 *>(C.xc + 6 * TX);      // the identity
-    G.ph = 0;
+    G.py = reinterpret_cast<const float4 *>(C.prof);
     // slab entry of the pair's first cell, in the layer its members lie in, and of its row
     const int xe = i < d ? i : i - (a.nx - 2 * d), sy = d > 0 && nv > 0 ? slab_of(j, a.ny, d) : -1;
     if (d > 0) {
@@ -867,14 +902,13 @@ __device__ __forceinline__ void run_rows(const Cons<NH> &C, const Item &it, Ring
         if (sy >= 0) {
             G.fl |= YM;
             G.py = prow(C.prof, 1, 0, 2 * d) + sy;
-            G.ph = 2 * d;
         }
     }
     G.off = (unsigned)j * a.pitch + i;
     G.xoff = j * a.px + xe;
     G.yoff = sy * a.pitch + i;
     // coefficient rows of the pair's cells (a second cell outside the grid: zeros)
-    const float4 *const zero = reinterpret_cast<const float4 *>(C.xc + 6 * TX + 4);
+    const float4 *const zero = reinterpret_cast<const float4 *>(C.xc + 6 * TX);
     auto row0 = [&](uint32_t cls) { return reinterpret_cast<const float4 *>(C.tab + (cls & 255u) * kTabStride); };
     auto row1 = [&](uint32_t cls) {
         return (G.fl & 3) == IN0 ? zero : reinterpret_cast<const float4 *>(C.tab + (cls >> 8) * kTabStride);
@@ -1010,14 +1044,13 @@ __device__ __forceinline__ void run_halo(const Cons<NH> &C, const Item &it, Ring
     R.pass_e();
 }
 
-// the x-layer coefficients of an item's columns (identity outside the layer
-// and the grid), one value per consumer thread
+// the x-layer coefficients of an item's columns, one value per consumer thread
 __device__ __forceinline__ void fill_xc(const StepArgs &a, const float *prof, float *xc, int x0, int tid)
 {
     for (int q = tid; q < 6 * TX; q += NCONS) {
         const int w = q / TX, i = x0 + q - w * TX, half = w / 3, comp = w - 3 * half;
         const int s = i < a.nx ? slab_of(i, a.nx, a.d) : -1;
-        xc[q] = s >= 0 ? prof[((half * 2 * a.d + s) << 2) + comp] : (comp == 2 ? 1.f : 0.f);
+        xc[q] = s >= 0 ? prof[((half * 2 * a.d + s) << 2) + comp] : 0.f;
     }
 }
 
@@ -1150,7 +1183,7 @@ __global__ void __launch_bounds__(NTHREADS, 2) step_tma_kernel(const __grid_cons
             }
         }
     }
-    if (threadIdx.x < 16) xc[6 * TX + threadIdx.x] = threadIdx.x == 2 ? 1.f : 0.f;
+    if (threadIdx.x < 12) xc[6 * TX + threadIdx.x] = 0.f;
     if (threadIdx.x == 0) {
         for (int q = 0; q < NE; ++q) {
             mbar_init(C.fullE(q), 1);
