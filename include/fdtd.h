@@ -308,7 +308,8 @@ int fdtd_finalize(fdtd_grid *g, int probe_capacity, void *arena, size_t arena_by
 
 /* Queue n full time steps (H to n+1/2, E to n+1 with the sources, probes)
  * on the grid's stream: replays of captured CUDA graphs of 32, 16, 8, 4 and
- * 2 steps (each captured on first use), a lone step launched directly.
+ * 2 steps, a lone step launched directly.  The first call that replays one
+ * captures all five, those it does not replay after its steps are queued.
  * Returns launch errors only; does not synchronise. */
 int fdtd_step(fdtd_grid *g, int n);
 
@@ -379,7 +380,7 @@ int fdtd_field_device(fdtd_grid *g, int component, void **dptr, int *row_pitch,
  * charges); when a domain has oblique wires, a launch with a CTA per domain
  * takes their segment currents to t_{n+1/2} beside the step kernel.
  * fdtd_batch_step replays captured CUDA graphs of 32, 16, 8, 4 and 2
- * steps (each captured on first use) and launches a lone step directly.
+ * steps (captured as fdtd_step's are) and launches a lone step directly.
  * The results are those of stepping each grid alone with fdtd_step. */
 typedef struct fdtd_batch fdtd_batch;
 

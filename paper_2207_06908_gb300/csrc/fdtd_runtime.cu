@@ -1505,22 +1505,23 @@ cudaError_t make_programmatic(cudaGraph_t graph) try
     return cudaErrorMemoryAllocation;
 }
 
-// Which graphs of 2^k steps (bit k, k = 1 .. 5) a call with n steps left
-// captures when it lacks one: up to 31 steps those of 2 to 16, so that the
-// next short call finds its own; from 32 on those it replays.  (All five at
-// once are 62 steps: 1.4 ms on a grid with a CPML and probes.)
-int graphs_for(int n) { return n < 32 ? 0x1e : 0x20 | (n & 0x1e); }
+// Graphs of 2^k steps (bit k, k = 1 .. 5).  A call with n steps left that
+// lacks one it replays captures those it replays, queues them, and captures
+// the others while they run, so no later call pays a capture and the first
+// one's steps do not wait for all five (62 steps: 1.4 ms on a grid with a
+// CPML and probes).
+constexpr int kAllGraphs = 0x3e;
+int graphs_for(int n) { return (n >= 32 ? 0x20 : 0) | (n & 0x1e); }
 
-// Capture the graphs of 2, 4, 8, 16 and 32 steps from parity 0 that a call
-// with n steps left needs
-int capture_graphs(fdtd_grid *g, int n)
+// Capture those graphs of mask, from parity 0, that the grid lacks
+int capture_graphs(fdtd_grid *g, int mask)
 {
     nvtxRangePushA("fdtd_step graph capture");
     cudaError_t e = cudaSuccess;
     if (!g->cap_stream) e = cudaStreamCreateWithFlags(&g->cap_stream, cudaStreamNonBlocking);
     for (int k = 1; k <= 5 && e == cudaSuccess; ++k) {
         const int len = 1 << k;
-        if (g->graph[k] || !(graphs_for(n) >> k & 1)) continue;
+        if (g->graph[k] || !(mask >> k & 1)) continue;
         cudaGraph_t graph = nullptr;
         e = cudaStreamBeginCapture(g->cap_stream, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
@@ -1543,14 +1544,17 @@ int capture_graphs(fdtd_grid *g, int n)
 // period
 int step_queue(fdtd_grid *g, int n)
 {
+    bool captured = false;
     while (n > 0) {
         const long before = g->step;
         if (g->parity == 0 && n >= 2) {
             int k = 1;
             while (k < 5 && (2 << k) <= n) ++k;          // largest 2^k <= min(n, 32)
             const int len = 1 << k;
-            if (!g->graph[k])
-                if (int rc = capture_graphs(g, n)) return rc;
+            if (!g->graph[k]) {
+                if (int rc = capture_graphs(g, graphs_for(n))) return rc;
+                captured = true;
+            }
             cudaError_t e = cudaGraphLaunch(g->graph[k], g->stream);
             if (e != cudaSuccess) return cuda_fail(g, e, "graph launch");
             n -= len;
@@ -1567,6 +1571,9 @@ int step_queue(fdtd_grid *g, int n)
             if (e != cudaSuccess) return cuda_fail(g, e, "watchdog launch");
         }
     }
+    // the steps are queued: a capture that fails here is reported by the call
+    // that needs it
+    if (captured && capture_graphs(g, kAllGraphs)) cudaGetLastError();
     return FDTD_OK;
 }
 
@@ -2578,36 +2585,45 @@ cudaError_t batch_enqueue(fdtd_batch *b, int parity, cudaStream_t s)
     return e;
 }
 
-// n batch steps: graph replays of 32, 16, 8, 4 or 2 steps (each captured
-// once, from parity 0) while the parity allows, direct launches otherwise
+// Capture those batch graphs of mask, from parity 0, that are missing
+cudaError_t batch_capture(fdtd_batch *b, int mask)
+{
+    nvtxRangePushA("fdtd_batch_step graph capture");
+    cudaError_t e = cudaSuccess;
+    if (!b->cap) e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
+    for (int k = 1; k <= 5 && e == cudaSuccess; ++k) {
+        if (b->graph[k] || !(mask >> k & 1)) continue;
+        cudaGraph_t graph = nullptr;
+        e = cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal);
+        if (e == cudaSuccess) {
+            for (int t = 0; t < (1 << k) && e == cudaSuccess; ++t) e = batch_enqueue(b, t & 1, b->cap);
+            cudaError_t e2 = cudaStreamEndCapture(b->cap, &graph);
+            if (e == cudaSuccess) e = e2;
+        }
+        if (e == cudaSuccess) e = make_programmatic(graph);
+        if (e == cudaSuccess) e = cudaGraphInstantiate(&b->graph[k], graph, 0);
+        if (graph) cudaGraphDestroy(graph);
+        if (e != cudaSuccess) b->graph[k] = nullptr;
+    }
+    nvtxRangePop();
+    return e;
+}
+
+// n batch steps: graph replays of 32, 16, 8, 4 or 2 steps (captured as a
+// grid's are) while the parity allows, direct launches otherwise
 int batch_queue(fdtd_batch *b, int n)
 {
     const int n0 = n;
+    bool captured = false;
     while (n > 0) {
         if (b->parity == 0 && n >= 2) {
             int k = 1;
             while (k < 5 && (2 << k) <= n) ++k;
             const int len = 1 << k;
             if (!b->graph[k]) {
-                nvtxRangePushA("fdtd_batch_step graph capture");
-                cudaError_t e = cudaSuccess;
-                if (!b->cap) e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
-                for (int kk = 1; kk <= 5 && e == cudaSuccess; ++kk) {
-                    if (b->graph[kk] || !(graphs_for(n) >> kk & 1)) continue;
-                    cudaGraph_t graph = nullptr;
-                    e = cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal);
-                    if (e == cudaSuccess) {
-                        for (int t = 0; t < (1 << kk) && e == cudaSuccess; ++t) e = batch_enqueue(b, t & 1, b->cap);
-                        cudaError_t e2 = cudaStreamEndCapture(b->cap, &graph);
-                        if (e == cudaSuccess) e = e2;
-                    }
-                    if (e == cudaSuccess) e = make_programmatic(graph);
-                    if (e == cudaSuccess) e = cudaGraphInstantiate(&b->graph[kk], graph, 0);
-                    if (graph) cudaGraphDestroy(graph);
-                    if (e != cudaSuccess) b->graph[kk] = nullptr;
-                }
-                nvtxRangePop();
+                const cudaError_t e = batch_capture(b, graphs_for(n));
                 if (e != cudaSuccess) return bfail(b, FDTD_ECUDA, std::string("graph capture: ") + cudaGetErrorString(e));
+                captured = true;
             }
             cudaError_t e = cudaGraphLaunch(b->graph[k], b->stream);
             if (e != cudaSuccess) return bfail(b, FDTD_ECUDA, std::string("graph launch: ") + cudaGetErrorString(e));
@@ -2624,6 +2640,7 @@ int batch_queue(fdtd_batch *b, int n)
         g->parity = b->parity;
         g->step = b->step;
     }
+    if (captured && batch_capture(b, kAllGraphs) != cudaSuccess) cudaGetLastError();
     return FDTD_OK;
 }
 
