@@ -302,6 +302,9 @@ int fdtd_arena_bytes(const fdtd_grid *g, int probe_capacity, size_t *bytes);
  * not recorded).  arena: device memory of at least fdtd_arena_bytes()
  * bytes, 256-byte aligned, owned by the caller and kept alive until
  * fdtd_destroy(); NULL makes the library allocate (and free) its own.
+ * Page-locks 64 KB of host memory for read-backs, at most 512 KB for all
+ * grids and batches of the process; the last of them to be destroyed gives
+ * it back.  The calls that read back allocate none.
  * Fails with FDTD_ECLASSES if more than 256 distinct coefficient sets
  * occur. */
 int fdtd_finalize(fdtd_grid *g, int probe_capacity, void *arena, size_t arena_bytes);
@@ -330,7 +333,8 @@ int fdtd_synchronize(fdtd_grid *g);
  * a caller hands fdtd_finalize() an arena it obtained elsewhere and steps
  * with this function, which calls no cudaMalloc, cudaFree or other
  * allocating routine and never builds a CUDA graph: it queues plain kernel
- * launches (and one cudaMemsetAsync) on the grid's stream.
+ * launches (and one cudaMemsetAsync) on the grid's stream.  Waiting with
+ * fdtd_synchronize() and reading probes allocate nothing either.
  *
  * The step kernel's scratch -- two work-distribution counters per launch and
  * the flag of a bounded wait that gave up, at most 5 ints today -- lives in

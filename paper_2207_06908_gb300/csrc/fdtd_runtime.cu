@@ -108,61 +108,68 @@ struct Fork {
 };
 
 // Page-locked staging blocks for small read-backs, shared by every grid and
-// batch of the process and handed to one call at a time.  At most kKept stay
-// allocated while unused, and only while a grid or batch lives (each holds a
-// User): the last one gives them back.
+// batch of the process and handed to one call at a time.  Each finalized grid
+// and batch adds one when it is set up, up to kMax in all; the last to go
+// gives them back.  A call never page-locks memory itself (it may be a loop
+// that cannot afford that): one that finds every block in use gets none.
 class Staging {
 public:
     static constexpr size_t kBytes = 64 << 10;
     Staging()
     {
-        {
-            std::lock_guard<std::mutex> lock(pool().mu);
-            if (pool().n) p_ = pool().kept[--pool().n];
-        }
-        if (!p_ && cudaHostAlloc(&p_, kBytes, cudaHostAllocPortable) != cudaSuccess) {
-            p_ = nullptr;
-            cudaGetLastError();
-        }
+        std::lock_guard<std::mutex> lock(pool().mu);
+        if (pool().n) p_ = pool().free[--pool().n];
     }
     ~Staging()
     {
         if (!p_) return;
-        {
-            std::lock_guard<std::mutex> lock(pool().mu);
-            if (pool().n < kKept) {
-                pool().kept[pool().n++] = p_;
-                return;
-            }
-        }
-        cudaFreeHost(p_);
+        std::lock_guard<std::mutex> lock(pool().mu);
+        pool().free[pool().n++] = p_;
     }
     Staging(const Staging &) = delete;
     Staging &operator=(const Staging &) = delete;
     char *data() const { return static_cast<char *>(p_); }
 
-    struct User {
-        User()
+    class User {
+    public:
+        User() = default;
+        // before the grid's or batch's first read-back
+        void add()
         {
+            if (added_) return;
+            added_ = true;
             std::lock_guard<std::mutex> lock(pool().mu);
             ++pool().users;
+            void *p = nullptr;
+            if (pool().total == kMax) return;
+            if (cudaHostAlloc(&p, kBytes, cudaHostAllocPortable) != cudaSuccess) {
+                cudaGetLastError();
+                return;
+            }
+            pool().free[pool().n++] = p;
+            ++pool().total;
         }
         ~User()
         {
+            if (!added_) return;
             std::lock_guard<std::mutex> lock(pool().mu);
             if (--pool().users) return;
-            while (pool().n) cudaFreeHost(pool().kept[--pool().n]);
+            while (pool().n) cudaFreeHost(pool().free[--pool().n]);
+            pool().total = 0;
         }
         User(const User &) = delete;
         User &operator=(const User &) = delete;
+
+    private:
+        bool added_ = false;
     };
 
 private:
-    static constexpr int kKept = 8;
+    static constexpr int kMax = 8;
     struct Pool {
         std::mutex mu;
-        void *kept[kKept];
-        int n, users;
+        void *free[kMax];
+        int n, total, users;
     };
     static Pool &pool()
     {
@@ -2117,6 +2124,7 @@ int fdtd_finalize(fdtd_grid *g, int probe_capacity, void *arena, size_t arena_by
         g->own_arena = true;
     }
     g->arena_bytes = p.total;
+    g->staging_user.add();
     char *base = (char *)g->arena;
     const size_t cells = (size_t)g->plane * g->nz;
     for (int b = 0; b < 2; ++b)
@@ -2655,6 +2663,7 @@ int fdtd_batch_create(int n, fdtd_grid *const *grids, void *cuda_stream, fdtd_ba
     fdtd_batch *b = new (std::nothrow) fdtd_batch();
     if (!b) return FDTD_ENOMEM;
     b->stream = (cudaStream_t)cuda_stream;
+    b->staging_user.add();
     for (int q = 0; q < n; ++q) {
         fdtd_grid *g = grids[q];
         if (!g || !g->finalized) { delete b; return FDTD_ESTATE; }
