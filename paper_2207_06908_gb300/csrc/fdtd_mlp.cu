@@ -19,9 +19,7 @@
 
 #include <algorithm>
 #include <cstdint>
-#include <map>
 #include <mutex>
-#include <utility>
 
 #include "fdtd.h"
 #include "fdtd_mlp.h"
@@ -791,20 +789,30 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 
 static_assert(TC_THREADS / 32 * 32 * TC_TS * 4 <= (TC_M + TC_N) * GC_K * 2, "transpose buffers fit the tile area");
 
-// raise a kernel's dynamic shared-memory limit once per device
+// Raise a kernel's dynamic shared-memory limit once per device.  Nothing is
+// allocated (a C entry calls this): past the table's end the limit is set on
+// every call.
 cudaError_t allow_smem(const void *kernel, int bytes)
 {
     static std::mutex mu;
-    static std::map<std::pair<int, const void *>, int> set;
+    static struct {
+        int dev;
+        const void *kernel;
+        int bytes;
+    } set[128];
+    static int n = 0;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     std::lock_guard<std::mutex> lock(mu);
-    int &cur = set[{dev, kernel}];
-    if (cur >= bytes) return cudaSuccess;
+    int q = 0;
+    while (q < n && (set[q].dev != dev || set[q].kernel != kernel)) ++q;
+    if (q < n && set[q].bytes >= bytes) return cudaSuccess;
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess) cur = bytes;
-    return e;
+    if (e != cudaSuccess || q == 128) return e;
+    set[q] = {dev, kernel, bytes};
+    n = std::max(n, q + 1);
+    return cudaSuccess;
 }
 
 // a launch in clusters of cx x cy CTAs
