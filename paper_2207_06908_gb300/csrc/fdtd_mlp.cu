@@ -513,20 +513,15 @@ constexpr int GC_K = 128;
 constexpr int GC_SMEM = 1024 + 1024 + (TC_M + TC_N) * GC_K * 2;
 constexpr int GC_SPLIT = 8;          // CTAs of a cluster that share a tile's reduction, at most
 
-template <typename T>
-__device__ __forceinline__ float elem(const T *p)
-{
-    if constexpr (sizeof(T) == 2) return __bfloat162float(*reinterpret_cast<const __nv_bfloat16 *>(p));
-    else return *reinterpret_cast<const float *>(p);
-}
-
 // A chunk of one operand, this thread's share: rows r0 .. r0 + R - 1 and
 // reduction indices k0 .. k0 + GC_K - 1 of X(row, k) = X[row s_row + k s_k],
-// zero outside rows x kend, in groups of 8 along k
+// zero outside rows x kend, in groups of 8 along k.  BF16 elements wait as
+// they are, two to a register.
 template <typename T, int R>
 struct Chunk {
     static constexpr int KGS = GC_K / 8, G = R * KGS / TC_THREADS;
-    float f[G][8];
+    static constexpr bool HALF = sizeof(T) == 2;
+    uint32_t f[G][HALF ? 4 : 8];
     __device__ __forceinline__ static void place(int u, int tid, bool row_fast, int &r, int &g)
     {
         const int q = tid + u * TC_THREADS;
@@ -544,11 +539,19 @@ struct Chunk {
             place(u, tid, s_row == 1, r, g);
             const int row = r0 + r, k = k0 + g * 8;
             const T *p = X + row * s_row + (long long)k * s_k;
-            if (sizeof(T) == 4 && vec) {
+            if constexpr (HALF) {
+                const unsigned short *h = reinterpret_cast<const unsigned short *>(p);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const uint32_t lo = (row < rows && k + 2 * j < kend) ? h[2 * j * s_k] : 0u;
+                    const uint32_t hi = (row < rows && k + 2 * j + 1 < kend) ? h[(2 * j + 1) * s_k] : 0u;
+                    f[u][j] = lo | hi << 16;
+                }
+            } else if (vec) {
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (row < rows && k + 4 * h < kend) v = __ldg(reinterpret_cast<const float4 *>(p) + h);
+                    uint4 v = make_uint4(0, 0, 0, 0);
+                    if (row < rows && k + 4 * h < kend) v = __ldg(reinterpret_cast<const uint4 *>(p) + h);
                     f[u][4 * h] = v.x;
                     f[u][4 * h + 1] = v.y;
                     f[u][4 * h + 2] = v.z;
@@ -556,7 +559,8 @@ struct Chunk {
                 }
             } else {
 #pragma unroll
-                for (int j = 0; j < 8; ++j) f[u][j] = (row < rows && k + j < kend) ? elem(p + j * s_k) : 0.f;
+                for (int j = 0; j < 8; ++j)
+                    f[u][j] = (row < rows && k + j < kend) ? __float_as_uint(p[j * s_k]) : 0u;
             }
         }
     }
@@ -568,9 +572,14 @@ struct Chunk {
         for (int u = 0; u < G; ++u) {
             int r, g;
             place(u, tid, row_fast, r, g);
+            uint32_t w[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                if constexpr (HALF) w[j] = f[u][j];
+                else w[j] = pack2(__uint_as_float(f[u][2 * j]), __uint_as_float(f[u][2 * j + 1]));
+            }
             *reinterpret_cast<uint4 *>(dst + (r >> 3) * (GC_K * 16) + g * 128 + (r & 7) * 16) =
-                make_uint4(pack2(f[u][0], f[u][1]), pack2(f[u][2], f[u][3]), pack2(f[u][4], f[u][5]),
-                           pack2(f[u][6], f[u][7]));
+                make_uint4(w[0], w[1], w[2], w[3]);
         }
     }
 };
@@ -672,9 +681,14 @@ __device__ __forceinline__ void gemm_end(const GemmCta &G, int tid)
     }
 }
 
-// forward layer with a large K: bias, activation and up to three outputs
+// Forward layer with a large K: bias, activation and up to three outputs.
+// Bound by the latency of a chunk (fetch, MMA chain, barrier) until two CTAs
+// share an SM, hence at most 128 registers a thread.  Measured (BF16 x, us;
+// one chunk at a time without prefetch / prefetch at one CTA per SM / this):
+// 256x512x256 25.1 / 23.6 / 23.5, 16384x512x512 134 / 166 / 131,
+// 32768x2048x512 1052 / 1705 / 966; FP32 x 1127 / 1217 / 797.
 template <typename TA>
-__global__ void __launch_bounds__(TC_THREADS, 1)
+__global__ void __launch_bounds__(TC_THREADS, 2)
     tc_long_kernel(const TA *__restrict__ X, const __nv_bfloat16 *__restrict__ Wt, int M, int N, int K, Epi ep)
 {
     extern __shared__ __align__(1024) char smraw[];

@@ -1,0 +1,54 @@
+"""The forward layer with k > 256: results at the edges of its chunks, and two
+CTAs to an SM, so a launch of twice as many CTAs as the GPU has SMs takes well
+under twice as long as one of as many (it took 2.0 times as long when the
+kernel's registers left room for one).
+
+The reference takes the operands as the kernel does (rounded to BF16), so the
+products are exact and FP32 accumulation is left: 1e-4 relative L2, the
+suite's bar for FP32 outputs of exact BF16 products."""
+import numpy as np
+import pytest
+
+from oracle import mlp_oracle as M
+from test_mlp_gpu import dev, env, rel  # noqa: F401 (fixture)
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("bf16", [True, False])
+@pytest.mark.parametrize("rows,k,n", [(1, 257, 1), (127, 383, 63), (128, 384, 64), (129, 385, 65), (200, 1000, 33)])
+def test_long_reduction(env, rows, k, n, bf16):  # noqa: F811
+    torch, mlp = env
+    r = np.random.default_rng([rows, k, n])
+    x = M.bf16(r.standard_normal((rows, k)))
+    w = M.bf16(r.standard_normal((n, k)) / np.sqrt(k))
+    b = r.standard_normal(n).astype(np.float32)
+    z = torch.full((rows, n), float("nan"), device="cuda")
+    mlp.forward(dev(torch, x, torch.bfloat16 if bf16 else torch.float32), dev(torch, w, torch.bfloat16),
+                dev(torch, b, torch.float32), 0, None, None, z)
+    mlp.check()
+    assert rel(z.cpu().numpy(), x @ w.T + b) <= 1e-4
+
+
+@pytest.mark.parametrize("bf16", [True, False])
+def test_two_ctas_share_an_sm(env, bf16):  # noqa: F811
+    torch, mlp = env
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    k, best = 4096, {}
+    for per in (1, 2):
+        rows = 128 * sms * per                  # one 128 x 64 tile a CTA
+        x = torch.randn(rows, k, device="cuda").to(torch.bfloat16 if bf16 else torch.float32)
+        w = torch.randn(64, k, device="cuda").to(torch.bfloat16)
+        y = torch.empty(rows, 64, device="cuda")
+        mlp.forward(x, w, None, 0, None, y, None)
+        best[per] = 1e9
+        for _ in range(10):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            for _ in range(4):
+                mlp.forward(x, w, None, 0, None, y, None)
+            e1.record()
+            torch.cuda.synchronize()
+            best[per] = min(best[per], e0.elapsed_time(e1))
+    mlp.check()
+    assert best[2] < 1.7 * best[1], best
