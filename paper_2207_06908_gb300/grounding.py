@@ -7,17 +7,20 @@ runs in the CUDA library.
 The tile depth (planes per work item) of each domain comes from a small
 autotuner: for each 16-cell size class it times the candidates on a batch of
 copies of a representative domain (the regime the depth serves) once and
-keeps the winners in a JSON cache in the build folder.
+keeps the winners in a JSON cache in the build folder, each under the sources
+of the kernels it was measured with.
 """
 from __future__ import annotations
 
+import functools
+import hashlib
 import json
 import os
 import time
 
 import numpy as np
 
-from . import fdtd, workloads as W
+from . import _build, fdtd, workloads as W
 
 _CACHE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_build", "tuning.json")
 CANDIDATES = (8, 12, 16, 24, 32, 48)
@@ -26,6 +29,21 @@ CANDIDATES = (8, 12, 16, 24, 32, 48)
 def size_class(n: int) -> int:
     """domains are tuned per 16-cell size class"""
     return (n + 15) // 16 * 16
+
+
+@functools.lru_cache(maxsize=None)
+def _sources() -> str:
+    """of the kernels and the code that launches them: a depth measured with
+    others says nothing about these"""
+    h = hashlib.sha256()
+    for path in sorted(_build._deps()):
+        with open(path, "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:16]
+
+
+def _key(n: int) -> str:
+    return f"ground_batch_n{size_class(n)}_{_sources()}"
 
 
 def _load_cache():
@@ -50,7 +68,7 @@ def tune_block(n: int, steps: int = 32, force: bool = False) -> int:
     representative domain (enough copies that the batch, not one domain,
     fills the GPU, as in the batches this serves; cached)."""
     import torch
-    key = f"ground_batch_n{size_class(n)}"
+    key = _key(n)
     cache = _load_cache()
     if key in cache and not force:
         return int(cache[key])
