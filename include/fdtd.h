@@ -395,8 +395,8 @@ typedef struct fdtd_batch fdtd_batch;
  * table (about 16 KB per domain: launch arguments, tensor maps and the
  * staging images the step kernel copies into shared memory).  FDTD_ESTATE
  * if a grid is not finalized or the step counts differ; FDTD_EINVAL for a
- * grid with Debye poles or a grid of 2^31 cells or more (batch domains use
- * 32-bit indices). */
+ * grid with Debye poles or a grid of 2^31 cells or more (one such grid fills
+ * the GPU by itself: it is stepped alone). */
 int fdtd_batch_create(int n_grids, fdtd_grid *const *grids, void *cuda_stream, fdtd_batch **out);
 
 /* Queue n steps of every domain on the batch stream (asynchronous).  Each

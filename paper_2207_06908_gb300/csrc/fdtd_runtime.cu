@@ -2668,7 +2668,7 @@ int fdtd_batch_create(int n, fdtd_grid *const *grids, void *cuda_stream, fdtd_ba
         fdtd_grid *g = grids[q];
         if (!g || !g->finalized) { delete b; return FDTD_ESTATE; }
         if (g->npoles) { delete b; return FDTD_EINVAL; }      // dispersive media run on their own
-        if ((double)g->plane * g->nz >= 2147483647.0) { delete b; return FDTD_EINVAL; }  // 32-bit indices
+        if ((double)g->plane * g->nz >= 2147483647.0) { delete b; return FDTD_EINVAL; }  // stepped alone
         if (g->parity != grids[0]->parity || g->step != grids[0]->step) { delete b; return FDTD_ESTATE; }
         b->grids.push_back(g);
     }
