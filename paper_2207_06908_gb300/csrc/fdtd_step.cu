@@ -25,14 +25,14 @@
 //     it, both in shared memory.  Two more warps recompute (never exchange)
 //     H^{n+1/2} of the low-y row and the low-x column of the halo meanwhile.
 //   - The layers an item meets are template arguments: an item that meets
-//     none runs without any CPML code, the others without a branch per cell.
+//     none runs without any CPML code, the others with one branch per layer.
 // What bounds it: DRAM on grids that fill the chip, otherwise the latency of
 // a plane's chain (copies landed, H, barrier, E), which a CTA cannot
 // overlap with more than the ring holds: 1300 cycles alone on an SM without a
 // layer, 2000 with one.  Hence few and wide instructions per plane, values
 // the same for a warp in uniform registers (item by shuffle, one base
 // pointer per array and plane, one 32-bit offset per lane), no choice inside
-// the plane loop, registers split by role (setmaxnreg) so that nothing
+// the plane loop but whether a lane is in a layer, registers split by role (setmaxnreg) so that nothing
 // spills, and few copies issued by a converged warp.  With four cells per
 // lane (16-byte accesses) the plane loop has fewer instructions but half the
 // warps to hide its latency, and measured slower (197 us on the 256^3 CPML
@@ -40,8 +40,8 @@
 // of offsets took 11 % more instructions (256^3 PEC 134 us).  Measured (us
 // per step; one cell per lane, fifteen copies a plane and 16 planes per item
 // before): 256^3 PEC 136.3 -> 129.8, 256^3 with a 10-cell CPML 175.9 ->
-// 160.8, 512x512x384 with 12 cells 956 -> 905, 128^3 with 8 cells 42.7 ->
-// 31.9, 64^3 with 8 cells 25.6 -> 9.3 (programmatic dependencies between the
+// 160.8, 512x512x384 with 12 cells 956 -> 914, 128^3 with 8 cells 42.7 ->
+// 30.8, 64^3 with 8 cells 25.6 -> 9.4 (programmatic dependencies between the
 // steps' kernels, fdtd_runtime.cu, included).
 // DRAM traffic per cell and step: 6 FP32 reads + 6 writes + 1 class byte
 // (49 B) plus the CPML auxiliaries in the layer; every halo read is an L2
@@ -394,8 +394,7 @@ __device__ __forceinline__ void h_core(const StepArgs &a, const float4 *t, const
 // with another, the index arithmetic and the barriers are paid once per two
 // cells, and the differences and layer sums run two cells to an instruction
 // (packed FP32 pairs).  The layers an item meets are template arguments and
-// the lanes outside them run along and leave out the last sum, so the plane
-// loop has no branches to wait on.  Every sum is written as explicit products
+// the lanes outside them skip them.  Every sum is written as explicit products
 // and fused multiply-adds, so every instantiation of the kernel rounds alike.
 using F2 = unsigned long long;           // two FP32 values
 __device__ __forceinline__ F2 pk(float lo, float hi)
@@ -446,9 +445,8 @@ struct Pair {
     int fl;                  // IN0, IN1: the first, second cell lies inside the grid; XM0, XM1: in an x layer;
                              // YM: the row lies in a y layer
     int xo;                  // float offset of the first cell's entry in the first x box
-    int yo;                  // float offset of the pair in the first y box (of the lane's column, outside the layer)
+    int yo;                  // float offset of the pair in the first y box
     const float4 *py;        // its y profile row at E positions, 2d rows before the one at H positions
-                             // (outside the layer: any)
     unsigned off;            // its element in a plane of the fields and z auxiliaries
     int xoff, yoff;          // of the x, y auxiliaries (a lane outside the layer: not used)
 };
@@ -474,19 +472,8 @@ __device__ __forceinline__ F2 cpmlx(F2 &dif, const PX &q, F2 o)
     dif = fma2(dif, q.ki, p);
     return p;
 }
-// The same for a lane that may lie outside the layer (in: inside); outside,
-// the difference stays as it is.  Coefficients of zero and one would not do
-// that: times an infinite difference, or an infinite auxiliary of the row
-// that a lane outside the layer reads, zero is a NaN.  Written so it costs
-// -0.3 to 0.6 % (20 steps of 256^3 with 10 cells 3338 -> 3336 us, 32 of
-// 160x160x200 2345 -> 2357); selects or inline PTX predicates spilled (1 to 4 %).
-__device__ __forceinline__ F2 cpmlx(F2 &dif, const PX &q, F2 o, bool in)
-{
-    const F2 p = fma2(q.b, o, mul2(q.c, dif));
-    if (in) dif = fma2(dif, q.ki, p);
-    return p;
-}
-// both differences of a pair cut by the layer: in0, in1 for its two cells
+// Both differences of a pair that the layer may cut: in0, in1 for its two
+// cells.  A difference outside the layer stays as it is.
 __device__ __forceinline__ void cpmlx_cut(F2 &d0, F2 &d1, const PX &q, F2 o0, F2 o1, bool in0, bool in1, F2 &p0, F2 &p1)
 {
     p0 = fma2(q.b, o0, mul2(q.c, d0));
@@ -509,36 +496,25 @@ __device__ __forceinline__ void cpmlx_cut(F2 &d0, F2 &d1, const PX &q, F2 o0, F2
 // 8-byte boundary (d and nx even); otherwise cell by cell (a choice made
 // inside the plane loop costs more than the layer's arithmetic).  A pair
 // never has members in both layers (they are two cells apart at least).
-// Cells outside the layer read 0.
+// Lanes outside a layer skip it.  Running along with coefficients of zero and
+// one in place of that, they made NaNs of an infinite difference, and of an
+// infinite auxiliary of the row they read; skipping is no slower (us per step:
+// 64^3 with 8 cells 9.37 -> 9.36, 128^3 with 8 31.3 -> 30.8, 96^3 with 10
+// 21.7 -> 21.4, 256^3 with 10 161.2 -> 160.9).  Selects or predicates on the
+// sums spilled or cost up to 4 %; skipping cell by cell spilled too, so a
+// pair that a layer may cut leaves out the sums.
 template <bool VEC>
 __device__ __forceinline__ void cpml_x(const StepArgs &a, const Pair &G, const PlaneX &P, int h, int k, F2 &d0, F2 &d1)
 {
+    if (VEC && !(G.fl & XM)) return;
     const int q = a.pg.xb >> 2, at = h ? 0 : 2;
     const float *b = P.base + at * q + G.xo;
     const PX pr = profx(P.xc + (h ? 3 * TX : 0));
-    F2 o0 = 0, o1 = 0;
-    if (VEC) {
-        if (G.fl & XM) {
-            o0 = ld2(b);
-            o1 = ld2(b + q);
-        }
-    } else {
-        float f[4] = {0.f, 0.f, 0.f, 0.f};
-        if (G.fl & XM0) {
-            f[0] = b[0];
-            f[1] = b[q];
-        }
-        if (G.fl & XM1) {
-            f[2] = b[1];
-            f[3] = b[q + 1];
-        }
-        o0 = pk(f[0], f[2]);
-        o1 = pk(f[1], f[3]);
-    }
+    const F2 o0 = VEC ? ld2(b) : pk(b[0], b[1]), o1 = VEC ? ld2(b + q) : pk(b[q], b[q + 1]);
     F2 p0, p1;
     if (VEC) {
-        p0 = cpmlx(d0, pr, o0, G.fl & XM);
-        p1 = cpmlx(d1, pr, o1, G.fl & XM);
+        p0 = cpmlx(d0, pr, o0);
+        p1 = cpmlx(d1, pr, o1);
     } else {
         cpmlx_cut(d0, d1, pr, o0, o1, G.fl & XM0, G.fl & XM1, p0, p1);
     }
@@ -546,8 +522,8 @@ __device__ __forceinline__ void cpml_x(const StepArgs &a, const Pair &G, const P
     float *u0 = a.psi_out[h ? PSI_HY_X : PSI_EY_X], *u1 = a.psi_out[h ? PSI_HZ_X : PSI_EZ_X];
     const long long n = psi_n(a, 0);
     if (VEC) {
-        put2(u0, pl, G.xoff, p0, G.fl & XM, n, 3, a.bounds);
-        put2(u1, pl, G.xoff, p1, G.fl & XM, n, 3, a.bounds);
+        put2(u0, pl, G.xoff, p0, true, n, 3, a.bounds);
+        put2(u1, pl, G.xoff, p1, true, n, 3, a.bounds);
     } else {
         u0 += pl;
         u1 += pl;
@@ -564,13 +540,14 @@ __device__ __forceinline__ void cpml_x(const StepArgs &a, const Pair &G, const P
 // of the y layer
 __device__ __forceinline__ void cpml_y(const StepArgs &a, const Pair &G, const PlaneX &P, int h, int k, F2 &d0, F2 &d1)
 {
+    if (!(G.fl & YM)) return;
     const int q = a.pg.yb >> 2, at = h ? 0 : 2;
     const float *b = P.base + G.yo + at * q;
     const PX pr = profx(G.py[h ? 2 * a.d : 0]);
-    const F2 p0 = cpmlx(d0, pr, ld2(b), G.fl & YM), p1 = cpmlx(d1, pr, ld2(b + q), G.fl & YM);
+    const F2 p0 = cpmlx(d0, pr, ld2(b)), p1 = cpmlx(d1, pr, ld2(b + q));
     const int pl = k * (2 * a.d * a.pitch);
-    put2(a.psi_out[h ? PSI_HX_Y : PSI_EX_Y], pl, G.yoff, p0, G.fl & YM, psi_n(a, 1), 3, a.bounds);
-    put2(a.psi_out[h ? PSI_HZ_Y : PSI_EZ_Y], pl, G.yoff, p1, G.fl & YM, psi_n(a, 1), 3, a.bounds);
+    put2(a.psi_out[h ? PSI_HX_Y : PSI_EX_Y], pl, G.yoff, p0, true, psi_n(a, 1), 3, a.bounds);
+    put2(a.psi_out[h ? PSI_HZ_Y : PSI_EZ_Y], pl, G.yoff, p1, true, psi_n(a, 1), 3, a.bounds);
 }
 // of the z layer
 __device__ __forceinline__ void cpml_z(const StepArgs &a, const Pair &G, const PlaneX &P, const float *prof, int h,
@@ -886,7 +863,7 @@ __device__ __forceinline__ void run_rows(const Cons<NH> &C, const Item &it, Ring
     const int nv = j < a.ny ? max(0, min(GX, a.nx - i)) : 0;
     Pair G;
     G.fl = (1 << nv) - 1;
-    G.xo = 0;
+    G.xo = 0;                       // a pair outside the layer reads, cell by cell, and does not use, what lies there
     G.yo = 0;
     G.py = reinterpret_cast<const float4 *>(C.prof);
     // slab entry of the pair's first cell, in the layer its members lie in, and of its row
@@ -897,10 +874,10 @@ __device__ __forceinline__ void run_rows(const Cons<NH> &C, const Item &it, Ring
 #pragma unroll
         for (int c = 0; c < GX; ++c)
             if (c < nv && slab_of(i + c, a.nx, d) >= 0) G.fl |= XM0 << c;
-        G.xo = a.ox / 4 + row * a.pg.w + xe - tb.xs;
-        G.yo = a.oy / 4 + (sy >= 0 ? sy - tb.ys : 0) * HBX + lx;
+        if (G.fl & XM) G.xo = a.ox / 4 + row * a.pg.w + xe - tb.xs;
         if (sy >= 0) {
             G.fl |= YM;
+            G.yo = a.oy / 4 + (sy - tb.ys) * HBX + lx;
             G.py = prow(C.prof, 1, 0, 2 * d) + sy;
         }
     }
