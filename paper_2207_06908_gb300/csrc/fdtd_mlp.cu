@@ -79,7 +79,7 @@ __device__ __forceinline__ float4 ld_peer4(uint32_t a)
 
 // dz = dy act'(z) and, with db, its column sums, in one pass.  A cluster of
 // CTAs takes ZB_COLS columns, each CTA every gridDim.y-th part of the rows: its
-// 32 row lanes keep ZB_ROWS loads in flight each, their sums meet in shared
+// 8 row lanes keep ZB_ROWS loads in flight each, their sums meet in shared
 // memory and the CTAs' in rank 0 through distributed shared memory, always in
 // the same order.  Bound by latency at a minibatch (256 x 256: the two
 // passes of before, elementwise and then a serial column sum on two CTAs,
@@ -726,8 +726,8 @@ __global__ void __launch_bounds__(TC_THREADS, 2)
 // rows is what gives a large minibatch more CTAs.  At a minibatch of 256 rows
 // the pass is a chain of latencies (fetch, MMA, epilogue; one chunk per CTA).
 // Measured with act_grad_kernel, a whole backward pass of a layer: 256 -> 256
-// at 256 rows 36.0 us in four launches before, 13.8 in two now; at 4096 rows
-// 317 before, 41; 256 -> 512 at 4096 rows 332 before, 65.
+// at 256 rows 36.0 us in four launches before, 12.1 in two now; at 4096 rows
+// 317 before, 37; 256 -> 512 at 4096 rows 332 before, 57.
 constexpr int GP_PITCH = TC_N + 4;   // floats per row of a CTA's partial tile
 static_assert(TC_M * GP_PITCH * 4 <= (TC_M + TC_N) * GC_K * 2, "a partial tile fits the operand area");
 

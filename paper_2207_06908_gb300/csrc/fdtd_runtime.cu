@@ -1320,17 +1320,21 @@ int blocks(int n, int k) { return (n + k - 1) / k; }
 // with many it is their sum plus about half an item at the end.  In planes,
 // with an item's start worth 1.5 of them (3 in a z layer):
 //  - shallow items while one CTA per SM holds them all: a second CTA slows
-//    both (64^3, 8-cell CPML: 4 and 3 planes, 12.6 us a step; 2 and 3 planes
-//    on more CTAs than SMs 15.7; 16 and 8 planes 25.6);
-//  - else one wave of all slots, the z layers whole (128^3 with 8 cells: 16
-//    planes, 38.0 us; 8 planes 38.3; 32 planes 53.9), or one wave of thin
-//    z-layer items and then one of the others, whichever is shorter
-//    (100x100x80 with 10 cells: 2 and 6 planes 27.5 us, 10 and 8 planes 30.1);
+//    both (64^3, 8-cell CPML: it takes 4 and, in the z layers, 3 planes, 9.7
+//    us a step; 2 and 3 planes on more CTAs than SMs 10.4; 16 and 8 19.9);
+//  - else one wave of all slots, the z layers whole (128^3 with 8 cells: it
+//    takes 16 planes, 30.9 us; 8 planes 34.0, 32 planes 38.6), or one wave of
+//    thin z-layer items and then one of the others, whichever this model has
+//    as the shorter (100x100x80 with 10 cells: it takes 6 and 2 planes, 22.2
+//    us, where whole z layers and 8 planes measure 20.6: the model sees the
+//    two waves too short there);
 //  - else the least of (columns x (planes + 1.5 per item)) / slots + half an
-//    item, within 8 .. 14 planes (160x160x200 with 10 cells: 10 planes 70.4
-//    us, 16 planes 74.0; 512x512x384 with 12 cells: 12 planes 901, 16 planes
-//    908, 24 planes 942, as deeper items leave the planes their neighbours
-//    share in L2 for too long).
+//    item, within 8 .. 14 planes (160x160x200 with 10 cells: it takes 9, 62.7
+//    us, 16 planes 67.4; 256^3 with 10 cells: 14, 160.5, 10 planes 156.3, 24
+//    planes 167.9; 512x512x384 with 12 cells: 14, 911, 10 planes 896, 24
+//    planes 976).  Deeper items leave the planes their neighbours share in L2
+//    for too long; that cost is not in the model but for the upper end of the
+//    range, which is why it takes 14 where 10 measures 2 % faster.
 Depth pick_depth(const std::vector<Columns> &doms, int sms, int slots)
 {
     int planes = 1, d = 0;
