@@ -34,7 +34,6 @@ def generate(params, per_batch=512, log=None):
     n = len(params)
     out = np.empty((n, N_OUT), dtype=np.float32)
     steps = W.GROUND_STEPS
-    block = grounding.tune_block(W.SURROGATE_N)
     streams = [torch.cuda.Stream(), torch.cuda.Stream()]
     pending = None
     t0 = time.perf_counter()
@@ -52,8 +51,9 @@ def generate(params, per_batch=512, log=None):
     for bi, lo in enumerate(range(0, n, per_batch)):
         s = streams[bi % 2]
         with torch.cuda.stream(s):
-            grids = [fdtd.from_scenario(W.surrogate_domain(p), stream=s, probe_capacity=steps, block=block)
-                     for p in params[lo:lo + per_batch]]
+            scs = [W.surrogate_domain(p) for p in params[lo:lo + per_batch]]
+            grids = [fdtd.from_scenario(sc, stream=s, probe_capacity=steps, block=kz)
+                     for sc, kz in zip(scs, grounding.depths(scs))]
             b = fdtd.Batch(grids, stream=s)
             b.step(steps)
         if pending is not None:
