@@ -683,12 +683,14 @@ __device__ __forceinline__ void gemm_end(const GemmCta &G, int tid)
 
 // Forward layer with a large K: bias, activation and up to three outputs.
 // Bound by the latency of a chunk (fetch, MMA chain, barrier) until two CTAs
-// share an SM, hence at most 128 registers a thread.  Measured (BF16 x, us;
-// one chunk at a time without prefetch / prefetch at one CTA per SM / this):
-// 256x512x256 25.1 / 23.6 / 23.5, 16384x512x512 134 / 166 / 131,
-// 32768x2048x512 1052 / 1705 / 966; FP32 x 1127 / 1217 / 797.
-template <typename TA>
-__global__ void __launch_bounds__(TC_THREADS, 2)
+// share an SM: PER_SM 2 keeps to 128 registers a thread for that, PER_SM 1
+// takes 202 to 220 and is the quicker one while every CTA has an SM to itself.
+// Measured (BF16 x, us; one chunk at a time without prefetch / PER_SM 1 / 2):
+// 1x4096x512 127 / 108 / 116, 256x2048x256 82 / 65 / 72, 19456x4096x64 (152
+// CTAs) 264 / 191 / 224, 38912x4096x64 (304) 305 / 382 / 279, 32768x2048x512
+// 1052 / 1705 (BF16 held as FP32) / 966; FP32 x 38912x4096x64 316 / 344 / 266.
+template <typename TA, int PER_SM>
+__global__ void __launch_bounds__(TC_THREADS, PER_SM)
     tc_long_kernel(const TA *__restrict__ X, const __nv_bfloat16 *__restrict__ Wt, int M, int N, int K, Epi ep)
 {
     extern __shared__ __align__(1024) char smraw[];
@@ -850,10 +852,16 @@ cudaLaunchConfig_t cluster_launch(dim3 grid, int threads, size_t smem, cudaStrea
 template <typename TA>
 cudaError_t tc_long(const TA *x, const __nv_bfloat16 *wt, int M, int N, int K, const Epi &ep, cudaStream_t s)
 {
-    cudaError_t e = allow_smem((const void *)tc_long_kernel<TA>, GC_SMEM);
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     const dim3 grid((M + TC_M - 1) / TC_M, (N + TC_N - 1) / TC_N);
-    tc_long_kernel<TA><<<grid, TC_THREADS, GC_SMEM, s>>>(x, wt, M, N, K, ep);
+    // two CTAs to an SM as soon as there are more of them than SMs
+    const auto kernel = (long long)grid.x * grid.y > sms ? tc_long_kernel<TA, 2> : tc_long_kernel<TA, 1>;
+    e = allow_smem((const void *)kernel, GC_SMEM);
+    if (e != cudaSuccess) return e;
+    kernel<<<grid, TC_THREADS, GC_SMEM, s>>>(x, wt, M, N, K, ep);
     return cudaGetLastError();
 }
 

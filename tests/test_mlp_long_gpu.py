@@ -16,7 +16,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("bf16", [True, False])
-@pytest.mark.parametrize("rows,k,n", [(1, 257, 1), (127, 383, 63), (128, 384, 64), (129, 385, 65), (200, 1000, 33)])
+@pytest.mark.parametrize("rows,k,n", [(1, 257, 1), (127, 383, 63), (128, 384, 64), (129, 385, 65), (200, 1000, 33),
+                                      (9601, 300, 130)])
 def test_long_reduction(env, rows, k, n, bf16):  # noqa: F811
     torch, mlp = env
     r = np.random.default_rng([rows, k, n])
